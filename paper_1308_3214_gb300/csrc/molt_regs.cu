@@ -274,7 +274,7 @@ cudaError_t run_strided_nb(const AxisDev &A, const LineSet &L, const ProgParams 
         const int in_rows = L.S * RPT + 4;
         tm.nbox = (in_rows + 255) / 256;
         tm.box_rows = (in_rows + tm.nbox - 1) / tm.nbox;
-        const int out_box = L.S * RPT > 256 ? 256 : L.S * RPT;
+        const int out_box = strided_nb_out_box(L.S, RPT);
         bool ok = true;
         if (stage & 1)
             ok = encode_field_map(&tm.in_hi, p.u_hi, L, A.n, tm.box_rows) &&

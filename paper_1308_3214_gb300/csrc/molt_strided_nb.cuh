@@ -42,6 +42,15 @@ namespace molt {
 // stages each output power in the tile and writes it with one tensor store.
 __host__ __device__ inline size_t strided_nb_slot_bytes(int S) { return (size_t)2 * S * 4 * 32 * sizeof(float); }
 __host__ __device__ inline size_t strided_nb_tile_off(int S) { return (strided_nb_slot_bytes(S) + 8 + 127) & ~(size_t)127; }
+// Rows of one tensor store of the CTA's S RPT output rows: at most 256 (the
+// box limit) and an even split, so that the boxes end where the tile and the
+// CTA's own rows end (5, 6 or 7 segments of 64 rows are two boxes of 160, 192
+// or 224 rows; RPT is even).
+__host__ __device__ inline int strided_nb_out_box(int S, int rpt)
+{
+    const int rows = S * rpt;
+    return rows / ((rows + 255) / 256);
+}
 __host__ __device__ inline size_t strided_nb_smem(int S, int rpt = 0, int stage = 0, int nbox = 0, int box_rows = 0)
 {
     if (stage == 0) return strided_nb_slot_bytes(S);
@@ -381,7 +390,7 @@ __global__ void __launch_bounds__(256, 2) k_strided_nb(AxisDev A, LineSet LS, Pr
                 fence_proxy_async();
                 __syncthreads();
                 if (threadIdx.x == 0) {
-                    const int orows = S * RPT, ob = orows > 256 ? 256 : orows;
+                    const int orows = S * RPT, ob = strided_nb_out_box(S, RPT);
                     for (int y = 0; y < orows; y += ob) tma_store_3d(&tm.out[p - 1], x0, a0 + y, z0, tile + (size_t)y * 32);
                     tma_store_commit();
                 }

@@ -667,3 +667,23 @@ def test_rows_neighbour_exchange_matches_oracle(shape, W, cfl, bc, P, rows_nb):
     tol = 8 * EPS32 * (1 + 1 / (1 - max(s.d))) * 2 * P * Fsum / np.linalg.norm(rc)
     assert rel_l2(uc.cpu().numpy(), rc) <= tol
     s.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ny", [320, 384, 448, 640, 832, 896])
+@pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
+@pytest.mark.parametrize("stage", [2, 3])
+def test_strided_tma_stores_of_uneven_segment_counts_match_oracle(ny, bc, stage):
+    """5, 6 or 7 segments of 64 rows per CTA (one CTA or a 2-CTA cluster per
+    column group): the CTA's rows are not a whole number of 256-row boxes, so
+    its tensor stores must stop at its own last row."""
+    s = make((ny, 64), 1.5 * spacing(ny, bc), 3, bc, "mixed")
+    v = field((ny, 64), 81, bc)
+    vd = dev(v)
+    s.set_tuning(rows_warps=0, strided_nb=1, strided_stage=stage)
+    for p in (1, 2, 3):
+        got = s.apply_D(vd, 1, p).cpu().numpy()
+        ref = oracle.D_axis(v, 1, s.nu[1], bc, 2, power=p)
+        assert rel_l2(got, ref) <= tol_for("mixed", s, p), (p, rel_l2(got, ref))
+    s.sync()
+    s.close()
