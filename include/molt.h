@@ -104,9 +104,11 @@ void mol_default_options(mol_options *opt);
 mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, int P,
                       mol_bc bc, mol_prec prec, const mol_options *opt, mol_handle *out);
 
-/* (2D Dirichlet grids with at most 1024 points per axis whose lines do not
- * split into whole register segments run mol_apply_F, mol_start, mol_step
- * and mol_solve_host on the batched kernels, as a batch of one problem.) */
+/* (2D Dirichlet MOL_MIXED grids with at most 1024 points per axis whose lines
+ * do not split into whole register segments run mol_apply_F, mol_start,
+ * mol_step and mol_solve_host on the batched kernels, as a batch of one
+ * problem.  MOL_FP64 passes take lines of any length; the launch choices of
+ * mol_autotune / mol_set_tuning are those of the float32 sweeps.) */
 
 /* Free the workspace and the handle (waits for the handle's work). */
 mol_status mol_destroy(mol_handle h);
@@ -606,8 +608,8 @@ mol_status mol_embed_pass_times(mol_embed e, double total_ms[3], int64_t launche
  * of the device, or a loop that cannot afford cudaFree's device-wide
  * synchronisation.
  *
- * Scratch: the intermediate planes, the tables d^j and the Horner
- * coefficients live in one static device array of 32 MiB (32 << 20 bytes)
+ * Scratch: the intermediate planes and the tables d^j live in one static
+ * device array of 32 MiB (32 << 20 bytes)
  * inside libmolt.  A call needs 512 + sum_a roundup32(n_a + 1) +
  * planes * roundup32(N) doubles, planes = 0 (1D), P (2D), 2P + 1 (3D),
  * N = the number of grid points; larger grids are rejected with MOL_EINVAL

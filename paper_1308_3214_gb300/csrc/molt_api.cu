@@ -13,6 +13,7 @@
 
 #include "molt.h"
 #include "molt_internal.h"
+#include "molt_f64.cuh"
 #include "molt_recv.cuh"
 
 using namespace molt;
@@ -43,8 +44,6 @@ struct mol_ctx {
     float *dpow32[3] = {nullptr, nullptr, nullptr};
     std::vector<double> f;       // expanded coefficients, (P+1)^ndim, x degree fastest
     HornerParams xtpl{}, ytpl{}; // coefficient templates of the Horner passes
-    double *coef_dev = nullptr;  // the same tables on the device: x coef, x cu, y coef, y cu
-    size_t off_xc = 0, off_xu = 0, off_yc = 0, off_yu = 0;
     double dmr[4][5] = {};       // d^{R 2^k} for register segments R = 8, 16, 32, 64 (per axis below)
     double dmr_ax[3][4][5] = {};
     Level lev[3];
@@ -71,7 +70,7 @@ struct mol_ctx {
     int tune_pdl = 0;                          // register pass kernels as programmatic dependent launches
                                                // (measured slower on the 2D and 3D steps: off)
     double tune_ms = 0.0;                      // step time of the chosen configuration
-    // 2D Dirichlet grids (n <= 1024 per axis) whose lines the register
+    // 2D Dirichlet MOL_MIXED grids (n <= 1024 per axis) whose lines the register
     // kernels cannot split into whole segments run on the batched kernels
     // (ragged lines) as a batch of one problem
     mol_batch batch = nullptr;
@@ -283,7 +282,73 @@ void smem_pass_geom(const mol_ctx *h, int axis, bool horner, PassGeom &G, AxisDe
     G.dps = pass_smem_bytes(horner, h->tbytes, G.W, A.ls, A.n, 1) <= h->smem_optin ? 1 : 0;
 }
 
-// Launch one pass program: the register-resident kernel when the line length
+// A float64 pass: the Horner weights arrive in the units of the powers (times
+// kappa per application of this axis' D, f64_units); raw powers stay in them.
+cudaError_t run_f64(const mol_ctx *h, int axis, const PowersParams *pp, const HornerParams *hp, cudaStream_t s)
+{
+    const PassGeom G = geom_of(h, axis);
+    F64Plan pl;
+    if (!f64_plan((int)h->n[axis], G.nlines, axis == 0, hp != nullptr, h->nu[axis], h->num_sms, &pl))
+        return cudaErrorInvalidValue;
+    F64Prog p{};
+    if (hp) {
+        p.P = hp->P;
+        p.ng = hp->ng;
+        p.nout = hp->nout;
+        p.epi = hp->epi;
+        for (int o = 0; o < std::max(hp->nout, 1); ++o)
+            for (int t = 0; t <= hp->P; ++t) {
+                for (int k = 0; k < hp->ng; ++k) {
+                    p.coef[o][t][k] = hp->coef[o][t][k];
+                    if (hp->coef[o][t][k] != 0.0) p.add[o][t] |= 1u << k;
+                }
+                p.cu[o][t] = hp->cu[o][t];
+                if (hp->cu[o][t] != 0.0) p.ucu[o] |= 1u << t;
+            }
+        for (int k = 0; k < MAXG; ++k) { p.g[k] = (const double *)hp->g[k]; p.out[k] = (double *)hp->out[k]; }
+        p.ea = hp->ea; p.eb = hp->eb; p.ec = hp->ec;
+        p.hea = hp->ea != 0.0; p.heb = hp->eb != 0.0; p.hec = hp->ec != 1.0;
+        p.u = (const double *)hp->u_hi;
+        p.up = (const double *)hp->up_hi;
+        p.un = (double *)hp->un_hi;
+    } else {
+        p.P = pp->P;
+        p.u = (const double *)pp->u_hi;
+        const double k = f64_kappa(h->nu[axis], h->opt.quad_order);
+        double sc = 1.0;
+        for (int q = 0; q < pp->P; ++q) {
+            sc *= k;
+            p.scale[q] = sc;
+            if (!pp->raw) p.scaled |= 1u << q;
+            p.out[q] = (double *)pp->out[q];
+        }
+    }
+    return launch_f64(h->bc, axis == 0, pl, h->nu[axis], h->opt.quad_order, h->ax[axis], G.stride, G.inner, G.nlines,
+                      hp != nullptr, p, s);
+}
+
+// kappa of an axis whose passes leave it to the weights, else 1
+double f64_unit(const mol_ctx *h, int axis)
+{
+    return h->tbytes == 8 && f64_axis_ok((int)h->n[axis], axis == 0) ? f64_kappa(h->nu[axis], h->opt.quad_order) : 1.0;
+}
+
+// Horner weights of a pass along an axis of unit kx whose field k carries
+// unit kg^(k+1): weight of step t times kx^t (and kg^(k+1) for field k)
+void f64_units(HornerParams &hp, double kx, double kg)
+{
+    if (kx == 1.0 && kg == 1.0) return;
+    for (int o = 0; o < std::max(hp.nout, 1); ++o) {
+        double ux = 1.0;
+        for (int t = 0; t <= hp.P; ++t, ux *= kx) {
+            double ug = kg;
+            for (int k = 0; k < hp.ng; ++k, ug *= kg) hp.coef[o][t][k] *= ux * ug;
+            hp.cu[o][t] *= ux;
+        }
+    }
+}
+
+// Launch one pass program: the float64 line pass, the register-resident kernel when the line length
 // and boundary condition allow it, else the shared-memory kernels.
 mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersParams *pp, const HornerParams *hp,
                        cudaStream_t s)
@@ -302,6 +367,8 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
         AxisDev A;
         smem_pass_geom(h, axis, true, G, A);
         e = launch_horner(h->tbytes, h->bc, axis == 0, A, G, *hp, s);
+    } else if (h->tbytes == 8 && f64_axis_ok(n, axis == 0)) {
+        e = run_f64(h, axis, pp, hp, s);
     } else if (pr.mode == 2 || pr.mode == 3) {
         // the transposed passes of the adjoint step (register kernels only;
         // single_adjoint checks that the grid has both plans)
@@ -324,7 +391,7 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
             if (h->tbytes == 4 && h->tune_strided_nb && regs_strided_nb_plan(A.d, n, rpt))
                 e = launch_strided_nb_T(rpt, A, L, pr, s);
             else
-                e = launch_strided(h->tbytes, h->bc, rpt, A, L, pr, s);
+                e = launch_strided(h->bc, rpt, A, L, pr, s);
         }
     } else if (axis == 0 && pr.mode == 1 && pr.nout == 1 && h->tune_rows_warps > 0 &&
         regs_rows_plan(h->tbytes, n, pr.ng, h->tune_rows_warps, &rpt)) {
@@ -335,7 +402,7 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
     } else if (axis == 0 && pr.mode == 1 && pr.nout == 1 && regs_res_plan(h->tbytes, n, pr.ng, &rpt)) {
         e = launch_res(h->bc, rpt, pr.ng, h->tune_res_warps, regs_axis(h, 0, rpt), lineset_of(h, 0), pr, s);
     } else if (axis == 0 && regs_contig_plan(h->tbytes, h->bc, n, &rpt)) {
-        e = launch_contig(h->tbytes, h->bc, rpt, regs_axis(h, 0, rpt), lineset_of(h, 0), pr, s);
+        e = launch_contig(h->bc, rpt, regs_axis(h, 0, rpt), lineset_of(h, 0), pr, s);
     } else if (axis > 0 && regs_strided_plan(h->tbytes, h->bc, n, &rpt, &S, &K, h->tune_strided_rpt,
                                              h->tune_strided_warps)) {
         LineSet L = lineset_of(h, axis);
@@ -347,7 +414,7 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
         else if (h->tbytes == 4 && pr.mode == 1 && h->tune_strided_nb && regs_strided_nb_plan(A.d, n, rpt))
             e = launch_strided_nb_h(h->bc, rpt, A, L, pr, s, h->tune_strided_nb == 2);
         else
-            e = launch_strided(h->tbytes, h->bc, rpt, A, L, pr, s);
+            e = launch_strided(h->bc, rpt, A, L, pr, s);
     } else {
         PassGeom G;
         AxisDev A;
@@ -360,10 +427,13 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
     return timing_end(h, s, axis, e0, e1);
 }
 
-mol_status run_powers(mol_ctx *h, int axis, const Level &u, int P, void *const *outs, cudaStream_t s)
+// raw: float64 outputs may stay in units of kappa^p (their consumer's Horner
+// weights carry them)
+mol_status run_powers(mol_ctx *h, int axis, const Level &u, int P, void *const *outs, cudaStream_t s, bool raw = false)
 {
     PowersParams p{};
     p.P = P;
+    p.raw = raw;
     p.u_hi = u.hi;
     p.u_lo = u.lo;
     ProgParams pr{};
@@ -375,8 +445,7 @@ mol_status run_powers(mol_ctx *h, int axis, const Level &u, int P, void *const *
     return run_program(h, axis, pr, &p, nullptr, s);
 }
 
-// hp carries the fields; dcoef / dcu are the device copies of its tables
-mol_status run_horner(mol_ctx *h, int axis, HornerParams &hp, const double *dcoef, const double *dcu, cudaStream_t s)
+mol_status run_horner(mol_ctx *h, int axis, HornerParams &hp, cudaStream_t s)
 {
     ProgParams pr{};
     pr.mode = 1;
@@ -384,8 +453,6 @@ mol_status run_horner(mol_ctx *h, int axis, HornerParams &hp, const double *dcoe
     pr.ng = hp.ng;
     pr.nout = hp.nout;
     for (int k = 0; k < MAXG; ++k) { pr.g[k] = hp.g[k]; pr.out[k] = hp.out[k]; }
-    pr.coef = dcoef;
-    pr.cu = dcu;
     pr.epi = hp.epi;
     pr.ea = hp.ea; pr.eb = hp.eb; pr.ec = hp.ec;
     prog_mirror(pr, hp);
@@ -446,23 +513,10 @@ void build_tables(mol_ctx *h)
     fill_tables(h->ndim, h->P, [h](int i, int j, int k) { return fco(h, i, j, k); }, h->xtpl, h->ytpl);
 }
 
-void flatten(const HornerParams &hp, std::vector<double> &coef, std::vector<double> &cu)
-{
-    coef.clear();
-    cu.clear();
-    for (int o = 0; o < std::max(hp.nout, 1); ++o)
-        for (int t = 0; t <= hp.P; ++t) {
-            for (int k = 0; k < hp.ng; ++k) coef.push_back(hp.coef[o][t][k]);
-            cu.push_back(hp.cu[o][t]);
-        }
-    if (coef.empty()) coef.push_back(0.0);
-}
-
 // un = ea*u + eb*up + ec*F[u]  (the full pass plan of one step).  inter:
-// the intermediate planes; xc/xu/yc/yu: device copies of the Horner tables.
-mol_status run_update_with(mol_ctx *h, void *const *inter, const double *xc, const double *xu, const double *yc,
-                           const double *yu, const Level &u, const Level &up, const Level &un, double ea, double eb,
-                           double ec, cudaStream_t s)
+// the intermediate planes.
+mol_status run_update_with(mol_ctx *h, void *const *inter, const Level &u, const Level &up, const Level &un, double ea,
+                           double eb, double ec, cudaStream_t s)
 {
     const int P = h->P;
     HornerParams hp = h->xtpl;
@@ -471,28 +525,28 @@ mol_status run_update_with(mol_ctx *h, void *const *inter, const double *xc, con
     hp.up_hi = up.hi; hp.up_lo = up.lo;
     hp.un_hi = un.hi; hp.un_lo = un.lo;
     mol_status st;
-    if (h->ndim == 1) return run_horner(h, 0, hp, xc, xu, s);
+    f64_units(hp, f64_unit(h, 0), h->ndim == 2 ? f64_unit(h, 1) : 1.0);
+    if (h->ndim == 1) return run_horner(h, 0, hp, s);
     if (h->ndim == 2) {
-        if ((st = run_powers(h, 1, u, P, inter, s)) != MOL_OK) return st;
+        if ((st = run_powers(h, 1, u, P, inter, s, true)) != MOL_OK) return st;
         for (int k = 0; k < P; ++k) hp.g[k] = inter[k];
-        return run_horner(h, 0, hp, xc, xu, s);
+        return run_horner(h, 0, hp, s);
     }
-    if ((st = run_powers(h, 2, u, P, inter, s)) != MOL_OK) return st;
+    if ((st = run_powers(h, 2, u, P, inter, s, true)) != MOL_OK) return st;
     HornerParams yp = h->ytpl;
+    f64_units(yp, f64_unit(h, 1), f64_unit(h, 2));
     yp.u_hi = u.hi; yp.u_lo = u.lo;
     for (int k = 0; k < P; ++k) yp.g[k] = inter[k];
     for (int o = 0; o <= P; ++o) yp.out[o] = inter[P + o];
-    if ((st = run_horner(h, 1, yp, yc, yu, s)) != MOL_OK) return st;
+    if ((st = run_horner(h, 1, yp, s)) != MOL_OK) return st;
     for (int k = 0; k <= P; ++k) hp.g[k] = inter[P + k];
-    return run_horner(h, 0, hp, xc, xu, s);
+    return run_horner(h, 0, hp, s);
 }
 
 mol_status run_update(mol_ctx *h, const Level &u, const Level &up, const Level &un,
                       double ea, double eb, double ec, cudaStream_t s)
 {
-    const double *b = h->coef_dev;
-    return run_update_with(h, h->inter.data(), b + h->off_xc, b + h->off_xu, b + h->off_yc, b + h->off_yu, u, up,
-                           un, ea, eb, ec, s);
+    return run_update_with(h, h->inter.data(), u, up, un, ea, eb, ec, s);
 }
 
 // 2D Dirichlet handles of float32-pair levels whose x rows split over warps
@@ -535,8 +589,6 @@ mol_status run_update_T(mol_ctx *h, const Level &u, const Level &up, const Level
     x.ng = hp.ng;
     x.nout = hp.nout;
     for (int k = 0; k < MAXG; ++k) { x.g[k] = hp.g[k]; x.out[k] = hp.out[k]; }
-    x.coef = h->coef_dev + h->off_xc;
-    x.cu = h->coef_dev + h->off_xu;
     x.epi = hp.epi;
     x.ea = ea; x.eb = eb; x.ec = ec;
     x.u_hi = u.hi; x.u_lo = u.lo; x.up_hi = up.hi; x.up_lo = up.lo; x.un_hi = un.hi; x.un_lo = un.lo;
@@ -776,6 +828,10 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
     }
     if ((e = configure_kernels()) != cudaSuccess) { st = cuda_fail(h, e, "kernel attributes"); goto bad; }
     if ((e = configure_regs_kernels()) != cudaSuccess) { st = cuda_fail(h, e, "kernel attributes"); goto bad; }
+    if (prec == MOL_FP64 && (e = configure_f64_kernels()) != cudaSuccess) {
+        st = cuda_fail(h, e, "kernel attributes");
+        goto bad;
+    }
     if (!expand_coefficients(h->ndim, P, beta, h->f)) { st = fail(h, MOL_EINVAL, "coefficient expansion failed"); goto bad; }
 
     for (int a = 0; a < h->ndim; ++a) {
@@ -802,26 +858,7 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
             for (int k = 0; k < 5; ++k)
                 h->dmr_ax[a][r][k] = std::exp(-h->nu[a] * (double)(8 << r) * (double)(1 << k));
     }
-    {
-        build_tables(h);
-        std::vector<double> xc, xu, yc, yu, all;
-        flatten(h->xtpl, xc, xu);
-        if (h->ndim == 3) flatten(h->ytpl, yc, yu);
-        else { yc.assign(1, 0.0); yu.assign(1, 0.0); }
-        h->off_xc = 0;
-        h->off_xu = xc.size();
-        h->off_yc = h->off_xu + xu.size();
-        h->off_yu = h->off_yc + yc.size();
-        all = xc;
-        all.insert(all.end(), xu.begin(), xu.end());
-        all.insert(all.end(), yc.begin(), yc.end());
-        all.insert(all.end(), yu.begin(), yu.end());
-        if ((st = dev_alloc(h, (void **)&h->coef_dev, sizeof(double) * all.size())) != MOL_OK) goto bad;
-        if ((e = cudaMemcpy(h->coef_dev, all.data(), sizeof(double) * all.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
-            st = cuda_fail(h, e, "coefficient upload");
-            goto bad;
-        }
-    }
+    build_tables(h);
     // levels: three rotating buffers
     for (int k = 0; k < 3; ++k) {
         if (prec == MOL_MIXED) {
@@ -841,7 +878,7 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
             if ((st = dev_alloc(h, &h->inter[k], (size_t)h->tbytes * h->N)) != MOL_OK) goto bad;
     }
     default_rows_split(h);
-    if (h->ndim == 2 && bc == MOL_BC_DIRICHLET && h->n[0] <= 1024 && h->n[1] <= 1024) {
+    if (prec == MOL_MIXED && h->ndim == 2 && bc == MOL_BC_DIRICHLET && h->n[0] <= 1024 && h->n[1] <= 1024) {
         int r = 0, S = 0, K = 0;
         const bool xreg = regs_res_plan(h->tbytes, (int)h->n[0], h->xtpl.ng, &r) ||
                           regs_contig_plan(h->tbytes, h->bc, (int)h->n[0], &r);
@@ -1036,7 +1073,8 @@ mol_status mol_autotune(mol_handle h, void *stream)
     int dummy = 0, r0 = 0, S0 = 0, K0 = 0;
     const bool res = h->ndim >= 2 && regs_res_plan(h->tbytes, (int)h->n[0], h->xtpl.ng, &dummy);
     bool strided = false;
-    for (int a = 1; a < h->ndim; ++a) strided |= regs_strided_plan(h->tbytes, h->bc, (int)h->n[a], &r0, &S0, &K0);
+    for (int a = 1; a < h->ndim; ++a)              // (the float64 passes pick their own shapes)
+        strided |= h->tbytes == 4 && regs_strided_plan(h->tbytes, h->bc, (int)h->n[a], &r0, &S0, &K0);
     // x variants: one warp per row with 1, 2 or 4 warps per CTA (code 1, 2, 4),
     // or each row split over 2, 4 or 8 warps, one CTA per row (code -2, -4,
     // -8) or persistent CTAs (code -102, -104, -108)
@@ -1378,8 +1416,7 @@ mol_status mol_solve_dirichlet(mol_handle h, const double *u0, int64_t nsteps, c
             }
         hp.bnew[0] = data[((k + 1) * 2 + 0) * Q];
         hp.bnew[1] = data[((k + 1) * 2 + 1) * Q];
-        const double *b = h->coef_dev;
-        if ((st = run_horner(h, 0, hp, b + h->off_xc, b + h->off_xu, s)) != MOL_OK) return st;
+        if ((st = run_horner(h, 0, hp, s)) != MOL_OK) return st;
         const int t0 = ip; ip = ic; ic = in; in = t0;
     }
     return store_level(h, h->lev[ic], u_out, s);
@@ -1543,17 +1580,16 @@ mol_status mol_pass_times(mol_handle h, double total_ms[3], int64_t launches[3])
 // nearly all of the device, so that cudaMalloc fails or forces the cache to
 // be emptied; and loops that cannot afford cudaFree, which synchronises the
 // whole device.  mol_apply_F_noalloc serves them.  Every buffer it needs
-// besides u and F -- the intermediate planes of the pass plan, the tables
-// d^j and the Horner coefficients -- lives in the fixed array below, so the
-// array's size bounds the grids it accepts.
+// besides u and F -- the intermediate planes of the pass plan and the tables
+// d^j -- lives in the fixed array below, so the array's size bounds the grids
+// it accepts.
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocScratchBytes / sizeof(double)];
 
 namespace {
 
 constexpr int kNoallocMaxDevices = 64;
-constexpr int kNoallocCoefCap = 512;   // doubles reserved for the Horner tables
-constexpr int kNoallocCoefMax = 288;   // >= the 258 table entries of 3D, P = 5; keeps the
-                                       // parameter block of k_noalloc_tables under 4 KB
+constexpr int kNoallocReserved = 512;  // doubles kept free at the start of the array (part of the
+                                       // documented size of a call)
 std::atomic<double *> g_noalloc_ptr[kNoallocMaxDevices];
 int g_noalloc_sms[kNoallocMaxDevices];
 int g_noalloc_smem[kNoallocMaxDevices];
@@ -1577,6 +1613,7 @@ mol_status noalloc_setup(int dev, double **out)
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaGetSymbolAddress of the static scratch");
         if ((e = configure_kernels()) != cudaSuccess) return cuda_fail(nullptr, e, "kernel attributes");
         if ((e = configure_regs_kernels()) != cudaSuccess) return cuda_fail(nullptr, e, "kernel attributes");
+        if ((e = configure_f64_kernels()) != cudaSuccess) return cuda_fail(nullptr, e, "kernel attributes");
         int v = 0;
         g_noalloc_sms[dev] = (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
                                  ? v : 152;
@@ -1654,9 +1691,6 @@ bool expand_fixed(int ndim, int P, double beta, FPoly &F)
 // Constants written into the scratch by one small kernel at the start of
 // every call (they travel as the kernel's parameters, so no host copy).
 struct NoallocTables {
-    double *coef_dst;
-    int ncoef;
-    double coef[kNoallocCoefMax];
     double *dpow[3];
     int n[3];
     double nu[3];
@@ -1665,7 +1699,6 @@ struct NoallocTables {
 __global__ void k_noalloc_tables(const NoallocTables t)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < t.ncoef) t.coef_dst[i] = t.coef[i];
     for (int a = 0; a < 3; ++a)
         if (t.dpow[a] && i <= t.n[a]) t.dpow[a][i] = exp(-t.nu[a] * (double)i);
 }
@@ -1696,13 +1729,12 @@ extern "C" mol_status mol_apply_F_noalloc(const mol_grid *grid, double c, double
     if (beta > bmax * (1.0 + 1e-12) && !unstable_allowed())
         return fail(nullptr, MOL_EUNSTABLE, "beta above beta_max(P): the scheme is not A-stable");
 
-    // scratch layout (doubles, every part 256-byte aligned): Horner tables,
-    // d^j per axis, intermediate planes (2D: D_y^k u; 3D: D_z^k u and the
+    // scratch layout (doubles, every part 256-byte aligned): d^j per axis, intermediate planes (2D: D_y^k u; 3D: D_z^k u and the
     // P + 1 outputs of the y pass)
     const int ndim = grid->ndim;
     const int nplanes = ndim == 2 ? P : (ndim == 3 ? 2 * P + 1 : 0);
     size_t off_dpow[3] = {0, 0, 0};
-    size_t need = kNoallocCoefCap;
+    size_t need = kNoallocReserved;
     for (int a = 0; a < ndim; ++a) { off_dpow[a] = need; need += round_up32((size_t)grid->n[a] + 1); }
     const size_t off_planes = need;
     need += (size_t)nplanes * round_up32((size_t)N);
@@ -1775,34 +1807,8 @@ extern "C" mol_status mol_apply_F_noalloc(const mol_grid *grid, double c, double
     if (!expand_fixed(ndim, P, beta, f)) return fail(nullptr, MOL_EINVAL, "coefficient expansion failed");
     fill_tables(ndim, P, [&f](int i, int j, int k) { return f.c[fidx(i, j, k)]; }, h.xtpl, h.ytpl);
     default_rows_split(&h);                           // as mol_create (float64: one warp per row either way)
-    // flattened like flatten(): per output o and Horner term t, the ng field
-    // weights, then the weights of u
-    double flat[2 * kNoallocCoefMax];
-    size_t off[4];
-    int nc = 0;
-    const HornerParams *tp[2] = {&h.xtpl, &h.ytpl};
-    for (int q = 0; q < 2; ++q) {
-        const HornerParams &hp = *tp[q];
-        const bool used = q == 0 || ndim == 3;
-        off[2 * q] = nc;
-        if (used)
-            for (int o = 0; o < std::max(hp.nout, 1); ++o)
-                for (int t = 0; t <= hp.P; ++t)
-                    for (int k = 0; k < hp.ng; ++k) flat[nc++] = hp.coef[o][t][k];
-        if (nc == (int)off[2 * q]) flat[nc++] = 0.0;
-        off[2 * q + 1] = nc;
-        if (used)
-            for (int o = 0; o < std::max(hp.nout, 1); ++o)
-                for (int t = 0; t <= hp.P; ++t) flat[nc++] = hp.cu[o][t];
-        if (nc == (int)off[2 * q + 1]) flat[nc++] = 0.0;
-    }
-    if (nc > kNoallocCoefMax) return fail(nullptr, MOL_EINVAL, "coefficient tables exceed their reserved space");
-    for (int i = 0; i < nc; ++i) tb.coef[i] = flat[i];
-    tb.coef_dst = scratch;
-    tb.ncoef = nc;
-
     cudaStream_t s = (cudaStream_t)stream;
-    const int nthr = 256, nblk = (std::max(nmax, nc) + nthr - 1) / nthr;
+    const int nthr = 256, nblk = (nmax + nthr - 1) / nthr;
     k_noalloc_tables<<<nblk, nthr, 0, s>>>(tb);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "table kernel launch");
 
@@ -1811,8 +1817,7 @@ extern "C" mol_status mol_apply_F_noalloc(const mol_grid *grid, double c, double
     Level U, O;
     U.hi = (void *)u;
     O.hi = F;
-    st = run_update_with(&h, inter, scratch + off[0], scratch + off[1], scratch + off[2], scratch + off[3], U, U, O,
-                         0.0, 0.0, 1.0, s);
+    st = run_update_with(&h, inter, U, U, O, 0.0, 0.0, 1.0, s);
     if (st != MOL_OK) g_err = h.err;
     return st;
 }

@@ -1,0 +1,482 @@
+// molt_f64.cuh -- float64 line passes (sm_103a), any line length.
+//
+// GB300 retires two float64 lane-operations per SM and clock (measured:
+// 0.53 T fma/s, against 0.85 T values/s of HBM traffic), so a float64 pass is
+// bound by how many float64 operations it spends on a point; everything else
+// -- shared memory, barriers, integer work -- runs in the shadow of that pipe.
+// These passes spend 7 on an application of D (the earlier ones 13):
+//
+//   * D in the form  e = kappa (rho s + g),  (1 + d^2) g_j - d (g_{j-1} + g_{j+1}) = s_j,
+//     s the second difference of the input.  It is the difference form
+//     q_j = c1 s_j + c2 (s_{j-1} + s_{j+1}) of molt_kernels.cuh with the part
+//     of q that the solve would undo taken out: with gamma = -c2 / d,
+//     c1 s_j + c2 (s_{j-1} + s_{j+1}) = gamma (T s)_j + (c1 - gamma (1 + d^2)) s_j
+//     for T the operator on the left, so e = gamma s + kappa T^{-1} s, kappa =
+//     c1 - gamma (1 + d^2), rho = gamma / kappa.  Forming s costs 2, the term
+//     rho s 1 instead of 3 for q.
+//   * kappa never touches a point: the powers leave their units to the
+//     consumer's Horner weights (host: coefficients times kappa^p).
+//   * each thread owns a segment of R points in registers and solves it once
+//     with zero inflow (causal, then anti-causal in place: 2 operations); what
+//     flows in from the other segments and the line ends adds a d^k +
+//     b d^(len-1-k) (2 operations), both powers being constants of the launch.
+//     The earlier scheme reduced, rescanned and reduced again.
+//
+// Carries: each segment publishes E (its zero-inflow y at its last point) and
+// G (its zero-inflow g at its first point).  After one barrier every segment
+// sums the inflow from as many neighbours as matter (d^(R win) <= 2^-60; the
+// whole line where the decay is slow):
+//   yin = sum_j d^(R (j-1)) E_{m-j},
+//   gin = sum_{l>m} d^(R (l-m-1)) (G_l + W Y_{l-1}),  Y_l = E_l + d^R Y_{l-1},
+//   W = d (1 - d^2R) / (1 - d^2);
+//   a = yin d / (1 - d^2),  b = gin d - yin d^(len+2) / (1 - d^2).
+// Dirichlet (e = 0, or given data, at the ends; s_0 := s_1, s_{n-1} := s_{n-2}):
+// the rows at the ends drop out of s, and A' d^j + B' d^(n-1-j) with
+//   A' + mu B' = r_0 = e_0/kappa - rho s_1 - g_0,
+//   mu A' + B' = r_1 = e_{n-1}/kappa - rho s_{n-2} - g_{n-1}
+// joins a and b in the segments it reaches.  Periodic lines wrap (all images
+// through 1 / (1 - mu) where the window covers the line).  The last segment
+// may hold fewer than R points.
+//
+// One kernel serves every axis: on the contiguous one neighbouring threads hold
+// neighbouring segments of a row and each reads its own segment in 32-byte
+// vectors (whole sectors; the segments of a warp are not coalesced, but the
+// load unit stays below a tenth of its rate beside the float64 pipe, and
+// neither staging nor its barriers are needed); on the strided ones
+// neighbouring threads hold neighbouring columns, so that every access is a
+// run of C columns.  s waits in shared memory while its registers hold y and g.
+//
+// Measured, us per pass, against the earlier warp-per-row, clustered and
+// shared-memory kernels: 2048^2, P = 3, y 419 -> 219, x 1470 -> 355 (23 and 40
+// operations a point: 86 % and 84 % of the float64 pipe's cycles); 96 x 100 x
+// 75, P = 2, x 154 -> 52, y 260 -> 143, z 72 -> 32; 256^3 periodic, P = 2, x
+// 1150 -> 764, y 3000 -> 2124, z 746 -> 466.
+#pragma once
+#include <cstdint>
+#include <cuda_runtime.h>
+#include "molt_kernels.cuh"
+
+namespace molt {
+
+constexpr int kF64MaxR = 32;
+constexpr int kF64Threads = 256;       // threads per CTA at most
+
+// Constants of one axis for segments of R points (host, molt_f64.cu).
+struct F64Axis {
+    int n, G, len_last;    // points, segments, points of the last one
+    int win;               // segments whose inflow matters on each side
+    double d, rho, kappa;
+    double dR, dRl;        // d^R, d^len_last
+    double W, Wl;          // d (1 - d^2len) / (1 - d^2), len = R and len_last
+    double a1;             // d / (1 - d^2)
+    double bR, bl;         // d^(len+2) / (1 - d^2)
+    double mu, inv;        // as AxisDev
+    double pw[kF64MaxR];   // d^k
+    const double *dpow;    // d^j, j = 0..n
+};
+
+struct F64Lines {
+    int64_t stride, inner, nlines;
+    int C, cshift;         // lines per CTA; log2 C (strided axes)
+};
+
+// The program of a pass: powers (P applications to u, out[p-1] = scale[p-1]
+// D^p u / kappa^p) or the Horner pass of HornerParams with its weights times
+// kappa^t.  Zero weights, unit scales and the level's weights are flagged by
+// the host (a comparison would cost the float64 pipe an operation).
+struct F64Prog {
+    int P, ng, nout, epi;
+    unsigned add[MAXP][MAXP];  // [o][t]: bit k set where field k has a weight
+    unsigned ucu[MAXP];        // [o]: bit t set where u has a weight in step t
+    unsigned scaled;           // bit p-1: scale[p-1] != 1
+    bool hea, heb, hec;        // ea, eb != 0, ec != 1
+    bool vec;                  // contiguous axis: every segment starts on 32 bytes
+    const double *g[MAXG];
+    double *out[MAXG];
+    double scale[MAXG];
+    double coef[MAXP][MAXP][MAXG];
+    double cu[MAXP][MAXP];
+    double ea, eb, ec;
+    const double *u, *up;
+    double *un;
+};
+
+// this thread's place on its line
+struct F64Seg {
+    double *E, *G, *ends;      // slots [threads] and [4][C]
+    double *s;                 // this segment's s: s[k ss]
+    int ss;
+    int t, st, t0;             // slot, distance to the next segment's slot, slot of segment 0
+    int seg, line, C;
+    bool live, last, tail;     // on the line; its last segment; shorter than R
+};
+
+template <int R>
+__device__ __forceinline__ double f64_pick(const double (&z)[R], int k)
+{
+    double v = z[0];
+#pragma unroll
+    for (int i = 1; i < R; ++i) v = (i == k) ? z[i] : v;
+    return v;
+}
+
+// Inflow of this segment, a d^k + b d^(len-1-k), and the right sides r_0, r_1
+// of the boundary terms where this thread has them: on the strided axes every
+// thread within reach of an end sums them for itself (a warp holds one
+// segment, so the others skip it); on the contiguous axis the end segments
+// alone have them, from their own inflow.
+template <int R, int BC, bool CONTIG>
+__device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, double &a, double &b, double &r0, double &r1)
+{
+    const int G = A.G, m = c.seg;
+    const int J = A.win < G ? A.win : G;
+    const double *E = c.E, *Gs = c.G;
+    auto slot = [&](int l) { return c.t0 + l * c.st; };
+    auto pl = [&](int l) -> double { return l == G - 1 ? A.dRl : A.dR; };
+    double yin = 0.0, gin = 0.0;
+    r0 = r1 = 0.0;
+    if (BC == BC_PERIODIC) {
+        // J segments back, farthest first; then J segments on
+        int l = m - J;
+        if (l < 0) l += G;
+        for (int j = 0; j < J; ++j) {
+            yin = fma(pl(l), yin, E[slot(l)]);
+            l = l + 1 == G ? 0 : l + 1;
+        }
+        if (J == G) yin *= A.inv;
+        double Y = fma(pl(m), yin, E[c.t]), pr = 1.0;
+        l = m + 1 == G ? 0 : m + 1;
+        for (int j = 0; j < J; ++j) {
+            gin = fma(pr, fma(l == G - 1 ? A.Wl : A.W, Y, Gs[slot(l)]), gin);
+            Y = fma(pl(l), Y, E[slot(l)]);
+            pr *= pl(l);
+            l = l + 1 == G ? 0 : l + 1;
+        }
+        if (J == G) gin *= A.inv;
+    } else {
+        for (int l = max(m - J, 0); l < m; ++l) yin = fma(A.dR, yin, E[slot(l)]);
+        double Y = fma(A.dR, yin, E[c.t]), pr = 1.0;
+        for (int l = m + 1; l <= min(m + J, G - 1); ++l) {
+            gin = fma(pr, fma(l == G - 1 ? A.Wl : A.W, Y, Gs[slot(l)]), gin);
+            Y = fma(A.dR, Y, E[slot(l)]);
+            pr *= A.dR;
+        }
+        if (CONTIG) {
+            if (m == 0) r0 = fma(-A.rho, c.ends[c.line], -fma(c.last ? A.dRl : A.dR, gin, Gs[c.t]));
+            if (c.last) r1 = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, yin, E[c.t]));
+        } else {
+            const bool all = A.win >= G;
+            if (all || m < A.win) {
+                double Yl = 0.0, pw = 1.0, g0 = 0.0;
+                for (int l = 0; l < min(J + 1, G); ++l) {
+                    g0 = fma(pw, fma(l == G - 1 ? A.Wl : A.W, Yl, Gs[slot(l)]), g0);
+                    Yl = fma(A.dR, Yl, E[slot(l)]);
+                    pw *= A.dR;
+                }
+                r0 = fma(-A.rho, c.ends[c.line], -g0);
+            }
+            if (all || G - 1 - m < A.win) {
+                double Yl = 0.0;
+                for (int l = max(G - 1 - J, 0); l < G - 1; ++l) Yl = fma(A.dR, Yl, E[slot(l)]);
+                r1 = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, Yl, E[slot(G - 1)]));
+            }
+        }
+    }
+    a = yin * A.a1;
+    b = fma(gin, A.d, -(yin * (c.last ? A.bl : A.bR)));
+}
+
+// z: s on entry, rho s + T^{-1} s (with the boundary terms) on exit.  Every
+// thread of the CTA calls it (one barrier; two on a contiguous Dirichlet axis).
+template <int R, int BC, bool CONTIG>
+__device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, const F64Seg &c)
+{
+    const double d = A.d;
+    const int L = A.len_last;
+    if (c.live) {
+        if (BC == BC_DIRICHLET) {
+            if (c.seg == 0) {
+                c.ends[c.line] = z[1];
+                z[0] = 0.0;
+            }
+            // s_{n-2}: the last segment's, or the end of the one before it
+            if (L >= 2 ? c.last : c.seg == A.G - 2) c.ends[c.C + c.line] = f64_pick<R>(z, L >= 2 ? L - 2 : R - 1);
+        }
+        if (c.last) {
+            const int keep = BC == BC_DIRICHLET ? L - 1 : L;
+#pragma unroll
+            for (int k = 0; k < R; ++k) z[k] = k < keep ? z[k] : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) c.s[k * c.ss] = z[k];
+#pragma unroll
+        for (int k = 1; k < R; ++k) z[k] = fma(d, z[k - 1], z[k]);
+        double e = z[R - 1];
+        if (c.tail) {                                  // y ends with the line
+            e = f64_pick<R>(z, L - 1);
+#pragma unroll
+            for (int k = 0; k < R; ++k) z[k] = k < L ? z[k] : 0.0;
+        }
+#pragma unroll
+        for (int k = R - 2; k >= 0; --k) z[k] = fma(d, z[k + 1], z[k]);
+        c.E[c.t] = e;
+        c.G[c.t] = z[0];
+    }
+    __syncthreads();
+    double a = 0.0, b = 0.0, r0 = 0.0, r1 = 0.0;
+    if (c.live) f64_inflow<R, BC, CONTIG>(A, c, a, b, r0, r1);
+    if (CONTIG && BC == BC_DIRICHLET) {
+        double *v = c.ends + 2 * c.C + c.line;
+        if (c.live && c.seg == 0) v[0] = r0;
+        if (c.live && c.last) v[c.C] = r1;
+        __syncthreads();
+        if (c.live) {
+            r0 = v[0];
+            r1 = v[c.C];
+        }
+    }
+    if (c.live) {
+        if (BC == BC_DIRICHLET) {
+            // the boundary terms in the segments they reach: of both ends
+            // where the window covers the line, else of the nearer end alone
+            const bool all = A.win >= A.G;
+            if (all) {
+                const double t0 = (r0 - A.mu * r1) * A.inv;
+                r1 = (r1 - A.mu * r0) * A.inv;
+                r0 = t0;
+            }
+            const int a0 = c.seg * R;
+            if (all || c.seg < A.win) a = fma(r0, A.dpow[a0], a);
+            if (all || A.G - 1 - c.seg < A.win) b = fma(r1, A.dpow[A.n - a0 - (c.last ? L : R)], b);
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) z[k] = fma(a, A.pw[k], fma(A.rho, c.s[k * c.ss], z[k]));
+        if (c.tail) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) z[k] = k < L ? fma(b, A.pw[k < L ? L - 1 - k : 0], z[k]) : 0.0;
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k) z[k] = fma(b, A.pw[R - 1 - k], z[k]);
+        }
+        if (BC == BC_DIRICHLET) {
+            if (c.seg == 0) z[0] = 0.0;
+            if (c.last) {
+#pragma unroll
+                for (int k = 0; k < R; ++k) z[k] = k == L - 1 ? 0.0 : z[k];
+            }
+        }
+    }
+}
+
+// z <- second difference of z (+ cu r), zl and zr the neighbours' values; the
+// last segment's right neighbour enters at its own length
+template <int R>
+__device__ __forceinline__ void f64_sdiff(double (&z)[R], double zl, double zr, const F64Axis &A, const F64Seg &c)
+{
+    if (c.tail) {
+#pragma unroll
+        for (int k = 1; k < R; ++k) z[k] = k == A.len_last ? zr : z[k];
+    }
+    double dm = z[0] - zl;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const double dp = (k + 1 < R ? z[k + 1] : zr) - z[k];
+        z[k] = dp - dm;
+        dm = dp;
+    }
+}
+
+// f(k, v) for this segment's points k < len of a field, v = q[k st].  vec: in
+// 32-byte vectors (contiguous axis; len is a multiple of 4 then).
+template <int R, bool CONTIG, class F>
+__device__ __forceinline__ void f64_each(const double *__restrict__ q, int64_t st, int len, bool vec, F &&f)
+{
+    if (CONTIG && vec) {
+#pragma unroll
+        for (int k = 0; k < R; k += 4)
+            if (k < len) {
+                const double4_32a v = *reinterpret_cast<const double4_32a *>(q + k);
+                f(k, v.x);
+                f(k + 1, v.y);
+                f(k + 2, v.z);
+                f(k + 3, v.w);
+            }
+    } else if (CONTIG) {
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            if (k < len) f(k, q[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            if (k < len) f(k, *q);
+            q += st;
+        }
+    }
+}
+
+template <int R, bool CONTIG>
+__device__ __forceinline__ void f64_store(double *q, int64_t st, int len, bool vec, const double (&z)[R])
+{
+    if (CONTIG && vec) {
+#pragma unroll
+        for (int k = 0; k < R; k += 4)
+            if (k < len) {
+                double4_32a v;
+                v.x = z[k];
+                v.y = z[k + 1];
+                v.z = z[k + 2];
+                v.w = z[k + 3];
+                *reinterpret_cast<double4_32a *>(q + k) = v;
+            }
+    } else {
+        const int64_t s1 = CONTIG ? 1 : st;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            if (k < len) *q = z[k];
+            q += s1;
+        }
+    }
+}
+
+// KM 0: powers; 1: Horner with nout outputs (or the next level).  Dynamic
+// shared memory: slots [4][threads] (E, G, first, last), ends [4][C], s [R]
+// [threads], (KM 1) r [R][threads].
+__host__ __device__ inline size_t f64_smem(int threads, int C, int R, bool horner)
+{
+    return sizeof(double) * ((size_t)threads * 4 + 4 * C + (size_t)R * threads * (horner ? 2 : 1));
+}
+
+template <int R, int BC, int KM, bool CONTIG>
+__global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ F64Axis A, F64Lines LS,
+                                                       const __grid_constant__ F64Prog p)
+{
+    extern __shared__ __align__(16) double sm64[];
+    const int T = blockDim.x, t = threadIdx.x, n = A.n, G = A.G;
+    double *first = sm64 + 2 * T, *last = sm64 + 3 * T, *sbuf = sm64 + 4 * T + 4 * LS.C;
+    F64Seg c;
+    c.E = sm64;
+    c.G = sm64 + T;
+    c.ends = sm64 + 4 * T;
+    c.s = sbuf + t;
+    c.ss = T;
+    c.t = t;
+    c.C = LS.C;
+    if (CONTIG) {
+        c.line = t / G;
+        c.seg = t - c.line * G;
+        c.t0 = c.line * G;
+        c.st = 1;
+        c.live = c.line < LS.C;
+    } else {
+        c.line = t & (LS.C - 1);
+        c.seg = t >> LS.cshift;
+        c.t0 = c.line;
+        c.st = LS.C;
+        c.live = c.seg < G;
+    }
+    c.last = c.seg == G - 1;
+    c.tail = c.last && A.len_last < R;
+    const int a = c.seg * R, len = c.last ? A.len_last : R;
+    const int64_t line = (int64_t)blockIdx.x * LS.C + c.line;
+    const bool io = c.live && line < LS.nlines;
+    const int64_t st = CONTIG ? 1 : LS.stride;
+    const int64_t lbase = !io ? 0 : CONTIG ? line * n : (line % LS.inner) + (line / LS.inner) * LS.inner * (int64_t)n;
+    const int64_t at = lbase + (int64_t)a * st;        // this segment's first point
+
+    double z[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) z[k] = 0.0;
+    // s of u: points a-1 .. a+len (wrapped or clamped)
+    if (io) {
+        auto row = [&](int j) -> int64_t {
+            if (BC == BC_PERIODIC) return j < 0 ? j + n : (j >= n ? j - n : j);
+            return j < 0 ? 0 : (j > n - 1 ? n - 1 : j);
+        };
+        const double zl = p.u[lbase + row(a - 1) * st], zr = p.u[lbase + row(a + len) * st];
+        f64_each<R, CONTIG>(p.u + at, st, len, p.vec, [&](int k, double v) { z[k] = v; });
+        f64_sdiff<R>(z, zl, zr, A, c);
+    }
+    // neighbours' values through shared memory, then the second difference
+    auto exchange_sdiff = [&]() {
+        if (c.live) {
+            first[t] = z[0];
+            last[t] = c.tail ? f64_pick<R>(z, A.len_last - 1) : z[R - 1];
+        }
+        __syncthreads();
+        if (c.live) {
+            double zl = 0.0, zr = 0.0;
+            const int sl = c.seg > 0 ? c.seg - 1 : (BC == BC_PERIODIC ? G - 1 : -1);
+            const int sr = c.last ? (BC == BC_PERIODIC ? 0 : -1) : c.seg + 1;
+            if (sl >= 0) zl = last[c.t0 + sl * c.st];
+            if (sr >= 0) zr = first[c.t0 + sr * c.st];
+            f64_sdiff<R>(z, zl, zr, A, c);
+        }
+    };
+
+    if (KM == 0) {
+        for (int q = 0; q < p.P; ++q) {
+            if (q > 0) exchange_sdiff();
+            f64_solve<R, BC, CONTIG>(z, A, c);
+            if (p.out[q] != nullptr && io) {
+                if (p.scaled >> q & 1u) {              // the last power of mol_apply_D
+                    const double sc = p.scale[q];
+                    double w[R];
+#pragma unroll
+                    for (int k = 0; k < R; ++k) w[k] = sc * z[k];
+                    f64_store<R, CONTIG>(p.out[q] + at, st, len, p.vec, w);
+                } else {
+                    f64_store<R, CONTIG>(p.out[q] + at, st, len, p.vec, z);
+                }
+            }
+        }
+        return;
+    }
+    // Horner: r = s of u stays in shared memory
+    double *r = sbuf + (size_t)R * T + t;
+#pragma unroll
+    for (int k = 0; k < R; ++k) r[k * T] = z[k];
+    for (int o = 0; o < p.nout; ++o) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) z[k] = 0.0;
+        bool zero = true;
+        for (int q = p.P; q >= 0; --q) {
+            const unsigned add = p.add[o][q];
+            if (io)
+                for (int f = 0; f < p.ng; ++f)
+                    if (add >> f & 1u) {
+                        const double w = p.coef[o][q][f];
+                        f64_each<R, CONTIG>(p.g[f] + at, st, len, p.vec, [&](int k, double v) { z[k] = fma(w, v, z[k]); });
+                    }
+            zero = zero && add == 0;
+            if (q == 0) break;
+            const double w = p.cu[o][q];
+            if (zero) {
+                if (!(p.ucu[o] >> q & 1u)) continue;
+                __syncthreads();                   // the slots' last readers are done
+#pragma unroll
+                for (int k = 0; k < R; ++k) z[k] = w * r[k * T];
+            } else {
+                exchange_sdiff();
+                if (p.ucu[o] >> q & 1u) {
+#pragma unroll
+                    for (int k = 0; k < R; ++k) z[k] = fma(w, r[k * T], z[k]);
+                }
+            }
+            f64_solve<R, BC, CONTIG>(z, A, c);
+            zero = false;
+        }
+        if (!io) continue;
+        if (p.epi) {
+            // next level: ea u + eb u_prev + ec F
+            if (p.hec) {
+#pragma unroll
+                for (int k = 0; k < R; ++k) z[k] *= p.ec;
+            }
+            if (p.hea) f64_each<R, CONTIG>(p.u + at, st, len, p.vec, [&](int k, double v) { z[k] = fma(p.ea, v, z[k]); });
+            if (p.heb) f64_each<R, CONTIG>(p.up + at, st, len, p.vec, [&](int k, double v) { z[k] = fma(p.eb, v, z[k]); });
+        }
+        f64_store<R, CONTIG>((p.epi ? p.un : p.out[o]) + at, st, len, p.vec, z);
+    }
+}
+
+}  // namespace molt

@@ -76,9 +76,9 @@ bool regs_contig_plan(int tbytes, int bc, int n, int *rpt);
 // choice); max_warps: segments per CTA at most (1..8)
 bool regs_strided_plan(int tbytes, int bc, int n, int *rpt, int *S, int *K, int pref_rpt = 0, int max_warps = 8);
 size_t regs_strided_smem(int tbytes, int S, int rpt, bool horner);
-cudaError_t launch_contig(int tbytes, int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
+cudaError_t launch_contig(int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
                           cudaStream_t s);
-cudaError_t launch_strided(int tbytes, int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
+cudaError_t launch_strided(int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
                            cudaStream_t s);
 cudaError_t configure_regs_kernels();
 // The strided powers pass with one neighbour exchange per sweep (float32):
@@ -102,6 +102,22 @@ cudaError_t launch_strided_nb_h(int bc, int rpt, const AxisDev &A, const LineSet
 // The transposed strided powers (the adjoint step's y pass, Dirichlet,
 // float32) with one neighbour exchange per sweep, under the same condition.
 cudaError_t launch_strided_nb_T(int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p, cudaStream_t s);
+// The float64 line passes (molt_f64.cu): every float64 pass without boundary
+// data whose axis they take (f64_axis_ok); lines longer than that keep the
+// shared-memory kernels.  f64_kappa: the factor D's powers and Horner steps
+// leave out (D = kappa times what a sweep computes); the launcher's program
+// carries it in its weights and output scales.
+struct F64Plan {
+    int R, G, C, threads;     // segment length, segments per line, lines per CTA
+    size_t smem;
+};
+struct F64Prog;
+double f64_kappa(double nu, int quad);
+bool f64_axis_ok(int n, bool contig);
+bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sms, F64Plan *out);
+cudaError_t launch_f64(int bc, bool contig, const F64Plan &pl, double nu, int quad, const AxisDev &ax, int64_t stride,
+                       int64_t inner, int64_t nlines, bool horner, F64Prog p, cudaStream_t s);
+cudaError_t configure_f64_kernels();
 // 1 if a bounded wait of a register kernel gave up since the last call (and
 // clears it), 0 if not, -1 if the flag could not be read; synchronizes s.
 int regs_timeout_take(cudaStream_t s);

@@ -98,6 +98,7 @@ struct PowersParams {
     const void *u_hi;        // T == float: hi plane; T == double: the field
     const void *u_lo;        // T == float: lo plane
     void *out[MAXG];         // out[p-1] receives D^p u (nullptr: not stored)
+    bool raw;                // float64 line passes: out[p-1] receives D^p u / kappa^p
 };
 
 struct HornerParams {
@@ -131,34 +132,19 @@ struct ProgParams {
     int P, ng, nout;
     const void *g[MAXG];
     void *out[MAXG];
-    const double *coef;   // device, [nout][P+1][ng]
-    const double *cu;     // device, [nout][P+1]
     int epi;              // 1: out_0 combined into the next level
     double ea, eb, ec;    // u_next = ea u + eb u_prev + ec F
     const void *u_hi, *u_lo, *up_hi, *up_lo;
     void *un_hi, *un_lo;
-    // float32 copies for the float kernels (no float64 arithmetic on their
-    // paths): the tables in the kernel's parameter space, the level weights
+    // float32 Horner weights [nout][P+1][ng] and [nout][P+1] (the passes of this
+    // program are float32: no float64 arithmetic on their paths), level weights
     float coef32[MAXP * MAXP * MAXG];
     float cu32[MAXP * MAXP];
     float fea, feb, fec;
 };
 
-// Horner weights in the kernel's precision: float kernels read the copies in
-// the parameter space, float64 kernels the device tables
-template <class T> __device__ __forceinline__ T prog_coef(const ProgParams &p, size_t i)
-{
-    if constexpr (sizeof(T) == 4) return p.coef32[i];
-    else return __ldg(p.coef + i);
-}
-template <class T> __device__ __forceinline__ T prog_cu(const ProgParams &p, size_t i)
-{
-    if constexpr (sizeof(T) == 4) return p.cu32[i];
-    else return __ldg(p.cu + i);
-}
-
 // fills the float32 copies of a program's level weights and Horner weights
-// (flattened as the device tables: [o][t][k] and [o][t])
+// (flattened: [o][t][k] and [o][t])
 inline void prog_mirror(ProgParams &p, const HornerParams &hp)
 {
     int nc = 0, nu = 0;

@@ -351,8 +351,9 @@ cudaError_t attr_strided()
 }  // namespace
 
 // Segment lengths: contiguous lines use the smallest RPT with 32*RPT >= n;
-// strided lines use 64 (float) / 32 (double) points per thread by default,
-// or 32 (float) as an alternative the tuner may pick.
+// strided lines use 64 points per thread by default, or 32 as an alternative
+// the tuner may pick.  (Float64 passes run in molt_f64.cu; their handles still
+// answer for the launch choices a caller may set, in 32-point segments.)
 constexpr int kStridedRptF = 64, kStridedRptF2 = 32, kStridedRptD = 32;
 
 // Register kernels need whole segments: n a multiple of RPT (both boundary
@@ -485,36 +486,28 @@ size_t regs_strided_smem(int tbytes, int S, int rpt, bool horner)
     default: break;                                                                      \
     }
 
-cudaError_t launch_contig(int tbytes, int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
+cudaError_t launch_contig(int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
                           cudaStream_t s)
 {
-    if (tbytes == 4) {
-        if (bc == BC_PERIODIC) {
-            MOLT_CONTIG_R(float, BC_PERIODIC)
-            if (rpt == 64) return run_contig<float, BC_PERIODIC, 64>(A, L, p, s);
-        } else {
-            MOLT_CONTIG_R(float, BC_DIRICHLET)
-            if (rpt == 64) return run_contig<float, BC_DIRICHLET, 64>(A, L, p, s);
-        }
+    if (bc == BC_PERIODIC) {
+        MOLT_CONTIG_R(float, BC_PERIODIC)
+        if (rpt == 64) return run_contig<float, BC_PERIODIC, 64>(A, L, p, s);
     } else {
-        if (bc == BC_PERIODIC) { MOLT_CONTIG_R(double, BC_PERIODIC) }
-        else { MOLT_CONTIG_R(double, BC_DIRICHLET) }
+        MOLT_CONTIG_R(float, BC_DIRICHLET)
+        if (rpt == 64) return run_contig<float, BC_DIRICHLET, 64>(A, L, p, s);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_strided(int tbytes, int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
+cudaError_t launch_strided(int bc, int rpt, const AxisDev &A, const LineSet &L, const ProgParams &p,
                            cudaStream_t s)
 {
-    if (tbytes == 4 && rpt == kStridedRptF)
+    if (rpt == kStridedRptF)
         return bc == BC_PERIODIC ? run_strided<float, BC_PERIODIC, kStridedRptF>(A, L, p, s)
                                  : run_strided<float, BC_DIRICHLET, kStridedRptF>(A, L, p, s);
-    if (tbytes == 4 && rpt == kStridedRptF2)
+    if (rpt == kStridedRptF2)
         return bc == BC_PERIODIC ? run_strided<float, BC_PERIODIC, kStridedRptF2>(A, L, p, s)
                                  : run_strided<float, BC_DIRICHLET, kStridedRptF2>(A, L, p, s);
-    if (tbytes == 8 && rpt == kStridedRptD)
-        return bc == BC_PERIODIC ? run_strided<double, BC_PERIODIC, kStridedRptD>(A, L, p, s)
-                                 : run_strided<double, BC_DIRICHLET, kStridedRptD>(A, L, p, s);
     return cudaErrorInvalidValue;
 }
 
@@ -611,13 +604,8 @@ cudaError_t configure_regs_kernels()
     MOLT_A((attr_contig<float, BC_PERIODIC, 32>())) MOLT_A((attr_contig<float, BC_PERIODIC, 64>()))
     MOLT_A((attr_contig<float, BC_DIRICHLET, 8>())) MOLT_A((attr_contig<float, BC_DIRICHLET, 16>()))
     MOLT_A((attr_contig<float, BC_DIRICHLET, 32>())) MOLT_A((attr_contig<float, BC_DIRICHLET, 64>()))
-    MOLT_A((attr_contig<double, BC_PERIODIC, 8>())) MOLT_A((attr_contig<double, BC_PERIODIC, 16>()))
-    MOLT_A((attr_contig<double, BC_PERIODIC, 32>()))
-    MOLT_A((attr_contig<double, BC_DIRICHLET, 8>())) MOLT_A((attr_contig<double, BC_DIRICHLET, 16>()))
-    MOLT_A((attr_contig<double, BC_DIRICHLET, 32>()))
     MOLT_A((attr_strided<float, BC_PERIODIC, kStridedRptF>())) MOLT_A((attr_strided<float, BC_DIRICHLET, kStridedRptF>()))
     MOLT_A((attr_strided<float, BC_PERIODIC, kStridedRptF2>())) MOLT_A((attr_strided<float, BC_DIRICHLET, kStridedRptF2>()))
-    MOLT_A((attr_strided<double, BC_PERIODIC, kStridedRptD>())) MOLT_A((attr_strided<double, BC_DIRICHLET, kStridedRptD>()))
 #undef MOLT_A
     return cudaSuccess;
 }

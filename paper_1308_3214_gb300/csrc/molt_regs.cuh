@@ -627,7 +627,7 @@ __device__ __forceinline__ void stage_accumulate(T *stage, const ProgParams &pr,
     constexpr int NV = RPT / VN;                    // vectors per lane (n <= 32*RPT)
     const int nvec = n / VN;                        // n is a multiple of RPT, hence of VN
     for (int k = 0; k < pr.ng; ++k) {
-        const T ck = prog_coef<T>(pr, cf + k);
+        const T ck = pr.coef32[cf + k];
         if (ck == (T)0) continue;
         const V *__restrict__ src = reinterpret_cast<const V *>(reinterpret_cast<const T *>(pr.g[k]) + base);
         V buf[NV];
@@ -773,7 +773,7 @@ __global__ void __launch_bounds__(32 * WARPS, 3) k_contig(AxisDev A, LineSet LS,
             stage_to_regs<T, RPT>(stage, z, lane, false);
             __syncwarp();
         }
-        warp_sweep<T, BC, RPT, 2>(z, rline, prog_cu<T>(pr, t), A, lane);
+        warp_sweep<T, BC, RPT, 2>(z, rline, pr.cu32[t], A, lane);
     }
     // out = stage (coalesced side): level combination or plain store
     if (pr.epi) {
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(128) k_contig_res(AxisDev A, LineSet LS, ProgP
     for (int k = 0; k < RPT; ++k) z[k] = 0;
     for (int t = P; t >= 0; --t) {
         for (int k = 0; k < ng; ++k) {
-            const T c = prog_coef<T>(pr, (size_t)t * ng + k);
+            const T c = pr.coef32[t * ng + k];
             if (c == (T)0) continue;
             const float4 *seg = reinterpret_cast<const float4 *>(B + k * St::LINE + lane * St::SST);
 #pragma unroll
@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(128) k_contig_res(AxisDev A, LineSet LS, ProgP
             }
         }
         if (t == 0) break;
-        warp_sweep_rreg<T, BC, RPT>(z, r, prog_cu<T>(pr, t), A, lane);
+        warp_sweep_rreg<T, BC, RPT>(z, r, pr.cu32[t], A, lane);
     }
 
     // 4. F (segment layout) -> coalesced side -> next level
@@ -1551,7 +1551,7 @@ __global__ void __launch_bounds__(32 * W, W == 2 ? 8 : (W == 4 ? 7 : 4)) k_conti
     }
     for (int tt = pr.P; tt >= 0; --tt) {
         for (int k = 0; k < ng; ++k) {
-            const T c = prog_coef<T>(pr, (size_t)tt * ng + k);
+            const T c = pr.coef32[tt * ng + k];
             if (c == (T)0) continue;
             const float4 *sg = reinterpret_cast<const float4 *>(B + k * LINE + t * St::SST);
 #pragma unroll
@@ -1568,14 +1568,14 @@ __global__ void __launch_bounds__(32 * W, W == 2 ? 8 : (W == 4 ? 7 : 4)) k_conti
             }
         }
         if (tt == 0) break;
-        if constexpr (ADJ) row_sweep_T<T, RPT, W>(z, r, prog_cu<T>(pr, tt), A, lane, warp, sl);
+        if constexpr (ADJ) row_sweep_T<T, RPT, W>(z, r, pr.cu32[tt], A, lane, warp, sl);
         else if constexpr (NBX && W == 2)
-            row_sweep_nb<BC, RPT, W>(z, r, rl, rr, prog_cu<T>(pr, tt), A, nc, lane, warp, sl, tt & 1, hz[0], hz[1],
+            row_sweep_nb<BC, RPT, W>(z, r, rl, rr, pr.cu32[tt], A, nc, lane, warp, sl, tt & 1, hz[0], hz[1],
                                      hz[2], hz[3]);
         else if constexpr (NBX)
-            row_sweep_nb2<BC, RPT, W>(z, r, rl, rr, prog_cu<T>(pr, tt), A, nc, lane, warp, sl, tt & 1, hz[0], hz[1],
+            row_sweep_nb2<BC, RPT, W>(z, r, rl, rr, pr.cu32[tt], A, nc, lane, warp, sl, tt & 1, hz[0], hz[1],
                                       hz[2], hz[3]);
-        else row_sweep<T, BC, RPT, W>(z, r, rl, rr, prog_cu<T>(pr, tt), A, lane, warp, sl);
+        else row_sweep<T, BC, RPT, W>(z, r, rl, rr, pr.cu32[tt], A, lane, warp, sl);
     }
 
     // F -> coalesced side -> next level
@@ -2083,7 +2083,7 @@ __global__ void __launch_bounds__(256, 2) k_strided(AxisDev A, LineSet LS, ProgP
             const size_t cf = cfo + (size_t)t * ng;
             if (io) {
                 for (int q = 0; q < ng; ++q) {
-                    const T cq = prog_coef<T>(pr, cf + q);
+                    const T cq = pr.coef32[cf + q];
                     if (cq == (T)0) continue;
                     const T *gq = reinterpret_cast<const T *>(pr.g[q]) + lbase + (int64_t)a * st;
 #pragma unroll
@@ -2094,7 +2094,7 @@ __global__ void __launch_bounds__(256, 2) k_strided(AxisDev A, LineSet LS, ProgP
             T l2, l1, r0, r1;
             strided_halos<T, BC, RPT>(c, z, l2, l1, r0, r1, hpar);
             hpar ^= 1;
-            strided_sweep<T, BC, RPT, 2>(c, A, z, prog_cu<T>(pr, (size_t)o * (P + 1) + t), l2, l1, r0, r1, rs, rl, rr);
+            strided_sweep<T, BC, RPT, 2>(c, A, z, pr.cu32[(size_t)o * (P + 1) + t], l2, l1, r0, r1, rs, rl, rr);
         }
         T *ob = reinterpret_cast<T *>(pr.out[o]);
         if (io) {
