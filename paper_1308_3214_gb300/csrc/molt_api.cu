@@ -14,6 +14,7 @@
 #include "molt.h"
 #include "molt_internal.h"
 #include "molt_f64.cuh"
+#include "molt_line.cuh"
 #include "molt_recv.cuh"
 
 using namespace molt;
@@ -729,6 +730,95 @@ mol_status build_graph(mol_ctx *h, int k)
     return MOL_OK;
 }
 
+// ---------------------------------------------------------------------------
+// 1D time loops: many steps per launch (molt_line.cuh)
+// ---------------------------------------------------------------------------
+constexpr int64_t kLineSteps = 4096;     // steps per launch without boundary data
+
+struct LineEnds {
+    double bgL[MAXP], bgR[MAXP], bnew[2];     // as HornerParams
+};
+
+// True when the handle's steps run that way: 1D, graphs on (use_graphs 0 asks
+// for one launch per step), no pass timing.  rpt: float32 lines of whole
+// segments; else A (and cta) of the shared-memory sweeps.
+bool line_loop(const mol_ctx *h, bool data, int *rpt, bool *cta, AxisDev *A)
+{
+    if (h->ndim != 1 || !h->opt.use_graphs || h->timing) return false;
+    *rpt = 0;
+    *cta = false;
+    const int n = (int)h->n[0];
+    if (h->prec == MOL_FP64) return true;
+    int r = 0;
+    if (!data && h->tune_rows_warps > 0 && regs_rows_plan(h->tbytes, n, 0, h->tune_rows_warps, &r)) return false;
+    if (!data && regs_res_plan(h->tbytes, n, 0, rpt)) {
+        *A = regs_axis(h, 0, *rpt);
+        return true;
+    }
+    PassGeom G;
+    smem_pass_geom(h, 0, true, G, *A);
+    *cta = G.cta != 0;
+    return line_smem_ok(*cta, *A, h->smem_optin);
+}
+
+// steps of the line from (u0, u1) = (u^{n-1}, u^n) (first: u1 = u^0 alone, the
+// first step is the start) to (v0, v1); the levels may be the same buffers.
+// data: one entry per step.
+mol_status run_line_f64(mol_ctx *h, const double *u0, const double *u1, double *v0, double *v1, int64_t steps, bool first,
+                        const LineEnds *data, cudaStream_t s)
+{
+    F64LineRun p{};
+    p.P = h->P;
+    p.steps = (int)steps;
+    p.first = first;
+    p.data = data != nullptr;
+    p.u0 = u0; p.u1 = u1; p.v0 = v0; p.v1 = v1;
+    const double k = f64_kappa(h->nu[0], h->opt.quad_order);
+    double unit = 1.0;                                  // kappa^(t-1)
+    for (int t = 1; t <= h->P; ++t, unit *= k) {
+        p.cu[t] = h->xtpl.cu[0][t] * unit * k;
+        for (int q = 0; data && q < steps; ++q) {
+            p.end[q][t][0] = data[q].bgL[t] * unit;
+            p.end[q][t][1] = data[q].bgR[t] * unit;
+        }
+    }
+    for (int q = 0; data && q < steps; ++q)
+        for (int e = 0; e < 2; ++e) p.bnew[q][e] = data[q].bnew[e];
+    CK(launch_line_f64(h->bc, h->nu[0], h->opt.quad_order, h->ax[0], p, s), "line launch");
+    h->launches++;
+    return MOL_OK;
+}
+
+// the same on the pair levels lev[0] = u^{n-1}, lev[1] = u^n, in place
+mol_status run_line_f32(mol_ctx *h, int rpt, bool cta, const AxisDev &A, int64_t steps, bool first,
+                        const LineEnds *data, cudaStream_t s)
+{
+    F32LineRun p{};
+    p.P = h->P;
+    p.steps = (int)steps;
+    p.first = first;
+    p.data = data != nullptr;
+    for (int t = 1; t <= h->P; ++t) p.cu[t] = (float)h->xtpl.cu[0][t];
+    p.h0 = p.vh0 = (float *)h->lev[0].hi;
+    p.l0 = p.vl0 = (float *)h->lev[0].lo;
+    p.h1 = p.vh1 = (float *)h->lev[1].hi;
+    p.l1 = p.vl1 = (float *)h->lev[1].lo;
+    for (int q = 0; data && q < steps; ++q) {
+        for (int t = 1; t <= h->P; ++t) {
+            p.end[q][t][0] = (float)data[q].bgL[t];
+            p.end[q][t][1] = (float)data[q].bgR[t];
+        }
+        for (int e = 0; e < 2; ++e) {
+            p.bh[q][e] = (float)data[q].bnew[e];
+            p.bl[q][e] = (float)(data[q].bnew[e] - (double)p.bh[q][e]);
+        }
+    }
+    CK(rpt ? launch_line_f32(h->bc, rpt, A, p, s) : launch_line_f32_smem(h->bc, cta, A, p, h->smem_optin, s),
+       "line launch");
+    h->launches++;
+    return MOL_OK;
+}
+
 mol_status check_ptr(mol_ctx *h, const void *p, const char *name)
 {
     if (!p) return fail(h, MOL_EINVAL, std::string(name) + " is NULL");
@@ -1009,7 +1099,24 @@ mol_status mol_step(mol_handle h, double *u_prev, double *u_cur, int64_t nsteps,
     if (u_prev == u_cur) return fail(h, MOL_EINVAL, "u_prev and u_cur must not overlap");
     if (nsteps == 0) return MOL_OK;
     cudaStream_t s = (cudaStream_t)stream;
+    int rpt = 0;
+    bool cta = false;
+    AxisDev A;
+    const bool line = line_loop(h, false, &rpt, &cta, &A);
+    if (line && h->prec == MOL_FP64) {                  // on the caller's levels
+        for (int64_t k = 0; k < nsteps; k += kLineSteps)
+            if ((st = run_line_f64(h, u_prev, u_cur, u_prev, u_cur, std::min(kLineSteps, nsteps - k), false, nullptr,
+                                   s)) != MOL_OK)
+                return st;
+        return MOL_OK;
+    }
     if ((st = load_levels(h, u_prev, h->lev[0], u_cur, h->lev[1], s)) != MOL_OK) return st;
+    if (line) {
+        for (int64_t k = 0; k < nsteps; k += kLineSteps)
+            if ((st = run_line_f32(h, rpt, cta, A, std::min(kLineSteps, nsteps - k), false, nullptr, s)) != MOL_OK)
+                return st;
+        return store_levels(h, h->lev[0], u_prev, h->lev[1], u_cur, s);
+    }
     int64_t done = 0;
     if (h->opt.use_graphs && !h->timing) {
         // whole rotations by graphs of 9 and 3 steps, the rest by a graph of 1 or 2
@@ -1382,10 +1489,9 @@ mol_status mol_solve_dirichlet(mol_handle h, const double *u0, int64_t nsteps, c
     }
     const double a2 = h->alpha * h->alpha;              // the data carries (d_tt / c^2)^m
     const double *cu = h->xtpl.cu[0];
-    int ip = 0, ic = 1, in = 2;
-    if ((st = load_level(h, u0, h->lev[ic], s)) != MOL_OK) return st;
-    for (int64_t k = 0; k < nsteps; ++k) {
-        // boundary values of D^p u at t_k from the data's time derivatives
+    // boundary values of step k: of D^p u at t_k from the data's time
+    // derivatives, then of the D applications of the Horner steps
+    auto step_data = [&](int64_t k, auto &hp) {
         double g[2][MAXP] = {};
         for (int side = 0; side < 2; ++side) {
             const double *dk = data + (k * 2 + side) * Q;
@@ -1398,15 +1504,6 @@ mol_status mol_solve_dirichlet(mol_handle h, const double *u0, int64_t nsteps, c
                 g[side][p] = (p & 1) ? -acc : acc;
             }
         }
-        HornerParams hp = h->xtpl;
-        const bool first = k == 0;
-        hp.ea = 1.0 + (first ? 0.0 : 1.0);
-        hp.eb = first ? 0.0 : -1.0;
-        hp.ec = first ? 0.5 : 1.0;
-        hp.u_hi = h->lev[ic].hi; hp.u_lo = h->lev[ic].lo;
-        hp.up_hi = h->lev[ip].hi; hp.up_lo = h->lev[ip].lo;
-        hp.un_hi = h->lev[in].hi; hp.un_lo = h->lev[in].lo;
-        hp.bcd = 1;
         // the D application of Horner step t returns sum_{p >= t} cu_p D^{p-t+1} u
         for (int t = 1; t <= P; ++t)
             for (int side = 0; side < 2; ++side) {
@@ -1416,6 +1513,38 @@ mol_status mol_solve_dirichlet(mol_handle h, const double *u0, int64_t nsteps, c
             }
         hp.bnew[0] = data[((k + 1) * 2 + 0) * Q];
         hp.bnew[1] = data[((k + 1) * 2 + 1) * Q];
+    };
+    int rpt = 0;
+    bool cta = false;
+    AxisDev A;
+    if (line_loop(h, true, &rpt, &cta, &A)) {
+        const bool f64 = h->prec == MOL_FP64;
+        const int64_t chunk = f64 ? kLineDataSteps : kLineDataStepsF32;
+        LineEnds ends[std::max(kLineDataSteps, kLineDataStepsF32)];
+        if (!f64 && (st = load_level(h, u0, h->lev[1], s)) != MOL_OK) return st;
+        double *l0 = (double *)h->lev[0].hi, *l1 = (double *)h->lev[1].hi;
+        for (int64_t k = 0; k < nsteps; k += chunk) {
+            const int64_t m = std::min(chunk, nsteps - k);
+            for (int64_t q = 0; q < m; ++q) step_data(k + q, ends[q]);
+            st = f64 ? run_line_f64(h, l0, k == 0 ? u0 : l1, l0, k + m == nsteps ? u_out : l1, m, k == 0, ends, s)
+                     : run_line_f32(h, rpt, cta, A, m, k == 0, ends, s);
+            if (st != MOL_OK) return st;
+        }
+        return f64 ? MOL_OK : store_level(h, h->lev[1], u_out, s);
+    }
+    int ip = 0, ic = 1, in = 2;
+    if ((st = load_level(h, u0, h->lev[ic], s)) != MOL_OK) return st;
+    for (int64_t k = 0; k < nsteps; ++k) {
+        HornerParams hp = h->xtpl;
+        const bool first = k == 0;
+        hp.ea = 1.0 + (first ? 0.0 : 1.0);
+        hp.eb = first ? 0.0 : -1.0;
+        hp.ec = first ? 0.5 : 1.0;
+        hp.u_hi = h->lev[ic].hi; hp.u_lo = h->lev[ic].lo;
+        hp.up_hi = h->lev[ip].hi; hp.up_lo = h->lev[ip].lo;
+        hp.un_hi = h->lev[in].hi; hp.un_lo = h->lev[in].lo;
+        hp.bcd = 1;
+        step_data(k, hp);
         if ((st = run_horner(h, 0, hp, s)) != MOL_OK) return st;
         const int t0 = ip; ip = ic; ic = in; in = t0;
     }

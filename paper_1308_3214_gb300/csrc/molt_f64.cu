@@ -25,17 +25,14 @@ F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
     const double om2 = -std::expm1(-2.0 * nu);             // 1 - d^2
     c.kappa = f64_kappa(nu, quad);
     c.rho = quad >= 2 ? -0.5 * quad_R(nu) / c.kappa : 0.0;
-    const int L[2] = {R, c.len_last};
-    double *pw[2] = {&c.dR, &c.dRl}, *W[2] = {&c.W, &c.Wl}, *b[2] = {&c.bR, &c.bl};
-    for (int i = 0; i < 2; ++i) {
-        *pw[i] = std::exp(-nu * (double)L[i]);
-        *W[i] = c.d * -std::expm1(-2.0 * nu * (double)L[i]) / om2;
-        *b[i] = std::exp(-nu * (double)(L[i] + 2)) / om2;
-    }
-    c.a1 = c.d / om2;
+    c.dR = std::exp(-nu * (double)R);
+    c.dRl = std::exp(-nu * (double)c.len_last);
+    f64_inverse_decay(c.d, om2, c.e1, c.id);
     c.mu = A.mu;
     c.inv = A.inv;
-    for (int k = 0; k < kF64MaxR; ++k) c.pw[k] = std::exp(-nu * (double)k);
+    for (int k = 0; k <= R; ++k) c.pw[k] = std::exp(-nu * (double)k);
+    f64_inflow_weights(nu, R, c.w);
+    f64_inflow_weights(nu, c.len_last, c.wl);
     c.dpow = A.dpow64;
     (void)bc;
     return c;
@@ -83,6 +80,21 @@ double f64_kappa(double nu, int quad)
 {
     const double R2 = quad >= 2 ? quad_R(nu) : 0.0;
     return -half_K(nu) - 0.5 * R2 * -std::expm1(-2.0 * nu);
+}
+
+// (1 - d^2) / d and 1 / d carry the boundary terms past a segment's first and
+// last point; where d is so small that the next point sees nothing of them,
+// they drop out (the end points themselves are set)
+void f64_inverse_decay(double d, double om2, double &e1, double &id)
+{
+    id = d > 1e-140 ? 1.0 / d : 0.0;
+    e1 = om2 * id;
+}
+
+void f64_inflow_weights(double nu, int len, double *w)
+{
+    const double om2 = -std::expm1(-2.0 * nu);
+    for (int k = 0; k < len; ++k) w[k] = std::exp(-nu * (double)(k + 1)) * (-std::expm1(-2.0 * nu * (double)(len - k)) / om2);
 }
 
 bool f64_axis_ok(int n, bool contig) { return n <= kF64MaxR * kF64Threads / (contig ? 1 : 2); }

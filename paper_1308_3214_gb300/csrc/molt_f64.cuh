@@ -18,23 +18,24 @@
 //     consumer's Horner weights (host: coefficients times kappa^p).
 //   * each thread owns a segment of R points in registers and solves it once
 //     with zero inflow (causal, then anti-causal in place: 2 operations); what
-//     flows in from the other segments and the line ends adds a d^k +
-//     b d^(len-1-k) (2 operations), both powers being constants of the launch.
-//     The earlier scheme reduced, rescanned and reduced again.
+//     flows in from the other segments and the line ends adds a w_k + b d^(len-k)
+//     (2 operations), w_k = d^(k+1) (1 - d^(2 (len-k))) / (1 - d^2) the response
+//     to an inflow from the left, both factors constants of the launch.  (As
+//     a d^k + b d^(len-1-k) the two terms would cancel at slow decay.)  The
+//     earlier scheme reduced, rescanned and reduced again.
 //
 // Carries: each segment publishes E (its zero-inflow y at its last point) and
 // G (its zero-inflow g at its first point).  After one barrier every segment
 // sums the inflow from as many neighbours as matter (d^(R win) <= 2^-60; the
 // whole line where the decay is slow):
 //   yin = sum_j d^(R (j-1)) E_{m-j},
-//   gin = sum_{l>m} d^(R (l-m-1)) (G_l + W Y_{l-1}),  Y_l = E_l + d^R Y_{l-1},
-//   W = d (1 - d^2R) / (1 - d^2);
-//   a = yin d / (1 - d^2),  b = gin d - yin d^(len+2) / (1 - d^2).
+//   gin = sum_{l>m} d^(R (l-m-1)) (G_l + w_0 Y_{l-1}),  Y_l = E_l + d^R Y_{l-1};
+//   a = yin,  b = gin.
 // Dirichlet (e = 0, or given data, at the ends; s_0 := s_1, s_{n-1} := s_{n-2}):
 // the rows at the ends drop out of s, and A' d^j + B' d^(n-1-j) with
 //   A' + mu B' = r_0 = e_0/kappa - rho s_1 - g_0,
 //   mu A' + B' = r_1 = e_{n-1}/kappa - rho s_{n-2} - g_{n-1}
-// joins a and b in the segments it reaches.  Periodic lines wrap (all images
+// joins a and b in the segments it reaches (d^k = (1 - d^2)/d w_k + d^(2 len - k)).  Periodic lines wrap (all images
 // through 1 / (1 - mu) where the window covers the line).  The last segment
 // may hold fewer than R points.
 //
@@ -67,11 +68,11 @@ struct F64Axis {
     int win;               // segments whose inflow matters on each side
     double d, rho, kappa;
     double dR, dRl;        // d^R, d^len_last
-    double W, Wl;          // d (1 - d^2len) / (1 - d^2), len = R and len_last
-    double a1;             // d / (1 - d^2)
-    double bR, bl;         // d^(len+2) / (1 - d^2)
+    double e1, id;         // (1 - d^2) / d, 1 / d
     double mu, inv;        // as AxisDev
-    double pw[kF64MaxR];   // d^k
+    double pw[kF64MaxR + 1];   // d^k
+    double w[kF64MaxR];    // w_k of a full segment
+    double wl[kF64MaxR];   // w_k of the last one
     const double *dpow;    // d^j, j = 0..n
 };
 
@@ -120,7 +121,7 @@ __device__ __forceinline__ double f64_pick(const double (&z)[R], int k)
     return v;
 }
 
-// Inflow of this segment, a d^k + b d^(len-1-k), and the right sides r_0, r_1
+// Inflow of this segment, a w_k + b d^(len-k), and the right sides r_0, r_1
 // of the boundary terms where this thread has them: on the strided axes every
 // thread within reach of an end sums them for itself (a warp holds one
 // segment, so the others skip it); on the contiguous axis the end segments
@@ -147,7 +148,7 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
         double Y = fma(pl(m), yin, E[c.t]), pr = 1.0;
         l = m + 1 == G ? 0 : m + 1;
         for (int j = 0; j < J; ++j) {
-            gin = fma(pr, fma(l == G - 1 ? A.Wl : A.W, Y, Gs[slot(l)]), gin);
+            gin = fma(pr, fma(l == G - 1 ? A.wl[0] : A.w[0], Y, Gs[slot(l)]), gin);
             Y = fma(pl(l), Y, E[slot(l)]);
             pr *= pl(l);
             l = l + 1 == G ? 0 : l + 1;
@@ -157,7 +158,7 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
         for (int l = max(m - J, 0); l < m; ++l) yin = fma(A.dR, yin, E[slot(l)]);
         double Y = fma(A.dR, yin, E[c.t]), pr = 1.0;
         for (int l = m + 1; l <= min(m + J, G - 1); ++l) {
-            gin = fma(pr, fma(l == G - 1 ? A.Wl : A.W, Y, Gs[slot(l)]), gin);
+            gin = fma(pr, fma(l == G - 1 ? A.wl[0] : A.w[0], Y, Gs[slot(l)]), gin);
             Y = fma(A.dR, Y, E[slot(l)]);
             pr *= A.dR;
         }
@@ -169,7 +170,7 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
             if (all || m < A.win) {
                 double Yl = 0.0, pw = 1.0, g0 = 0.0;
                 for (int l = 0; l < min(J + 1, G); ++l) {
-                    g0 = fma(pw, fma(l == G - 1 ? A.Wl : A.W, Yl, Gs[slot(l)]), g0);
+                    g0 = fma(pw, fma(l == G - 1 ? A.wl[0] : A.w[0], Yl, Gs[slot(l)]), g0);
                     Yl = fma(A.dR, Yl, E[slot(l)]);
                     pw *= A.dR;
                 }
@@ -182,8 +183,8 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
             }
         }
     }
-    a = yin * A.a1;
-    b = fma(gin, A.d, -(yin * (c.last ? A.bl : A.bR)));
+    a = yin;
+    b = gin;
 }
 
 // z: s on entry, rho s + T^{-1} s (with the boundary terms) on exit.  Every
@@ -246,17 +247,21 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
                 r0 = t0;
             }
             const int a0 = c.seg * R;
-            if (all || c.seg < A.win) a = fma(r0, A.dpow[a0], a);
-            if (all || A.G - 1 - c.seg < A.win) b = fma(r1, A.dpow[A.n - a0 - (c.last ? L : R)], b);
+            if (all || c.seg < A.win) {
+                const double t0 = r0 * A.dpow[a0];
+                a = fma(t0, A.e1, a);
+                b = fma(t0, c.last ? A.dRl : A.dR, b);
+            }
+            if (all || A.G - 1 - c.seg < A.win) b = fma(r1 * A.dpow[A.n - a0 - (c.last ? L : R)], A.id, b);
         }
 #pragma unroll
-        for (int k = 0; k < R; ++k) z[k] = fma(a, A.pw[k], fma(A.rho, c.s[k * c.ss], z[k]));
+        for (int k = 0; k < R; ++k) z[k] = fma(A.rho, c.s[k * c.ss], z[k]);
         if (c.tail) {
 #pragma unroll
-            for (int k = 0; k < R; ++k) z[k] = k < L ? fma(b, A.pw[k < L ? L - 1 - k : 0], z[k]) : 0.0;
+            for (int k = 0; k < R; ++k) z[k] = k < L ? fma(b, A.pw[k < L ? L - k : 0], fma(a, A.wl[k], z[k])) : 0.0;
         } else {
 #pragma unroll
-            for (int k = 0; k < R; ++k) z[k] = fma(b, A.pw[R - 1 - k], z[k]);
+            for (int k = 0; k < R; ++k) z[k] = fma(b, A.pw[R - k], fma(a, A.w[k], z[k]));
         }
         if (BC == BC_DIRICHLET) {
             if (c.seg == 0) z[0] = 0.0;

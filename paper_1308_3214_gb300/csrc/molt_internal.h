@@ -113,11 +113,22 @@ struct F64Plan {
 };
 struct F64Prog;
 double f64_kappa(double nu, int quad);
+// w_k = d^(k+1) (1 - d^(2 (len-k))) / (1 - d^2), k < len (molt_f64.cuh)
+void f64_inflow_weights(double nu, int len, double *w);
+void f64_inverse_decay(double d, double om2, double &e1, double &id);
 bool f64_axis_ok(int n, bool contig);
 bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sms, F64Plan *out);
 cudaError_t launch_f64(int bc, bool contig, const F64Plan &pl, double nu, int quad, const AxisDev &ax, int64_t stride,
                        int64_t inner, int64_t nlines, bool horner, F64Prog p, cudaStream_t s);
 cudaError_t configure_f64_kernels();
+// The time loop of a single line as one launch (molt_line.cu).  rpt: segment
+// length of regs_res_plan; A of the smem form as smem_pass_geom fills it.
+struct F64LineRun;
+struct F32LineRun;
+cudaError_t launch_line_f64(int bc, double nu, int quad, const AxisDev &ax, const F64LineRun &p, cudaStream_t s);
+cudaError_t launch_line_f32(int bc, int rpt, const AxisDev &A, const F32LineRun &p, cudaStream_t s);
+bool line_smem_ok(bool cta, const AxisDev &A, size_t smem_max);
+cudaError_t launch_line_f32_smem(int bc, bool cta, const AxisDev &A, const F32LineRun &p, size_t smem_max, cudaStream_t s);
 // 1 if a bounded wait of a register kernel gave up since the last call (and
 // clears it), 0 if not, -1 if the flag could not be read; synchronizes s.
 int regs_timeout_take(cudaStream_t s);
