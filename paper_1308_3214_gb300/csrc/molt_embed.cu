@@ -1,6 +1,6 @@
 // molt_embed.cu -- embedded boundaries (Sec. 4.3): the 2D scheme on a domain
 // cut out of a grid, its lines being "line objects" (the interior grid nodes
-// of a grid line plus a boundary point at each end, off the grid).  Float64.
+// of a grid line plus a boundary point at each end, off the grid).
 //
 // L^{-1} on a line object of m interior nodes: nodes x_0 = a, x_1..x_m (spacing
 // h, x_1 = a + ga), x_{m+1} = b = x_m + gb; the data at a and b are zero.
@@ -10,18 +10,9 @@
 // that node does not exist), integrated exactly; I^L_k = e^{-alpha(x_k -
 // x_{k-1})} I^L_{k-1} + J^L_k from I^L_0 = 0, I^R likewise from the right;
 // w = I^L + I^R + A e^{-alpha (x - a)} + B e^{-alpha (b - x)} with w(a) = w(b)
-// = 0.  Cells between grid nodes take the axis' uniform weights; the cells
-// and stencils that touch a boundary point take per-line weights computed on
-// the host in float64.
-//
-// The kernel: one warp per line object; the line's two partial sums sit in
-// shared memory (the increments overwrite the line's values in place); each
-// lane owns a chunk of consecutive nodes, and both recurrences run as
-// chunked scans of affine maps (a lane's chunk maps the inflow y to P y + Q;
-// a 5-step shuffle scan composes them).
-// A line is read and written in place in the caller's layout: x lines with
-// stride 1, y lines with stride nx (the 4 warps of a CTA take 4 neighbouring
-// columns, which share the 32-byte sectors of each row).
+// = 0.  Both precisions evaluate D = 1 - L^{-1} in a difference form on the
+// line object (the kernels' comments); a line is read and written in place in
+// the caller's layout: x lines with stride 1, y lines with stride nx.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -33,47 +24,54 @@
 namespace {
 
 constexpr int kObjMaxM = 2046;             // interior nodes of a line object at most
-constexpr int kObjWarps = 4;               // line objects (warps) per CTA
 constexpr int kObjThreads32 = 128;         // threads per line object in the float32 sweep
 constexpr int kObjCpb[2] = {1, 4};         // float32 sweep: line objects per CTA, contiguous / strided axis
 
+// Float64 line objects: the difference form of the float32 sweeps (below) with
+// the chain of molt_f64.cuh.  With e = D v and T' = (1 - d^2) T the recurrences
+// read T'_k = q_k + d T'_{k+1} (from b to a) and e_k = d e_{k-1} + T'_k (from a to
+// b), all cells decaying by d: the short end cells enter only as factors, e_1 =
+// lam T'_1 (lam = (1 - dA^2)/(1 - d^2)), and in the boundary terms.  q_k combines
+// second differences as in the float32 sweeps (weights times 1 - d^2).
 struct ObjLine {
     long long base;     // element index of the first interior node
     int m;              // interior nodes
     int pad_;
     double dA, dB;      // e^{-alpha ga}, e^{-alpha gb}
-    double rA, rB;      // dA / d, dB / d (d = e^{-alpha h})
+    double lam;
     double mu, inv;     // e^{-alpha (b - a)}, 1 / (1 - mu^2)
-    double wl[6];       // J^R_0, J^L_1, J^R_1 as weights on (u_1, u_2)
-    double wr[6];       // J^L_{m+1}, J^L_m, J^R_m as weights on (u_m, u_{m-1})
+    double g11, g12;    // q_1 = g11 s_1 + g12 s_2
+    double gNa, gNb;    // q_m = gNa s_{m-1} + gNb s_m
+    double p1, q1;      // s_1 = p1 (v_2 - v_1) - q1 v_1 (v_2 = 0 when m = 1)
+    double pm, qm;      // s_m = pm (0 - v_m) - qm (v_m - v_{m-1})
 };
+
+constexpr int kObjR = 16;                  // points per thread at most
 
 struct ObjAxis {
     long long stride;   // element stride along the lines (1 for x, nx for y)
-    double d;           // e^{-alpha h}
-    double uL[3];       // uniform J^L_k weights on (u_{k-1}, u_k, u_{k+1})
-    double uR[3];       // uniform J^R_k weights on (u_{k-1}, u_k, u_{k+1})
+    int threads, ctas;  // launch shape
+    const int4 *items;  // [ctas][threads]: line (-1: none), segment, slot of the line's segment 0,
+                        // slots to the next segment
+    int win;            // segments whose inflow matters
+    double d, e1, id;   // e^{-alpha h}, (1 - d^2)/d, 1/d
+    double gc, ge;      // uniform rows
     const double *dpow; // d^k, k = 0..kObjMaxM
+    double pw[kObjR + 1];
+    double w[kObjR + 1][kObjR];   // inflow weights of a segment of len points (molt_f64.cuh)
 };
 
-enum : int { OBJ_LINV = 0, OBJ_D = 1, OBJ_SUB = 2 };
+enum : int { OBJ_D = 0, OBJ_LINV = 1, OBJ_BOTH = 2 };
 
-// inclusive scan of affine maps y -> p y + q over the lanes (lane order =
-// application order when FWD, reversed otherwise)
-template <bool FWD>
-__device__ __forceinline__ void affine_scan(double &p, double &q, int lane)
-{
-#pragma unroll
-    for (int k = 1; k < 32; k <<= 1) {
-        const double pp = FWD ? __shfl_up_sync(0xffffffffu, p, k) : __shfl_down_sync(0xffffffffu, p, k);
-        const double qq = FWD ? __shfl_up_sync(0xffffffffu, q, k) : __shfl_down_sync(0xffffffffu, q, k);
-        const bool take = FWD ? lane >= k : lane + k < 32;
-        if (take) {                               // this lane's maps follow the other's
-            q = qq * p + q;
-            p = pp * p;
-        }
-    }
-}
+constexpr int kCombMax = 8;
+// out = sum_t c_t x_t (+ cw times a sweep's result)
+struct CombTerms {
+    int n;
+    double cw;
+    double c[kCombMax];
+    const double *x[kCombMax];
+    double *out;        // nullptr: none
+};
 
 template <bool FWD>
 __device__ __forceinline__ void affine_scan32(float &p, float &q, int lane)
@@ -90,130 +88,198 @@ __device__ __forceinline__ void affine_scan32(float &p, float &q, int lane)
     }
 }
 
-// out[k] (interior node k of every line) = w = L^{-1} in (OBJ_LINV),
-// in - w (OBJ_D) or sub - w (OBJ_SUB); accum adds it to out instead.  slot:
-// shared-memory elements per line array (>= the longest line's m + 2; two
-// arrays per warp).
-__global__ void __launch_bounds__(32 * kObjWarps) k_obj_sweep(ObjAxis ax, const ObjLine *lines, int nlines,
-                                                             const double *__restrict__ in, double *out,
-                                                             const double *sub, int mode, int accum, int slot)
+// OBJ_D: out = D v; OBJ_LINV: out = v - D v (= L^{-1} v); OBJ_BOTH: out = D v, out2 =
+// v - D v (and out3 = D v when given).  accum adds to out.  cb.out: the result is
+// not stored but combined, cb.out = cw result + sum c_t x_t (the level update
+// rides on the last sweep of F).
+//
+// A thread owns R consecutive nodes of a line, counted from the line's far end
+// (index 0 = node m), so that the first chain runs forward.  Which segment of
+// which line is a table made with the handle: whole lines packed into the CTAs
+// whatever their lengths, the segments of a row on neighbouring threads, those
+// of (up to) 4 neighbouring columns interleaved.  The sweep reads its nodes and two halo nodes on each side straight from the
+// field; one barrier carries the segments' E and G, a second the line's two
+// end values (T'_1 is large where the first gap is small: lam multiplies it
+// before it is added to anything).  Bound by float64 latency on grids of a few hundred nodes per
+// line (64 cycles an operation and a warp per SM quarter), by the float64 pipe
+// above: about 11 operations a node instead of 18, spread over a line's worth
+// of threads instead of one warp.  us per step of the ellipse at P = 2, 10 sweeps
+// and a combination before, 9 sweeps now: 129^2 89 -> 76, 400^2 137 -> 96, 777^2
+// 217 -> 141, 2048^2 647 -> 562 (74 % of the float64 pipe).
+template <int R>
+__global__ void __launch_bounds__(512) k_obj_sweep(const __grid_constant__ ObjAxis ax, const ObjLine *__restrict__ lines,
+                                                   const double *__restrict__ in, double *out, double *out2, double *out3,
+                                                   int mode, int accum, const __grid_constant__ CombTerms cb)
 {
-    extern __shared__ __align__(16) double sm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *L = sm + (size_t)warp * 2 * slot;
-    double *R = L + slot;
-    const double d = ax.d;
-    for (int li = blockIdx.x * kObjWarps + warp; li < nlines; li += gridDim.x * kObjWarps) {
-        const ObjLine &ln = lines[li];
-        const int m = ln.m, N = m + 1;
-        const long long base = ln.base;
-        const double dA = ln.dA, dB = ln.dB;
-        __syncwarp();
-        // the line's values into R (zero at the boundary points)
-        const long long st = ax.stride;
-        for (int k = lane; k <= N; k += 32) R[k] = (k >= 1 && k <= m) ? in[base + (k - 1) * st] : 0.0;
-        __syncwarp();
-        // chunk of nodes [k0, k1) of this lane
-        const int s = (N + 1 + 31) / 32;
-        const int k0 = min(lane * s, N + 1), k1 = min(k0 + s, N + 1);
-        // values the increments need from outside the lane's chunk, read before
-        // any lane overwrites R
-        const double u1 = R[1], u2 = R[2], um = R[m], um1 = R[m - 1];
-        double a = (k0 >= 1 && k0 <= N) ? R[k0 - 1] : 0.0;      // u_{k-1}
-        double b = (k0 <= N) ? R[k0] : 0.0;                     // u_k
-        const double after = (k1 <= N) ? R[k1] : 0.0;          // u_{k1}
-        __syncwarp();
-        // increments, in place: L[k] = J^L_k (L[0] = 0), R[k] = J^R_k (R[N] = 0)
-        for (int k = k0; k < k1; ++k) {
-            const double c = (k + 1 < k1) ? R[k + 1] : after;     // u_{k+1}, not yet overwritten
-            double jl = 0.0, jr = 0.0;
-            if (k == 1) jl = ln.wl[2] * u1 + ln.wl[3] * u2;
-            else if (k == N) jl = ln.wr[0] * um + ln.wr[1] * um1;
-            else if (k == m) jl = ln.wr[2] * um + ln.wr[3] * um1;
-            else if (k > 1) jl = ax.uL[0] * a + ax.uL[1] * b + ax.uL[2] * c;
-            if (k == 0) jr = ln.wl[0] * u1 + ln.wl[1] * u2;
-            else if (k == 1) jr = ln.wl[4] * u1 + ln.wl[5] * u2;
-            else if (k == m) jr = ln.wr[4] * um + ln.wr[5] * um1;
-            else if (k < m) jr = ax.uR[0] * a + ax.uR[1] * b + ax.uR[2] * c;
-            L[k] = jl;
-            R[k] = jr;
-            a = b;
-            b = c;
+    extern __shared__ __align__(16) double smo[];
+    const int T = blockDim.x, t = threadIdx.x;
+    double *E = smo, *G = smo + T, *ends = smo + 2 * T;          // [2][T], at the line's slot 0: its
+    const int4 it = ax.items[blockIdx.x * T + t];                // zero-inflow e_m and inflow to T'_1
+    const int seg = it.y, t0 = it.z, st = it.w;
+    const bool on = it.x >= 0;
+    const ObjLine &ln = lines[on ? it.x : 0];
+    const int m = ln.m, a = seg * R;
+    // the tables are constant; the fields are the work of the kernels before
+    molt::pdl_enter();
+    const bool live = on, last = live && a + R >= m;
+    const int len = live ? min(R, m - a) : 0;
+    // node of index j (0 = node m): field element top - j stride
+    const long long top = ln.base + (long long)(m - 1 - a) * ax.stride;
+    double v[R], z[R];
+    if (live) {
+        const double *q = in + top;
+        auto val = [&](int j) -> double { return a + j >= 0 && a + j < m ? q[-(long long)j * ax.stride] : 0.0; };
+        double f[R + 4];                                          // v at j = -2 .. R + 1
+#pragma unroll
+        for (int j = -2; j < R + 2; ++j) f[j + 2] = val(j);
+#pragma unroll
+        for (int j = 0; j < R; ++j) v[j] = f[j + 2];
+        // second differences at j = -1 .. R; the end triples with their spacings
+        // (only the threads that hold them: a predicated operation costs the
+        // float64 pipe as much as an executed one)
+        double sd[R + 2];
+        double dm = f[1] - f[0];
+#pragma unroll
+        for (int j = -1; j <= R; ++j) {
+            const double dp = f[j + 3] - f[j + 2];
+            sd[j + 1] = dp - dm;
+            dm = dp;
         }
-        __syncwarp();
-        // causal: I^L_k = e_k I^L_{k-1} + J^L_k, e_1 = dA, e_N = dB, else d; the
-        // chunk's decay is d^{k1-k0} with the end cells' factors swapped in
-        {
-            double q = 0.0;
-            for (int k = k0; k < k1; ++k) {
-                const double e = (k == 1) ? dA : (k == N ? dB : d);
-                q = e * q + L[k];
+        const int k1 = m - 1 - a;                                 // node 1
+        if (seg == 0) sd[1] = ln.qm * (f[3] - f[2]) - ln.pm * (f[2] - f[1]);      // node m
+        if (k1 <= R) {
+            double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+#pragma unroll
+            for (int j = 0; j <= R; ++j) {
+                c0 = j == k1 ? f[j + 1] : c0;
+                c1 = j == k1 ? f[j + 2] : c1;
+                c2 = j == k1 && j < R ? f[j < R ? j + 3 : 0] : c2;    // (the boundary's zero at j = R)
             }
-            double p = ax.dpow[k1 - k0];
-            if (k0 <= 1 && 1 < k1) p *= ln.rA;
-            if (k0 <= N && N < k1) p *= ln.rB;
-            affine_scan<true>(p, q, lane);
-            double y = __shfl_up_sync(0xffffffffu, q, 1);
-            y = (lane == 0) ? 0.0 : y;
-            for (int k = k0; k < k1; ++k) {
-                const double e = (k == 1) ? dA : (k == N ? dB : d);
-                y = e * y + L[k];
-                L[k] = y;
-            }
+            const double s1 = ln.q1 * (c2 - c1) - ln.p1 * (c1 - c0);
+#pragma unroll
+            for (int j = 0; j <= R; ++j) sd[j + 1] = j == k1 ? s1 : sd[j + 1];
         }
-        // anti-causal: I^R_k = f_k I^R_{k+1} + J^R_k, f_0 = dA, f_m = dB, else d
-        // (the chunk holding N passes no inflow on: every later chunk is empty)
-        {
-            double q = 0.0;
-            for (int k = k1 - 1; k >= k0; --k) {
-                const double f = (k == 0) ? dA : (k == m ? dB : d);
-                const double r = (k == N) ? 0.0 : R[k];
-                q = f * q + r;
+#pragma unroll
+        for (int j = 0; j < R; ++j) z[j] = fma(ax.ge, sd[j] + sd[j + 2], ax.gc * sd[j + 1]);
+        if (seg == 0) z[0] = fma(ln.gNb, sd[1], ln.gNa * sd[2]);
+        if (last) {
+            double s1 = 0.0, s2 = 0.0;
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                s1 = j == k1 ? sd[j + 1] : s1;
+                s2 = j == k1 ? sd[j] : s2;
             }
-            double p = ax.dpow[k1 - k0];
-            if (k0 <= 0 && 0 < k1) p *= ln.rA;
-            if (k0 <= m && m < k1) p *= ln.rB;
-            affine_scan<false>(p, q, lane);
-            double y = __shfl_down_sync(0xffffffffu, q, 1);
-            y = (lane == 31) ? 0.0 : y;
-            for (int k = k1 - 1; k >= k0; --k) {
-                const double f = (k == 0) ? dA : (k == m ? dB : d);
-                const double r = (k == N) ? 0.0 : R[k];
-                y = (k == N) ? 0.0 : f * y + r;
-                R[k] = y;
-            }
+            const double q1 = fma(ln.g11, s1, ln.g12 * s2);
+#pragma unroll
+            for (int j = 0; j < R; ++j) z[j] = j < k1 ? z[j] : (j == k1 ? q1 : 0.0);
         }
-        __syncwarp();
-        // homogeneous terms: w(a) = I^R_0 + A + mu B = 0, w(b) = I^L_N + mu A + B = 0
-        const double r0 = -R[0], r1 = -L[N];
-        const double Acoef = (r0 - ln.mu * r1) * ln.inv;
-        const double Bcoef = (r1 - ln.mu * r0) * ln.inv;
-        for (int k = 1 + lane; k <= m; k += 32) {
-            const double w = L[k] + R[k] + Acoef * dA * ax.dpow[k - 1] + Bcoef * dB * ax.dpow[m - k];
-            double res = w;
-            const long long at = base + (k - 1) * st;
-            if (mode == OBJ_D) res = in[at] - w;
-            else if (mode == OBJ_SUB) res = sub[at] - w;
-            double *o = out + at;
-            *o = accum ? *o + res : res;
+#pragma unroll
+        for (int j = 1; j < R; ++j) z[j] = fma(ax.d, z[j - 1], z[j]);
+        const double e = z[R - 1];
+        if (last) {                                               // T'_1 enters e_1 times lam
+            double e1 = z[0];
+#pragma unroll
+            for (int j = 1; j < R; ++j) e1 = j == len - 1 ? z[j] : e1;
+            e1 *= ln.lam;
+#pragma unroll
+            for (int j = 0; j < R; ++j) z[j] = j < len - 1 ? z[j] : (j == len - 1 ? e1 : 0.0);
+        }
+#pragma unroll
+        for (int j = R - 2; j >= 0; --j) z[j] = fma(ax.d, z[j + 1], z[j]);
+        E[t] = e;
+        G[t] = z[0];
+    }
+    // what the result is added to, and the decays of the boundary terms: on
+    // their way while the carries are
+    const int ns = (m + R - 1) / R;
+    double add[R], d1 = 0.0, da = 0.0, db = 0.0;
+#pragma unroll
+    for (int j = 0; j < R; ++j) add[j] = 0.0;
+    if (live) {
+        d1 = __ldg(ax.dpow + m - 1);
+        da = __ldg(ax.dpow + a);
+        db = __ldg(ax.dpow + m - a - len);
+        if (accum) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                if (j < len) add[j] = out[top - (long long)j * ax.stride];
+        }
+        if (cb.out) {
+            if (accum) {
+#pragma unroll
+                for (int j = 0; j < R; ++j) add[j] *= cb.cw;
+            }
+            for (int k = 0; k < cb.n; ++k) {
+                const double *x = cb.x[k] + top;
+                const double c = cb.c[k];
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    if (j < len) add[j] = fma(c, x[-(long long)j * ax.stride], add[j]);
+            }
         }
     }
+    __syncthreads();
+    double yin = 0.0, gin = 0.0;
+    if (live) {
+        const int J = min(ax.win, ns);
+        const double dR = ax.pw[R], dl = ax.pw[m - (ns - 1) * R], w0 = ax.w[R][0], wl = ax.w[m - (ns - 1) * R][0];
+        for (int l = max(seg - J, 0); l < seg; ++l) yin = fma(dR, yin, E[t0 + l * st]);
+        double Y = fma(dR, yin, E[t]), pr = 1.0;
+        for (int l = seg + 1; l <= min(seg + J, ns - 1); ++l) {
+            gin = fma(pr, fma(l == ns - 1 ? wl : w0, Y, G[t0 + l * st]), gin);
+            Y = fma(dR, Y, E[t0 + l * st]);
+            pr *= dR;
+        }
+        if (seg == 0) ends[t0] = fma(last ? dl : dR, gin, G[t]);
+        if (last) ends[T + t0] = dl * yin;
+    }
+    __syncthreads();
+    if (!live) return;
+    // boundary terms: what the inflow's part of e_1 lacks (lam - 1) and e = 0 at b
+    {
+        const bool all = ax.win + 1 >= ns, nl = all || seg < ax.win, nr = all || ns - 1 - seg <= ax.win;
+        if (nl || nr) {
+            const double y1 = (ln.lam - 1.0) * ends[T + t0];
+            const double em = fma(y1, d1, ends[t0]);
+            const double B = -ln.dB * em * ln.inv;
+            if (nl) {
+                const double ca = B * ln.dB * da;
+                yin = fma(ca, ax.e1, yin);
+                gin = fma(ca, ax.pw[len], gin);
+            }
+            if (nr) gin = fma(fma(-B * ln.mu, ln.dA, y1) * db, ax.id, gin);
+        }
+    }
+    // e, then the result
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        if (j < len) z[j] = fma(gin, ax.pw[len - j], fma(yin, ax.w[len][j], z[j]));
+    double *o = (cb.out ? cb.out : out) + top;
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        if (j < len) {
+            const long long at = -(long long)j * ax.stride;
+            if (mode == OBJ_BOTH) {
+                out2[top + at] = v[j] - z[j];
+                if (out3) out3[top + at] = z[j];
+            }
+            double r = mode == OBJ_LINV ? v[j] - z[j] : z[j];
+            if (cb.out) r = fma(cb.cw, r, add[j]);
+            else if (accum) r += add[j];
+            o[at] = r;
+        }
 }
 
-constexpr int kCombMax = 8;
-struct CombTerms {
-    int n;
-    double c[kCombMax];
-    const double *x[kCombMax];
-};
-
-// out = sum_t c_t x_t (out may be one of the x_t)
-__global__ void __launch_bounds__(256) k_obj_combine(CombTerms t, double *out, int64_t N)
+// out = sum_t c_t x_t at the interior nodes (out may be one of the x_t)
+__global__ void __launch_bounds__(256) k_obj_combine(CombTerms t, const ObjLine *rows, int nrows)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int k = 0; k < t.n; ++k) v += t.c[k] * t.x[k][i];
-        out[i] = v;
+    for (int li = blockIdx.x; li < nrows; li += gridDim.x) {
+        const long long base = rows[li].base;
+        for (int k = threadIdx.x; k < rows[li].m; k += blockDim.x) {
+            double v = 0.0;
+            for (int j = 0; j < t.n; ++j) v += t.c[j] * t.x[j][base + k];
+            t.out[base + k] = v;
+        }
     }
 }
 
@@ -514,51 +580,48 @@ void obj_cell_weights(const double s[3], double len, double alpha, double w[3])
     }
 }
 
-// the per-line constants of a line object of m interior nodes
+// H(l) = Q / (2 alpha^2 (1 - e^{-2 alpha l})), Q = t M_1 - M_2 at t = alpha l: what
+// the quadratic part of the increments of a cell of length l adds to q
+double obj_cell_H(double l, double alpha)
+{
+    const double t = alpha * l;
+    return (t * exp_moment(1, t) - exp_moment(2, t)) / (2.0 * alpha * alpha * -std::expm1(-2.0 * t));
+}
+
+// The float64 constants of a line object.  With D_k the second divided
+// difference at node k and H as above, inserting the increments (Newton form
+// on each cell) into q_k = T_k - g_{k+1} T_{k+1} leaves
+//   q_k = D_k (H_k + H_{k+1} - (x_{k+1} - x_{k-1}) / (2 alpha))
+//         - g_k H_k D_{k-1} - g_{k+1} H_{k+1} D_{k+1},
+// the one-sided interpolants of the end cells putting D_1 for D_0 and D_m for
+// D_{m+1}; no term cancels where a gap is small.  Scaled by 1 - d^2 and by
+// h^2 = s_k / (2 D_k).
 ObjLine make_line(long long base, int m, double h, double ga, double gb, double alpha)
 {
     ObjLine L{};
     L.base = base;
     L.m = m;
-    const double x1 = ga, xm = ga + (double)(m - 1) * h, b = xm + gb;
-    const double x2 = (m >= 2) ? ga + h : b;              // node 2 (b itself when m = 1)
-    const double xm1 = (m >= 2) ? xm - h : 0.0;           // node m - 1 (a itself when m = 1)
+    const double b = ga + (double)(m - 1) * h + gb, c = -std::expm1(-2.0 * alpha * h);
+    const double d = std::exp(-alpha * h), sc = c / (2.0 * h * h);
     L.dA = std::exp(-alpha * ga);
     L.dB = std::exp(-alpha * gb);
-    L.rA = std::exp(-alpha * (ga - h));
-    L.rB = std::exp(-alpha * (gb - h));
+    L.lam = -std::expm1(-2.0 * alpha * ga) / c;
     L.mu = std::exp(-alpha * b);
     L.inv = 1.0 / (-std::expm1(-2.0 * alpha * b));
-    double w[3];
-    {   // J^R_0: destination a, cell [a, x_1], nodes a, x_1, x_2
-        const double s[3] = {0.0, x1, x2};
-        obj_cell_weights(s, x1, alpha, w);
-        L.wl[0] = w[1]; L.wl[1] = w[2];
-    }
-    {   // J^L_1: destination x_1, cell [a, x_1], nodes a, x_1, x_2
-        const double s[3] = {x1, 0.0, x1 - x2};
-        obj_cell_weights(s, x1, alpha, w);
-        L.wl[2] = w[1]; L.wl[3] = w[2];
-    }
-    {   // J^R_1: destination x_1, cell [x_1, x_2], nodes a, x_1, x_2
-        const double s[3] = {-x1, 0.0, x2 - x1};
-        obj_cell_weights(s, x2 - x1, alpha, w);
-        L.wl[4] = w[1]; L.wl[5] = w[2];
-    }
-    {   // J^L_{m+1}: destination b, cell [x_m, b], nodes x_{m-1}, x_m, b
-        const double s[3] = {b - xm1, b - xm, 0.0};
-        obj_cell_weights(s, b - xm, alpha, w);
-        L.wr[0] = w[1]; L.wr[1] = w[0];
-    }
-    {   // J^L_m: destination x_m, cell [x_{m-1}, x_m], nodes x_{m-1}, x_m, b
-        const double s[3] = {xm - xm1, 0.0, xm - b};
-        obj_cell_weights(s, xm - xm1, alpha, w);
-        L.wr[2] = w[1]; L.wr[3] = w[0];
-    }
-    {   // J^R_m: destination x_m, cell [x_m, b], nodes x_{m-1}, x_m, b
-        const double s[3] = {xm1 - xm, 0.0, b - xm};
-        obj_cell_weights(s, b - xm, alpha, w);
-        L.wr[4] = w[1]; L.wr[5] = w[0];
+    const double Ha = obj_cell_H(ga, alpha), Hb = obj_cell_H(gb, alpha), H = obj_cell_H(h, alpha);
+    const double ca = -std::expm1(-alpha * ga), cb = -std::expm1(-alpha * gb);       // 1 - g of the end cells
+    const double nx = m >= 2 ? h : gb, pv = m >= 2 ? h : ga;       // cell after node 1, cell before node m
+    const double h2 = 2.0 * h * h;
+    L.p1 = h2 / ((ga + nx) * nx);
+    L.q1 = h2 / ((ga + nx) * ga);
+    L.pm = h2 / ((pv + gb) * gb);
+    L.qm = h2 / ((pv + gb) * pv);
+    if (m >= 2) {
+        L.g11 = sc * (ca * Ha + H - (ga + h) / (2.0 * alpha));
+        L.gNb = sc * (cb * Hb + H - (gb + h) / (2.0 * alpha));
+        L.g12 = L.gNa = -sc * d * H;
+    } else {
+        L.g11 = L.gNb = sc * (ca * Ha + cb * Hb - (ga + gb) / (2.0 * alpha));
     }
     return L;
 }
@@ -681,10 +744,12 @@ struct mol_embed_ctx {
     int nlines[2] = {0, 0};
     double *dpow[2] = {nullptr, nullptr};
     double *V[kMaxP + 1] = {};          // V[1..P]: the Table 3 auxiliaries
-    double *tmp = nullptr, *t1 = nullptr, *lev = nullptr, *Fb = nullptr;
+    double *tmp = nullptr, *t1 = nullptr, *t2 = nullptr, *t3 = nullptr, *lev = nullptr, *Fb = nullptr;
     double *io[2] = {nullptr, nullptr}; // device copies of mol_embed_solve_host
     std::vector<void *> allocs;
-    int smem = 0, grid = 1, slot = 2;     // sweep launch: shared memory, CTAs, elements per line array
+    int seg = 8;                          // float64 sweeps: points per thread
+    int sms = 152;
+    int slot = 2;                         // float32 sweeps: elements per line array
     int smem32[2] = {0, 0}, grid32[2] = {1, 1};   // float32 sweep launch per axis
     int64_t launches = 0;
     std::string err;
@@ -772,24 +837,96 @@ struct Timed {
 };
 
 // one sweep along axis a (0: the rows, 1: the columns of the field)
-mol_status sweep(mol_embed_ctx *e, int a, const double *in, double *out, int mode, int accum, const double *sub,
-                 cudaStream_t s)
+mol_status sweep(mol_embed_ctx *e, int a, const double *in, double *out, double *out2, int mode, int accum, cudaStream_t s,
+                 double *out3 = nullptr, const CombTerms *cb = nullptr)
 {
     if (e->nlines[a] == 0) return MOL_OK;
-    const int grid = std::min(e->grid, (e->nlines[a] + kObjWarps - 1) / kObjWarps);
+    const CombTerms none{};
+    const ObjAxis &X = e->ax[a];
+    const size_t smem = sizeof(double) * 4 * (size_t)X.threads;
     Timed t(e, a, s);
-    k_obj_sweep<<<grid, 32 * kObjWarps, e->smem, s>>>(e->ax[a], e->lines[a], e->nlines[a], in, out, sub, mode,
-                                                        accum, e->slot);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)X.ctas);
+    cfg.blockDim = dim3((unsigned)X.threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    // a sweep that leaves SMs free lets the next one start while it ends (the
+    // next one's threads fetch their tables and wait): 9 launches a step, each
+    // as short as its latencies on small grids
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = X.ctas <= e->sms && !e->timing ? 1 : 0;
+    ECK(cudaLaunchKernelEx(&cfg, e->seg == 4 ? k_obj_sweep<4> : e->seg == 8 ? k_obj_sweep<8>
+                                 : e->seg == 12 ? k_obj_sweep<12> : k_obj_sweep<16>,
+                           X, (const ObjLine *)e->lines[a], in, out, out2, out3, mode, accum, cb ? *cb : none),
+        "line-object sweep");
     ++e->launches;
     ECK(cudaGetLastError(), "line-object sweep");
     return MOL_OK;
 }
 
-mol_status combine(mol_embed_ctx *e, const CombTerms &t, double *out, cudaStream_t s)
+// The work table of axis a (k_obj_sweep): m = the interior nodes of its lines.
+// Rows one by one, columns in groups of 4 (fewer where a group would not fit a
+// CTA), the longest first, each into the first CTA with room for it.
+mol_status obj_items(mol_embed_ctx *e, int a, const std::vector<int> &m)
 {
-    const int64_t blocks = std::min<int64_t>((e->N + 255) / 256, 4096);
+    ObjAxis &X = e->ax[a];
+    const int R = e->seg, n = (int)m.size();
+    auto segs = [&](int l) { return (m[l] + R - 1) / R; };
+    int gmax = 1;
+    for (int l = 0; l < n; ++l) gmax = std::max(gmax, segs(l));
+    const int T = X.threads = gmax <= 128 ? 128 : gmax <= 256 ? 256 : 512;
+    const double nu = e->alpha * (a == 0 ? e->hx : e->hy);
+    X.win = std::max(1, (int)std::ceil(60.0 * std::log(2.0) / (nu * (double)R)));
+    struct Group { int line, count, len; };              // len: segments of its longest line
+    std::vector<Group> gr;
+    for (int l = 0; l < n;) {
+        int c = a == 0 ? 1 : std::min(4, n - l), g = 1;
+        for (;; c = c > 2 ? 2 : 1) {
+            g = 1;
+            for (int q = 0; q < c; ++q) g = std::max(g, segs(l + q));
+            if (c == 1 || c * g <= T) break;
+        }
+        gr.push_back({l, c, g});
+        l += c;
+    }
+    std::stable_sort(gr.begin(), gr.end(), [](const Group &x, const Group &y) { return x.count * x.len > y.count * y.len; });
+    std::vector<int> used;                               // slots taken, per CTA
+    std::vector<int4> items;
+    size_t open = 0;                                     // CTAs before it have no room for anything more
+    for (const Group &g : gr) {
+        const int need = g.count * g.len;
+        size_t c = open;
+        while (c < used.size() && used[c] + need > T) ++c;
+        if (c == used.size()) {
+            used.push_back(0);
+            items.resize(items.size() + T, int4{-1, 0, 0, 0});
+        }
+        const int base = used[c];
+        for (int k = 0; k < g.len; ++k)
+            for (int q = 0; q < g.count; ++q)
+                if (k * R < m[g.line + q]) items[c * T + base + k * g.count + q] = int4{g.line + q, k, base + q, g.count};
+        used[c] += need;
+        while (open < used.size() && used[open] == T) ++open;
+    }
+    X.ctas = (int)used.size();
+    if (items.empty()) return MOL_OK;
+    int4 *d = nullptr;
+    mol_status st = ealloc(e, (void **)&d, sizeof(int4) * items.size());
+    if (st != MOL_OK) return st;
+    if (cudaMemcpy(d, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        return efail(e, MOL_ECUDA, "work table upload");
+    X.items = d;
+    return MOL_OK;
+}
+
+mol_status combine(mol_embed_ctx *e, const CombTerms &t, cudaStream_t s)
+{
+    if (e->nlines[0] == 0) return MOL_OK;
     Timed tm(e, 2, s);
-    k_obj_combine<<<(unsigned)blocks, 256, 0, s>>>(t, out, e->N);
+    k_obj_combine<<<e->nlines[0], 256, 0, s>>>(t, e->lines[0], e->nlines[0]);
     ++e->launches;
     ECK(cudaGetLastError(), "combine");
     return MOL_OK;
@@ -801,54 +938,71 @@ mol_status combine(mol_embed_ctx *e, const CombTerms &t, double *out, cudaStream
         if (st_ != MOL_OK) return st_;         \
     } while (0)
 
-// out = C v = L_y^{-1} D_x v + L_x^{-1} D_y v   (eq. C_def_ADI)
-mol_status apply_C(mol_embed_ctx *e, const double *v, double *out, cudaStream_t s)
+// out = C v (eq. C_def_ADI) with L^{-1} = 1 - D: L_y^{-1} D_x v + L_x^{-1} D_y v.  dyv:
+// D_y v when an earlier sweep has formed it, else null.  cb: combined instead
+// of stored (out then holds L_y^{-1} D_x v only).
+mol_status apply_C(mol_embed_ctx *e, const double *v, double *out, cudaStream_t s, const double *dyv = nullptr,
+                   const CombTerms *cb = nullptr)
 {
-    EST(sweep(e, 0, v, e->t1, OBJ_D, 0, nullptr, s));          // t1 = D_x v
-    EST(sweep(e, 1, e->t1, out, OBJ_LINV, 0, nullptr, s));     // out = L_y^{-1} t1
-    EST(sweep(e, 1, v, e->t1, OBJ_D, 0, nullptr, s));          // t1 = D_y v
-    return sweep(e, 0, e->t1, out, OBJ_LINV, 1, nullptr, s);   // out += L_x^{-1} t1
+    EST(sweep(e, 0, v, e->t1, nullptr, OBJ_D, 0, s));                   // t1 = D_x v
+    EST(sweep(e, 1, e->t1, out, nullptr, OBJ_LINV, 0, s));              // out = L_y^{-1} t1
+    if (!dyv) {
+        EST(sweep(e, 1, v, e->t1, nullptr, OBJ_D, 0, s));               // t1 = D_y v
+        dyv = e->t1;
+    }
+    return sweep(e, 0, dyv, out, nullptr, OBJ_LINV, 1, s, nullptr, cb);   // out += L_x^{-1} D_y v
 }
 
-// out = D v = v - L_x^{-1} L_y^{-1} v   (eq. D_def_ADI)
-mol_status apply_Dadi(mol_embed_ctx *e, const double *v, double *out, cudaStream_t s)
+// out = D v (eq. D_def_ADI) = v - L_x^{-1} L_y^{-1} v = D_y v + D_x (L_y^{-1} v); dyv
+// receives D_y v as well
+mol_status apply_Dadi(mol_embed_ctx *e, const double *v, double *out, cudaStream_t s, double *dyv)
 {
-    EST(sweep(e, 1, v, e->t1, OBJ_LINV, 0, nullptr, s));       // t1 = L_y^{-1} v
-    return sweep(e, 0, e->t1, out, OBJ_SUB, 0, v, s);          // out = v - L_x^{-1} t1
+    EST(sweep(e, 1, v, out, e->t2, OBJ_BOTH, 0, s, dyv));               // out = D_y v, t2 = L_y^{-1} v
+    return sweep(e, 0, e->t2, out, nullptr, OBJ_D, 1, s);               // out += D_x t2
 }
 
-// lev = ea u + eb up + ec F[u]   (eq. Full_2D, terms in Table 3 order: after
-// stage p, V[k] = C^{p-k+1} D^{k-1} u)
+// out = ea u + eb up + ec F[u] at the interior nodes (eq. Full_2D, terms in
+// Table 3 order: after stage p, V[k] = C^{p-k+1} D^{k-1} u).  The last stage's
+// last C is combined with the other terms by its own last sweep.
 mol_status run_update(mol_embed_ctx *e, const double *u, const double *up, double *out, double ea, double eb,
                       double ec, cudaStream_t s)
 {
     const int P = e->P;
     for (int p = 1; p <= P; ++p) {
-        if (p == 1) {
-            EST(apply_C(e, u, e->V[1], s));
-        } else {
-            EST(apply_Dadi(e, e->V[p - 1], e->V[p], s));
-            for (int k = 1; k < p; ++k) {
-                EST(apply_C(e, e->V[k], e->tmp, s));
-                std::swap(e->V[k], e->tmp);
-            }
-        }
-        // the stage-1 term tw_11 C u is still in tmp after stage 2 (whose only C
-        // swaps V_1 out): with P > 1 it joins stage 2's sum, no pass of its own
-        if (p == 1 && P > 1) continue;
-        CombTerms t{};
         const bool last = p == P;
-        if (p == 2) { t.c[t.n] = (last ? ec : 1.0) * e->tw[1 * 8 + 1]; t.x[t.n++] = e->tmp; }
-        if (p > 2) { t.c[t.n] = last ? ec : 1.0; t.x[t.n++] = e->Fb; }
-        for (int k = 1; k <= p; ++k) {
-            t.c[t.n] = (last ? ec : 1.0) * e->tw[p * 8 + (p - k + 1)];
-            t.x[t.n++] = e->V[k];
+        // terms of F's sum: those of earlier stages, then c_{p,p-k+1} V[k]
+        CombTerms t{};
+        t.out = last ? out : e->Fb;
+        const double f = last ? ec : 1.0;
+        auto add = [&](double c, const double *x) { t.c[t.n] = c; t.x[t.n++] = x; };
+        if (last && ea != 0.0) add(ea, u);
+        if (last && eb != 0.0) add(eb, up);
+        auto weight = [&](int k) { return f * e->tw[p * 8 + (p - k + 1)]; };
+        if (p == 1) {
+            t.cw = weight(1);
+            EST(apply_C(e, u, e->V[1], s, nullptr, last ? &t : nullptr));
+            continue;                                   // C u joins stage 2's sum
         }
-        if (last) {
-            if (ea != 0.0) { t.c[t.n] = ea; t.x[t.n++] = u; }
-            if (eb != 0.0) { t.c[t.n] = eb; t.x[t.n++] = up; }
+        if (p > 2) add(f, e->Fb);
+        // D_y V_{p-1} serves both D V_{p-1} and C V_{p-1}: formed once
+        EST(apply_Dadi(e, e->V[p - 1], e->V[p], s, e->t3));
+        add(weight(p), e->V[p]);
+        for (int k = 1; k < p; ++k) {
+            const bool end = last && k == p - 1;
+            if (k == p - 1) {
+                // V[1] is still C u here when p = 2; the other stages' C are done
+                if (p == 2) add(f * e->tw[1 * 8 + 1], e->V[1]);
+                for (int q = 1; q < k; ++q) add(weight(q), e->V[q]);
+                t.cw = weight(k);
+            }
+            EST(apply_C(e, e->V[k], e->tmp, s, k == p - 1 ? e->t3 : nullptr, end ? &t : nullptr));
+            if (!end) std::swap(e->V[k], e->tmp);
         }
-        EST(combine(e, t, last ? out : e->Fb, s));
+        if (last) continue;
+        // not the last stage: its own sum (V[1], its C u now in tmp, when p = 2)
+        if (p == 2) t.x[1] = e->tmp;
+        add(t.cw, e->V[p - 1]);
+        EST(combine(e, t, s));
     }
     return MOL_OK;
 }
@@ -1045,17 +1199,20 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
         for (int m = 1; m <= p; ++m) e->tw[p * 8 + m] = term_weight(p, m, beta);
     mol_status st = MOL_OK;
     cudaError_t ce;
+    std::vector<int> msz[2];                             // interior nodes of the lines
     for (int a = 0; a < 2 && st == MOL_OK; ++a) {
         const double h = a == 0 ? e->hx : e->hy, alpha = e->alpha;
         ObjAxis &X = e->ax[a];
         X.stride = a == 0 ? 1 : nx;
         X.d = std::exp(-alpha * h);
-        double w[3];
-        const double sL[3] = {h, 0.0, -h}, sR[3] = {-h, 0.0, h};
-        obj_cell_weights(sL, h, alpha, w);
-        for (int i = 0; i < 3; ++i) X.uL[i] = w[i];
-        obj_cell_weights(sR, h, alpha, w);
-        for (int i = 0; i < 3; ++i) X.uR[i] = w[i];
+        {
+            const double c = -std::expm1(-2.0 * alpha * h), sc = c / (2.0 * h * h), H = obj_cell_H(h, alpha);
+            X.gc = sc * (2.0 * H - h / alpha);
+            X.ge = -sc * X.d * H;
+            f64_inverse_decay(X.d, c, X.e1, X.id);
+            for (int k = 0; k <= kObjR; ++k) X.pw[k] = std::exp(-alpha * h * (double)k);
+            for (int k = 1; k <= kObjR; ++k) f64_inflow_weights(alpha * h, k, X.w[k]);
+        }
         std::vector<double> tab(kObjMaxM + 1);
         for (int k = 0; k <= kObjMaxM; ++k) tab[k] = std::exp(-alpha * h * (double)k);
         std::vector<ObjLine> ls;
@@ -1066,6 +1223,7 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
             if (lo[l] > hi[l]) continue;
             const long long base = a == 0 ? l * nx + lo[l] : lo[l] * nx + l;   // first interior node
             ls.push_back(make_line(base, (int)(hi[l] - lo[l] + 1), h, ga[l], gb[l], alpha));
+            msz[a].push_back(ls.back().m);
         }
         e->nlines[a] = (int)ls.size();
         if ((st = ealloc(e, (void **)&e->dpow[a], sizeof(double) * tab.size())) != MOL_OK) break;
@@ -1117,7 +1275,7 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
     std::vector<std::pair<void **, size_t>> work;
     const size_t plane = sizeof(double) * (size_t)e->N, plane32 = sizeof(float) * (size_t)e->N;
     if (prec == MOL_FP64) {
-        for (double **b : {&e->tmp, &e->t1, &e->lev, &e->Fb}) work.push_back({(void **)b, plane});
+        for (double **b : {&e->tmp, &e->t1, &e->t2, &e->t3, &e->lev, &e->Fb}) work.push_back({(void **)b, plane});
         for (int k = 1; k <= P; ++k) work.push_back({(void **)&e->V[k], plane});
     } else {
         for (float **b : {&e->tmp32, &e->t132, &e->t232, &e->t332, &e->Fb32}) work.push_back({(void **)b, plane32});
@@ -1135,20 +1293,26 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
     if (st == MOL_OK) {
         // line arrays sized for the longest line (even, for 16-byte alignment)
         e->slot = (int)((maxm + 2 + 1) & ~(int64_t)1);
-        // float64: two line arrays of doubles per warp; float32: four arrays of
-        // floats per line
-        int dev = 0, sms = 152, per_sm = 1;
+        // (float32: four arrays per line)
+        int dev = 0, sms = 152;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        e->sms = sms;
         if (prec == MOL_FP64) {
-            e->smem = (int)(sizeof(double) * 2 * (size_t)e->slot * kObjWarps);
-            if ((ce = cudaFuncSetAttribute(k_obj_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, e->smem)) !=
-                cudaSuccess)
-                st = efail(e, MOL_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(ce));
-            if (st == MOL_OK && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_obj_sweep, 32 * kObjWarps,
-                                                                              e->smem) != cudaSuccess) {
-                cudaGetLastError();
-                per_sm = 1;
+            // points per thread: about 12 operations each and 48 of inflow and
+            // line ends per thread, whole warps over the SMs' quarters
+            int64_t nodes = 0;
+            for (int v : msz[0]) nodes += v;
+            double best = 0.0;
+            for (int R : {4, 8, 12, 16}) {
+                if (maxm > (int64_t)R * 512) continue;
+                const double w = 1.08 * (double)nodes / (32.0 * R) / (4.0 * sms);
+                const double cost = (12.0 * R + 48.0) * (w <= 8.0 ? std::ceil(w) : w + 0.5);
+                if (best == 0.0 || cost < best) {
+                    best = cost;
+                    e->seg = R;
+                }
             }
+            for (int a = 0; a < 2 && st == MOL_OK; ++a) st = obj_items(e, a, msz[a]);
         } else {
             const void *kf[2][2] = {{(const void *)k_obj_sweep32<true, 1>, (const void *)k_obj_sweep32<false, 1>},
                                     {(const void *)k_obj_sweep32<true, kObjCpb[1]>,
@@ -1169,7 +1333,6 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
                 e->grid32[a] = std::max(1, sms) * std::max(1, ps);
             }
         }
-        e->grid = std::max(1, sms) * std::max(1, per_sm);
     }
     if (st != MOL_OK) {
         set_global_error(e->err);
@@ -1208,7 +1371,7 @@ mol_status mol_embed_linv(mol_embed e, const double *v, double *w, int axis, voi
         return MOL_OK;
     }
     ECK(cudaMemsetAsync(w, 0, sizeof(double) * (size_t)e->N, s), "memset");
-    return sweep(e, axis, v, w, OBJ_LINV, 0, nullptr, s);
+    return sweep(e, axis, v, w, nullptr, OBJ_LINV, 0, s);
 }
 
 mol_status mol_embed_apply_F(mol_embed e, const double *u, double *F, void *stream)
@@ -1225,6 +1388,7 @@ mol_status mol_embed_apply_F(mol_embed e, const double *u, double *F, void *stre
         ++e->launches;
         return MOL_OK;
     }
+    ECK(cudaMemsetAsync(F, 0, sizeof(double) * (size_t)e->N, s), "memset");      // (the update writes the interior)
     return run_update(e, u, nullptr, F, 0.0, 0.0, 1.0, s);
 }
 
@@ -1240,6 +1404,7 @@ mol_status mol_embed_start(mol_embed e, const double *u0, double *u1, void *stre
         EST(run_update32(e, e->lh[0], e->ll[0], nullptr, nullptr, e->lh[1], e->ll[1], nullptr, 1.f, 0.f, 0.5f, s));
         return from_pair(e, 1, u1, s);
     }
+    ECK(cudaMemsetAsync(u1, 0, sizeof(double) * (size_t)e->N, s), "memset");
     return run_update(e, u0, nullptr, u1, 1.0, 0.0, 0.5, s);
 }
 
