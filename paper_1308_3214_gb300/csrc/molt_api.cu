@@ -55,7 +55,7 @@ struct mol_ctx {
     int num_sms = 152;
     size_t smem_optin = 227 * 1024;
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t gexec[4] = {nullptr, nullptr, nullptr, nullptr};   // graphs of kGraphSteps[k] steps
+    cudaGraphExec_t gexec[5] = {};       // graphs of kGraphSteps[k] steps
     int64_t launches = 0;
     // launch choices (mol_autotune): warps per CTA of the resident x pass,
     // strided segment length (0 = default) and segments per CTA at most
@@ -100,7 +100,8 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
-constexpr int kGraphSteps[4] = {1, 2, 3, 9};
+constexpr int kGraphs = 5;
+constexpr int kGraphSteps[kGraphs] = {1, 2, 4, 8, 16};
 
 void drop_graphs(mol_ctx *h)
 {
@@ -705,11 +706,21 @@ mol_status store_levels(mol_ctx *h, const Level &L0, double *x0, const Level &L1
 
 int passes_per_step(const mol_ctx *h) { return h->ndim; }
 
-// Capture three steps (one full rotation of the three level buffers) as a graph.
-// Graph k holds kGraphSteps[k] time steps from the first level buffer
-// rotation (lev[0] = u^{n-1}, lev[1] = u^n); 3 and 9 steps return to it, 1 and
-// 2 end a call's run.  Captured lazily, dropped whenever a launch choice
-// changes.
+// One time step of the loop, in place: u^{n+1} is written over u^{n-1} (every
+// x pass reads a point's u^{n-1} and writes its u^{n+1} in the same thread), so
+// that two levels and the intermediate planes are all a step touches.  On
+// 2048^2, P = 3 that is 117 MB, which stays in the 129 MB of L2; three rotating
+// levels made it 151 MB.  k: steps done since the levels were lev[0] = u^{n-1},
+// lev[1] = u^n.
+mol_status run_step(mol_ctx *h, int64_t k, cudaStream_t s)
+{
+    const Level &prev = h->lev[k % 2], &cur = h->lev[(k + 1) % 2];
+    return run_update(h, cur, prev, prev, 2.0, -1.0, 1.0, s);
+}
+
+// Graph k holds kGraphSteps[k] time steps from lev[0] = u^{n-1}, lev[1] = u^n; even
+// counts return to that order, a single step ends a call's run.  Captured
+// lazily, dropped whenever a launch choice changes.
 mol_status build_graph(mol_ctx *h, int k)
 {
     if (h->gexec[k]) return MOL_OK;
@@ -719,7 +730,7 @@ mol_status build_graph(mol_ctx *h, int k)
     const int64_t before = h->launches;
     mol_status st = MOL_OK;
     for (int j = 0; j < kGraphSteps[k] && st == MOL_OK; ++j)
-        st = run_update(h, h->lev[(j + 1) % 3], h->lev[j % 3], h->lev[(j + 2) % 3], 2.0, -1.0, 1.0, h->cap_stream);
+        st = run_step(h, j, h->cap_stream);
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
     h->launches = before;
     if (st != MOL_OK) { if (g) cudaGraphDestroy(g); return st; }
@@ -949,7 +960,7 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
                 h->dmr_ax[a][r][k] = std::exp(-h->nu[a] * (double)(8 << r) * (double)(1 << k));
     }
     build_tables(h);
-    // levels: three rotating buffers
+    // levels: two for the time loop, a third for the operators and the other loops
     for (int k = 0; k < 3; ++k) {
         if (prec == MOL_MIXED) {
             if ((st = dev_alloc(h, &h->lev[k].hi, sizeof(float) * h->N)) != MOL_OK) goto bad;
@@ -1119,23 +1130,20 @@ mol_status mol_step(mol_handle h, double *u_prev, double *u_cur, int64_t nsteps,
     }
     int64_t done = 0;
     if (h->opt.use_graphs && !h->timing) {
-        // whole rotations by graphs of 9 and 3 steps, the rest by a graph of 1 or 2
+        // the largest graph that fits, again and again
         while (done < nsteps) {
-            const int64_t left = nsteps - done;
-            const int k = left >= 9 ? 3 : (left >= 3 ? 2 : (int)left - 1);
+            int k = kGraphs - 1;
+            while (kGraphSteps[k] > nsteps - done) --k;
             if ((st = build_graph(h, k)) != MOL_OK) return st;
             CK(cudaGraphLaunch(h->gexec[k], s), "graph launch");
             h->launches += kGraphSteps[k] * passes_per_step(h);
             done += kGraphSteps[k];
         }
     }
-    for (; done < nsteps; ++done) {
-        const int k = (int)(done % 3);
-        if ((st = run_update(h, h->lev[(k + 1) % 3], h->lev[k], h->lev[(k + 2) % 3], 2.0, -1.0, 1.0, s)) != MOL_OK)
-            return st;
-    }
-    const int k = (int)(nsteps % 3);
-    return store_levels(h, h->lev[k], u_prev, h->lev[(k + 1) % 3], u_cur, s);
+    for (; done < nsteps; ++done)
+        if ((st = run_step(h, done, s)) != MOL_OK) return st;
+    const int k = (int)(nsteps % 2);
+    return store_levels(h, h->lev[k], u_prev, h->lev[1 - k], u_cur, s);
 }
 
 mol_status mol_solve_host(mol_handle h, const double *u0, double *u_out, int64_t nsteps, void *stream)
@@ -1251,7 +1259,7 @@ mol_status mol_autotune(mol_handle h, void *stream)
             for (int rep = 0; rep < 4 && st == MOL_OK; ++rep) {
                 if (rep > 0 && cudaEventRecord(e0, s) != cudaSuccess) { st = fail(h, MOL_ECUDA, "event record"); break; }
                 for (int k = 0; k < (rep == 0 ? 2 : 3) && st == MOL_OK; ++k)
-                    st = run_update(h, h->lev[(k + 1) % 3], h->lev[k % 3], h->lev[(k + 2) % 3], 2.0, -1.0, 1.0, s);
+                    st = run_step(h, k, s);
                 if (st != MOL_OK) break;
                 if (rep > 0) {
                     float ms = 0.f;
