@@ -122,6 +122,52 @@ struct HornerParams {
     double bnew[2];
 };
 
+// The same in the kernel's precision (the shared-memory passes): a float32 pass
+// that converts or compares the float64 weights at every point runs at the
+// rate of the float64 pipe (64 cycles a warp and operation).  With these, and
+// four points' loads in flight per thread, the Horner pass on float32 rows of
+// 1000 x 1200, P = 3, takes 70 us instead of 148; the y pass of 96 x 160 x 251,
+// P = 2, 274 instead of 404.
+template <class T> struct HornerArgs {
+    int P, ng, nout, epi;
+    const void *g[MAXG];
+    void *out[MAXG];
+    T coef[MAXP][MAXP][MAXG], cu[MAXP][MAXP];
+    unsigned add[MAXP][MAXP];        // [o][step]: bit k set where g_k has a weight
+    T ea, eb, ec;
+    bool prev;                       // eb != 0
+    const void *u_hi, *u_lo, *up_hi, *up_lo;
+    void *un_hi, *un_lo;
+    int bcd;
+    T bgL[MAXP], bgR[MAXP];
+    T bh[2], bl[2];                  // the new level's end values (float32: as pairs)
+};
+
+template <class T> inline HornerArgs<T> horner_args(const HornerParams &p)
+{
+    HornerArgs<T> a{};
+    a.P = p.P; a.ng = p.ng; a.nout = p.nout; a.epi = p.epi;
+    for (int k = 0; k < MAXG; ++k) { a.g[k] = p.g[k]; a.out[k] = p.out[k]; }
+    for (int o = 0; o < MAXP; ++o)
+        for (int t = 0; t < MAXP; ++t) {
+            for (int k = 0; k < MAXG; ++k) {
+                a.coef[o][t][k] = (T)p.coef[o][t][k];
+                if (k < p.ng && p.coef[o][t][k] != 0.0) a.add[o][t] |= 1u << k;
+            }
+            a.cu[o][t] = (T)p.cu[o][t];
+        }
+    a.ea = (T)p.ea; a.eb = (T)p.eb; a.ec = (T)p.ec;
+    a.prev = p.eb != 0.0;
+    a.u_hi = p.u_hi; a.u_lo = p.u_lo; a.up_hi = p.up_hi; a.up_lo = p.up_lo; a.un_hi = p.un_hi; a.un_lo = p.un_lo;
+    a.bcd = p.bcd;
+    for (int t = 0; t < MAXP; ++t) { a.bgL[t] = (T)p.bgL[t]; a.bgR[t] = (T)p.bgR[t]; }
+    for (int e = 0; e < 2; ++e) {
+        a.bh[e] = (T)p.bnew[e];
+        a.bl[e] = (T)(p.bnew[e] - (double)a.bh[e]);
+    }
+    return a;
+}
+
 // Coefficients and fields of a pass program.
 //   mode 0 (powers): out[p-1] = D^p u, p = 1..P
 //   mode 1 (Horner): for each output o:
@@ -811,6 +857,37 @@ __device__ __forceinline__ void for_block(const PassGeom &G, int n, int nl, F &&
     }
 }
 
+// The same walk, four (line, point) pairs at a time, so that a thread has
+// four points' loads in flight: f(l, j, c) for pairs 0..c-1.
+template <bool CONTIG, class F>
+__device__ __forceinline__ void for_block4(const PassGeom &G, int n, int nl, F &&f)
+{
+    const int tid = threadIdx.x, nth = blockDim.x;
+    int l[4], j[4];
+    if (CONTIG) {
+        for (int q = 0; q < nl; ++q)
+            for (int j0 = tid; j0 < n; j0 += 4 * nth) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    l[i] = q;
+                    j[i] = j0 + i * nth;
+                }
+                f(l, j, min(4, (n - j0 + nth - 1) / nth));
+            }
+    } else {
+        const int W = G.W, q = tid & (W - 1), rstep = nth >> G.wshift;
+        if (q < nl)
+            for (int j0 = tid >> G.wshift; j0 < n; j0 += 4 * rstep) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    l[i] = q;
+                    j[i] = j0 + i * rstep;
+                }
+                f(l, j, min(4, (n - j0 + rstep - 1) / rstep));
+            }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Powers pass: out[p-1] = D^p u along the axis, p = 1..P.
 // ---------------------------------------------------------------------------
@@ -872,35 +949,47 @@ __global__ void __launch_bounds__(512) k_powers(AxisDev A, PassGeom G, PowersPar
 // ---------------------------------------------------------------------------
 template <class T> struct LevelIO;
 template <> struct LevelIO<float> {
-    __device__ static void combine(const HornerParams &p, int64_t i, float F)
+    using Args = HornerArgs<float>;
+    float uh, ul, ph, pl;
+    __device__ void load(const Args &p, int64_t i)
     {
-        const float *uh = (const float *)p.u_hi, *ul = (const float *)p.u_lo;
-        float ph = 0.f, pl = 0.f;
-        if (p.eb != 0.0) { ph = ((const float *)p.up_hi)[i]; pl = ((const float *)p.up_lo)[i]; }
+        uh = ((const float *)p.u_hi)[i];
+        ul = ((const float *)p.u_lo)[i];
+        ph = p.prev ? ((const float *)p.up_hi)[i] : 0.f;
+        pl = p.prev ? ((const float *)p.up_lo)[i] : 0.f;
+    }
+    __device__ void combine(const Args &p, int64_t i, float F) const
+    {
         float nh, nl;
-        level_pair(uh[i], ul[i], ph, pl, F, (float)p.ea, (float)p.eb, (float)p.ec, nh, nl);
+        level_pair(uh, ul, ph, pl, F, p.ea, p.eb, p.ec, nh, nl);
         ((float *)p.un_hi)[i] = nh;
         ((float *)p.un_lo)[i] = nl;
     }
-    __device__ static void set(const HornerParams &p, int64_t i, double v)
+    __device__ static void set(const Args &p, int64_t i, int e)
     {
-        const float h = __double2float_rn(v);
-        ((float *)p.un_hi)[i] = h;
-        ((float *)p.un_lo)[i] = __double2float_rn(v - (double)h);
+        ((float *)p.un_hi)[i] = p.bh[e];
+        ((float *)p.un_lo)[i] = p.bl[e];
     }
 };
 template <> struct LevelIO<double> {
-    __device__ static void combine(const HornerParams &p, int64_t i, double F)
+    using Args = HornerArgs<double>;
+    double u, q;
+    __device__ void load(const Args &p, int64_t i)
     {
-        double v = p.ea * ((const double *)p.u_hi)[i] + p.ec * F;
-        if (p.eb != 0.0) v += p.eb * ((const double *)p.up_hi)[i];
+        u = ((const double *)p.u_hi)[i];
+        q = p.prev ? ((const double *)p.up_hi)[i] : 0.0;
+    }
+    __device__ void combine(const Args &p, int64_t i, double F) const
+    {
+        double v = p.ea * u + p.ec * F;
+        if (p.prev) v += p.eb * q;
         ((double *)p.un_hi)[i] = v;
     }
-    __device__ static void set(const HornerParams &p, int64_t i, double v) { ((double *)p.un_hi)[i] = v; }
+    __device__ static void set(const Args &p, int64_t i, int e) { ((double *)p.un_hi)[i] = p.bh[e]; }
 };
 
 template <class T, int BC, bool CONTIG>
-__global__ void __launch_bounds__(512) k_horner(AxisDev A, PassGeom G, HornerParams prm)
+__global__ void __launch_bounds__(512) k_horner(AxisDev A, PassGeom G, const __grid_constant__ HornerArgs<T> prm)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = A.n, W = G.W;
@@ -933,32 +1022,50 @@ __global__ void __launch_bounds__(512) k_horner(AxisDev A, PassGeom G, HornerPar
         for (int t = prm.P; t >= 0; --t) {
             // buf = (t == P ? 0 : buf) + sum_k coef g_k
             const bool first = (t == prm.P);
-            for_block<CONTIG>(G, n, nl, [&](int l, int j) {
-                const int64_t gi = lbase[l] + (int64_t)j * G.stride;
-                const size_t si = (size_t)l * A.ls + spos_raw(j, A.m, A.ms, A.mmagic);
-                T acc = first ? (T)0 : lines[si];
-                for (int k = 0; k < prm.ng; ++k) {
-                    const double w = prm.coef[o][t][k];
-                    if (w != 0.0) acc += (T)w * reinterpret_cast<const T *>(prm.g[k])[gi];
+            const unsigned add = prm.add[o][t];
+            for_block4<CONTIG>(G, n, nl, [&](const int (&l)[4], const int (&j)[4], int c) {
+                int64_t gi[4];
+                size_t si[4];
+                T acc[4];
+                LevelIO<T> lev[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    gi[i] = lbase[l[i]] + (int64_t)j[i] * G.stride;
+                    si[i] = (size_t)l[i] * A.ls + spos_raw(j[i], A.m, A.ms, A.mmagic);
+                    acc[i] = first || i >= c ? (T)0 : lines[si[i]];
+                    if (t == 0 && prm.epi && i < c) lev[i].load(prm, gi[i]);
                 }
-                if (t > 0) {
-                    lines[si] = acc;
-                } else if (prm.epi == 0) {
-                    reinterpret_cast<T *>(prm.out[o])[gi] = acc;
-                } else if (BC == BC_DIRICHLET && prm.bcd && (j == 0 || j == n - 1)) {
-                    LevelIO<T>::set(prm, gi, prm.bnew[j == 0 ? 0 : 1]);    // the data at the end nodes
-                } else {
-                    LevelIO<T>::combine(prm, gi, acc);
+                for (int k = 0; k < prm.ng; ++k)
+                    if (add >> k & 1u) {
+                        const T w = prm.coef[o][t][k];
+                        const T *g = reinterpret_cast<const T *>(prm.g[k]);
+                        T v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i] = i < c ? g[gi[i]] : (T)0;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[i] += w * v[i];
+                    }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= c) break;
+                    if (t > 0) {
+                        lines[si[i]] = acc[i];
+                    } else if (prm.epi == 0) {
+                        reinterpret_cast<T *>(prm.out[o])[gi[i]] = acc[i];
+                    } else if (BC == BC_DIRICHLET && prm.bcd && (j[i] == 0 || j[i] == n - 1)) {
+                        LevelIO<T>::set(prm, gi[i], j[i] == 0 ? 0 : 1);    // the data at the end nodes
+                    } else {
+                        lev[i].combine(prm, gi[i], acc[i]);
+                    }
                 }
             });
             __syncthreads();
+            const T gL = prm.bcd ? prm.bgL[t] : (T)0, gR = prm.bcd ? prm.bgR[t] : (T)0;
             if (t > 0 && G.cta)
-                sweep_D_cta<T, 2, BC>(lines, rlines, (T)prm.cu[o][t], A, dp,
-                                      reinterpret_cast<T *>(smem_raw + SL.scratch), prm.bcd ? (T)prm.bgL[t] : (T)0,
-                                      prm.bcd ? (T)prm.bgR[t] : (T)0);
+                sweep_D_cta<T, 2, BC>(lines, rlines, prm.cu[o][t], A, dp, reinterpret_cast<T *>(smem_raw + SL.scratch),
+                                      gL, gR);
             else if (t > 0 && warp < nl)
-                sweep_D<T, 2, BC>(mine, rmine, (T)prm.cu[o][t], A, dp, lane, prm.bcd ? (T)prm.bgL[t] : (T)0,
-                                  prm.bcd ? (T)prm.bgR[t] : (T)0);
+                sweep_D<T, 2, BC>(mine, rmine, prm.cu[o][t], A, dp, lane, gL, gR);
             __syncthreads();
         }
     }

@@ -211,7 +211,7 @@ static cudaError_t run_horner(const AxisDev &A, const PassGeom &G, const HornerP
 {
     const size_t smem = pass_smem_bytes(true, sizeof(T), G.W, A.ls, A.n, G.dps);
     const int64_t grid = (G.nlines + G.W - 1) / G.W;
-    k_horner<T, BC, CONTIG><<<(unsigned)grid, pass_threads<CONTIG>(G), smem, s>>>(A, G, p);
+    k_horner<T, BC, CONTIG><<<(unsigned)grid, pass_threads<CONTIG>(G), smem, s>>>(A, G, horner_args<T>(p));
     return cudaGetLastError();
 }
 
