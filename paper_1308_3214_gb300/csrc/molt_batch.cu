@@ -43,7 +43,7 @@ struct mol_batch_ctx {
     int nrec = 0, irec_cap = 0;          //   nodes, the node groups' starts and the receivers by node
     int nnode = 0;
     void *inter[BMAXP] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    int xW[2] = {8, 8}, xgrid[2] = {1, 1}, nbuf = 1, cgrid = 1;
+    int xW[2] = {8, 8}, xgrid[2] = {1, 1}, nbuf = 1, cgrid = 1, cgrid_y = 1;
     int ycls_begin[4] = {0, 0, 0, 0};   // y work list: the items of clusters of 1, 2, 4, 8 CTAs
     int ycls_count[4] = {0, 0, 0, 0};
     size_t xsmem[2] = {0, 0}, ysmem = 0;
@@ -498,10 +498,10 @@ mol_status run_update(mol_batch_ctx *b, const BLevel &u, const BLevel &up, const
 mol_status pack(mol_batch_ctx *b, const double *x, const BLevel &L, cudaStream_t s)
 {
     if (b->tbytes == 4)
-        k_batch_pack<float><<<b->cgrid, 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows, x,
+        k_batch_pack<float><<<dim3(b->cgrid, b->cgrid_y), 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows, x,
                                                      (float *)L.hi, (float *)L.lo);
     else
-        k_batch_pack<double><<<b->cgrid, 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows, x,
+        k_batch_pack<double><<<dim3(b->cgrid, b->cgrid_y), 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows, x,
                                                       (double *)L.hi, nullptr);
     BCK(cudaGetLastError(), "batched level conversion");
     b->launches++;
@@ -511,10 +511,10 @@ mol_status pack(mol_batch_ctx *b, const double *x, const BLevel &L, cudaStream_t
 mol_status unpack(mol_batch_ctx *b, const BLevel &L, double *x, cudaStream_t s, const double *add = nullptr)
 {
     if (b->tbytes == 4)
-        k_batch_unpack<float><<<b->cgrid, 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows,
+        k_batch_unpack<float><<<dim3(b->cgrid, b->cgrid_y), 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows,
                                                        (const float *)L.hi, (const float *)L.lo, x, add);
     else
-        k_batch_unpack<double><<<b->cgrid, 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows,
+        k_batch_unpack<double><<<dim3(b->cgrid, b->cgrid_y), 256, 0, s>>>(b->probs, b->row_prob, b->uoff_dev, (int)b->nrows,
                                                         (const double *)L.hi, nullptr, x, add);
     BCK(cudaGetLastError(), "batched level conversion");
     b->launches++;
@@ -885,6 +885,8 @@ mol_status mol_batch_create(int nprob, const mol_grid *grids, const double *c, c
         }
         b->ysmem = batch_y_smem((size_t)b->tbytes);
         b->cgrid = (int)std::min<int64_t>((b->nrows + 7) / 8, 8 * (int64_t)b->num_sms);
+        // (rows of up to 1024 points: 8 chunks of 128 each)
+        b->cgrid_y = (int)std::max<int64_t>(1, std::min<int64_t>(8, 8 * (int64_t)b->num_sms / b->cgrid));
         e = b->tbytes == 4 ? set_kernel_smem<float>(b) : set_kernel_smem<double>(b);
         if (e != cudaSuccess) { st = bcuda(b, e, "kernel attributes"); goto bad; }
     }

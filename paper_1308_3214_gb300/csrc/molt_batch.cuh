@@ -1030,7 +1030,7 @@ __global__ void __launch_bounds__(256, 8) k_batch_pack(const BatchProb *probs, c
         const double *src = x + __ldg(uoff + p) + (int64_t)row * nx;
         const int64_t dst = __ldg(&pb->off) + (int64_t)row * pitch;
 #pragma unroll 2
-        for (int j0 = lane; j0 < pitch; j0 += 128) {
+        for (int j0 = lane + 128 * (int)blockIdx.y; j0 < pitch; j0 += 128 * (int)gridDim.y) {
             double v[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) v[c] = (j0 + 32 * c < nx) ? __ldg(src + j0 + 32 * c) : 0.0;
@@ -1069,7 +1069,7 @@ __global__ void __launch_bounds__(256, 8) k_batch_unpack(const BatchProb *probs,
         const int64_t u0 = __ldg(uoff + p) + (int64_t)row * nx;
         double *dstp = x + u0;
         const int64_t src = __ldg(&pb->off) + (int64_t)row * pitch;
-        for (int j0 = lane; j0 < nx; j0 += 128) {
+        for (int j0 = lane + 128 * (int)blockIdx.y; j0 < nx; j0 += 128 * (int)gridDim.y) {
             double v[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
