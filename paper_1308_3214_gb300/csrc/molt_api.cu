@@ -64,7 +64,7 @@ struct mol_ctx {
     int tune_rows_persist = 0;                 // row-split x pass: persistent CTAs with next-row L2 prefetch
     int tune_rows_nb = 1;                      // row-split x pass: one neighbour exchange per sweep where
                                                // exact to rounding (two warps per row)
-    int tune_strided_nb = 1;                   // float32 strided passes: one neighbour exchange per sweep
+    int tune_strided_nb = 2;                   // float32 strided passes: one neighbour exchange per sweep
                                                // where that is exact to rounding (2: the Horner pass
                                                // also stages its input fields in shared memory)
     int tune_strided_stage = 2;                // ... its tiles: 0 direct, 1 TMA loads, 2 TMA stores, 3 both

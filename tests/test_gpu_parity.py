@@ -687,3 +687,17 @@ def test_strided_tma_stores_of_uneven_segment_counts_match_oracle(ny, bc, stage)
         assert rel_l2(got, ref) <= tol_for("mixed", s, p), (p, rel_l2(got, ref))
     s.sync()
     s.close()
+
+
+@pytest.mark.parametrize("shape", [(32, 64, 33), (16, 96, 100), (20, 128, 257)])
+@pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
+def test_staged_3d_horner_gives_the_bits_of_the_direct_one(shape, bc):
+    """The y pass' input fields staged in shared memory (the default) or read
+    from global memory for every output: the same arithmetic."""
+    s = make(shape, 0.5 * spacing(shape[1], bc), 2, bc, "mixed")
+    u = dev(field(shape, 91, bc))
+    assert s.tuning()["strided_nb"] == 2
+    got = s.apply_F(u).clone()
+    s.set_tuning(strided_nb=1)
+    assert torch.equal(got, s.apply_F(u))
+    s.close()
