@@ -284,6 +284,19 @@ void smem_pass_geom(const mol_ctx *h, int axis, bool horner, PassGeom &G, AxisDe
     G.dps = pass_smem_bytes(horner, h->tbytes, G.W, A.ls, A.n, 1) <= h->smem_optin ? 1 : 0;
 }
 
+// Segments per CTA of the neighbour-exchange passes (their result does not
+// depend on it): fewer where the column groups would leave SMs without a CTA.
+void spread_segments(const mol_ctx *h, int64_t nlines, int n, int *rpt, int *S, int *K)
+{
+    for (int mw = *S / 2; mw >= 2 && (nlines + 31) / 32 * *K < h->num_sms; mw /= 2) {
+        int r = 0, s2 = 0, k2 = 0;
+        if (!regs_strided_plan(h->tbytes, h->bc, n, &r, &s2, &k2, h->tune_strided_rpt, mw)) return;
+        *rpt = r;
+        *S = s2;
+        *K = k2;
+    }
+}
+
 // A float64 pass: the Horner weights arrive in the units of the powers (times
 // kappa per application of this axis' D, f64_units); raw powers stay in them.
 cudaError_t run_f64(const mol_ctx *h, int axis, const PowersParams *pp, const HornerParams *hp, cudaStream_t s)
@@ -387,6 +400,7 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
             if (!regs_strided_plan(h->tbytes, h->bc, n, &rpt, &S, &K, h->tune_strided_rpt, h->tune_strided_warps))
                 return fail(h, MOL_EINVAL, "no register plan for the transposed y pass");
             LineSet L = lineset_of(h, axis);
+            if (h->tune_strided_nb && regs_strided_nb_plan(h->ax[axis].d, n, rpt)) spread_segments(h, L.nlines, n, &rpt, &S, &K);
             L.S = S;
             L.K = K;
             const AxisDev A = regs_axis(h, axis, rpt);
@@ -408,6 +422,7 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
     } else if (axis > 0 && regs_strided_plan(h->tbytes, h->bc, n, &rpt, &S, &K, h->tune_strided_rpt,
                                              h->tune_strided_warps)) {
         LineSet L = lineset_of(h, axis);
+        if (h->tune_strided_nb && regs_strided_nb_plan(h->ax[axis].d, n, rpt)) spread_segments(h, L.nlines, n, &rpt, &S, &K);
         L.S = S;
         L.K = K;
         const AxisDev A = regs_axis(h, axis, rpt);

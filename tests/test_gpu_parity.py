@@ -689,6 +689,29 @@ def test_strided_tma_stores_of_uneven_segment_counts_match_oracle(ny, bc, stage)
     s.close()
 
 
+# ---------------------------------------------------------------------------
+# grids with few column groups split each column over more CTAs; the segments'
+# arithmetic does not depend on that, so D_y of a column is the same bits on a
+# narrow grid as on a wide one
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("n", [128, 256, 512, 1024, 2048])
+@pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
+def test_strided_powers_do_not_depend_on_the_columns_beside_them(n, bc):
+    wide = 32 * 152 + 32
+    base = field((n, wide), 90, bc)
+    ref = None
+    for nx in (wide, 1000, 97, 32):
+        s = make((n, nx), 1.5 * spacing(n, bc), 3, bc, "mixed")
+        v = dev(base[:, :nx])
+        got = [s.apply_D(v, 1, p).cpu() for p in (1, 2, 3)]
+        s.close()
+        if ref is None:
+            ref = got
+        for p in range(3):
+            # (the end columns of a Dirichlet grid are boundary nodes)
+            assert torch.equal(got[p][:, 1:nx - 1], ref[p][:, 1:nx - 1]), (nx, p)
+
+
 @pytest.mark.parametrize("shape", [(32, 64, 33), (16, 96, 100), (20, 128, 257)])
 @pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
 def test_staged_3d_horner_gives_the_bits_of_the_direct_one(shape, bc):
