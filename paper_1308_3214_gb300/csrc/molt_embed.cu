@@ -323,6 +323,39 @@ struct ObjAxisF {
 
 enum : int { OBJF_D = 0, OBJF_LINV = 1, OBJF_BOTH = 2 };
 
+// out = sum_t c_t x_t in float32 (the partial sums of F)
+struct CombTermsF {
+    int n;
+    float c[kCombMax];
+    const float *x[kCombMax];
+};
+
+// The level update that rides on F's last sweep: (nh, nl) = a u + b up + c
+// sum_t c_t x_t in pair arithmetic, term own being the sweep's result, which
+// is not stored.  (A pass of its own read every term again, 20 us at 2048^2.)
+// With that and the small sweeps overlapping their launches, us per step of
+// the ellipse at P = 2: 257^2 61 -> 50, 400^2 75 -> 61, 777^2 85 -> 79, 1025^2
+// 104 -> 98, 2048^2 190 -> 181.
+struct LevelF {
+    CombTermsF t;
+    int own;
+    float a, b, c;
+    const float *uh, *ul, *ph, *pl;
+    float *nh, *nl;       // nullptr: none
+};
+
+__device__ __forceinline__ void obj_level32(const LevelF &lv, long long i, float own)
+{
+    const float uh = lv.uh[i], ul = lv.ul[i];
+    const float ph = lv.b != 0.f ? lv.ph[i] : 0.f, pl = lv.b != 0.f ? lv.pl[i] : 0.f;
+    float F = 0.f;
+    for (int j = 0; j < lv.t.n; ++j) F += lv.t.c[j] * (j == lv.own ? own : lv.t.x[j][i]);
+    float h, l;
+    molt::level_pair(uh, ul, ph, pl, F, lv.a, lv.b, lv.c, h, l);
+    lv.nh[i] = h;
+    lv.nl[i] = l;
+}
+
 // MODE OBJF_D: out = D v; OBJF_LINV: out = v - D v (= L^{-1} v); OBJF_BOTH:
 // out = D v and out2 = v - D v (and out3 = D v when given).  accum adds to
 // out.  PAIR: v is a float32 pair level (in = hi, lo = lo plane), else a
@@ -334,13 +367,18 @@ enum : int { OBJF_D = 0, OBJF_LINV = 1, OBJF_BOTH = 2 };
 // recurrences each thread reduces a chunk of its group's line, the chunk maps
 // are composed over the lanes of a warp (shuffles) and over the group's warps
 // (their totals in shared memory), and each chunk is re-run from its carry.
-// slot: elements per line array (>= m + 2), four arrays per line.
+// slot: elements per line array (> obj_slot(m + 1)), four arrays per line.  lv.nh: the
+// result is not stored but combined into the next level.
+// one word of padding per 32: threads that walk chunks of 4 or 8 nodes start
+// on different banks
+__host__ __device__ __forceinline__ int obj_slot(int k) { return k + (k >> 5); }
+
 template <bool PAIR, int CPB>
 __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax, const ObjLineF *lines, int nlines,
                                                                     const float *__restrict__ in,
                                                                     const float *__restrict__ lo, float *out,
                                                                     float *out2, float *out3, int mode, int accum,
-                                                                    int slot)
+                                                                    int slot, const __grid_constant__ LevelF lv)
 {
     constexpr int NW = kObjThreads32 / 32, NT = kObjThreads32 * CPB;
     extern __shared__ __align__(16) float smf[];
@@ -353,6 +391,7 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
     const int ij = tid % CPB, ii = tid / CPB;           // interleaved load/store mapping: line, position
     const long long st = ax.stride;
     const float d = ax.d, c = ax.c;
+    molt::pdl_enter();
     for (int gb = blockIdx.x * CPB; gb < nlines; gb += gridDim.x * CPB) {
         __syncthreads();
         if (tid < CPB) {
@@ -390,7 +429,7 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
         float *H = smf + (size_t)grp * 4 * slot;
         float *Lo = H + slot;        // lo plane (PAIR)
         float *S = Lo + slot;        // second differences s_t
-        float *Q = S + slot;         // q_k, then T_k, then e_k
+        float *Q = S + slot;         // q_k, then T_k, then e_k (obj_slot)
         const ObjLineF &ln = lines[li < nlines ? li : 0];
         // second differences s_t, t = 1..m (end triples with their spacings)
         for (int t = 1 + gt; t <= m; t += kObjThreads32) {
@@ -414,9 +453,9 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
             if (k == 1) q = ln.g11 * S[1] + (m >= 2 ? ln.g12 * S[2] : 0.f);
             else if (k == m) q = ln.gNa * S[m - 1] + ln.gNb * S[m];
             else q = ax.ge * (S[k - 1] + S[k + 1]) + ax.gc * S[k];
-            Q[k] = q;
+            Q[obj_slot(k)] = q;
         }
-        if (gt == 0) { Q[0] = 0.f; Q[N] = 0.f; }
+        if (gt == 0) { Q[0] = 0.f; Q[obj_slot(N)] = 0.f; }
         __syncthreads();
         const int s = (N + kObjThreads32) / kObjThreads32;      // ceil((N + 1) / threads)
         const int k0 = m > 0 ? min(gt * s, N + 1) : 0, k1 = m > 0 ? min(k0 + s, N + 1) : 0;
@@ -426,7 +465,7 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
             float qq = 0.f;
             for (int k = k1 - 1; k >= k0; --k) {
                 const float g = (k == N - 1) ? ln.dB : d;
-                qq = (k == N) ? 0.f : g * qq + Q[k];
+                qq = (k == N) ? 0.f : g * qq + Q[obj_slot(k)];
             }
             float p = ax.dpow[k1 - k0];
             if (k0 <= N - 1 && N - 1 < k1) p *= ln.rB;
@@ -439,8 +478,8 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
             float y = (lane == 31) ? yin : pn * yin + qn;
             for (int k = k1 - 1; k >= k0; --k) {
                 const float g = (k == N - 1) ? ln.dB : d;
-                y = (k == N) ? 0.f : g * y + Q[k];
-                Q[k] = y;
+                y = (k == N) ? 0.f : g * y + Q[obj_slot(k)];
+                Q[obj_slot(k)] = y;
             }
         }
         // causal: e_k = g_k e_{k-1} + (1 - g_k^2) T_k, e_0 = 0 (g_1 = dA, g_N = dB)
@@ -449,7 +488,7 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
             for (int k = k0; k < k1; ++k) {
                 const float g = (k == 1) ? ln.dA : (k == N ? ln.dB : d);
                 const float cg = (k == 1) ? ln.cA : (k == N ? ln.cB : c);
-                qq = (k == 0) ? 0.f : g * qq + cg * Q[k];
+                qq = (k == 0) ? 0.f : g * qq + cg * Q[obj_slot(k)];
             }
             float p = ax.dpow[k1 - k0];
             if (k0 <= 1 && 1 < k1) p *= ln.rA;
@@ -464,14 +503,14 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
             for (int k = k0; k < k1; ++k) {
                 const float g = (k == 1) ? ln.dA : (k == N ? ln.dB : d);
                 const float cg = (k == 1) ? ln.cA : (k == N ? ln.cB : c);
-                y = (k == 0) ? 0.f : g * y + cg * Q[k];
-                Q[k] = y;
+                y = (k == 0) ? 0.f : g * y + cg * Q[obj_slot(k)];
+                Q[obj_slot(k)] = y;
             }
         }
         __syncthreads();
         // e += A' e^{-alpha (x - a)} + B' e^{-alpha (b - x)} with e_0 = e_N = 0
         if (gt == 0 && m > 0) {
-            const float Bp = -Q[N] * ln.inv, Ap = -Bp * ln.mu;
+            const float Bp = -Q[obj_slot(N)] * ln.inv, Ap = -Bp * ln.mu;
             l_Ad[grp] = Ap * ln.dA;
             l_Bd[grp] = Bp * ln.dB;
         }
@@ -485,11 +524,16 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
                 const long long kk = r - pj + 1;
                 if (kk >= 1 && kk <= mj) {
                     const int k = (int)kk;
-                    const float e = Qj[k] + Ad * ax.dpow[k - 1] + Bd * ax.dpow[mj - k];
+                    const float e = Qj[obj_slot(k)] + Ad * ax.dpow[k - 1] + Bd * ax.dpow[mj - k];
                     const float v = Hj[k] + Lj[k];
                     const long long at = bj + (k - 1) * st;
-                    const float rr = (mode == OBJF_LINV) ? v - e : e;
-                    out[at] = accum ? out[at] + rr : rr;
+                    float rr = (mode == OBJF_LINV) ? v - e : e;
+                    if (accum) rr = out[at] + rr;
+                    if (lv.nh) {
+                        obj_level32(lv, at, rr);
+                        continue;
+                    }
+                    out[at] = rr;
                     if (mode == OBJF_BOTH) {
                         out2[at] = v - e;
                         if (out3) out3[at] = e;
@@ -500,14 +544,15 @@ __global__ void __launch_bounds__(kObjThreads32 * CPB) k_obj_sweep32(ObjAxisF ax
     }
 }
 
-// out = sum_t c_t x_t in float32 (the partial sums of F)
-struct CombTermsF {
-    int n;
-    float c[kCombMax];
-    const float *x[kCombMax];
-};
-// Both kernels below touch the interior nodes only, row by row (the line
-// objects of the contiguous axis): outside the domain every field stays zero.
+// the sweep of axis a, from a pair level or a float32 field
+auto sweep32_kernel(bool pair, int a)
+{
+    return a == 0 ? (pair ? k_obj_sweep32<true, kObjCpb[0]> : k_obj_sweep32<false, kObjCpb[0]>)
+                  : (pair ? k_obj_sweep32<true, kObjCpb[1]> : k_obj_sweep32<false, kObjCpb[1]>);
+}
+
+// out = sum_t c_t x_t at the interior nodes, row by row (the line objects of
+// the contiguous axis): outside the domain every field stays zero.
 __global__ void __launch_bounds__(256) k_obj_combine32(CombTermsF t, const ObjLineF *rows, int nrows, float *out)
 {
     for (int li = blockIdx.x; li < nrows; li += gridDim.x) {
@@ -518,26 +563,6 @@ __global__ void __launch_bounds__(256) k_obj_combine32(CombTermsF t, const ObjLi
             float v = 0.f;
             for (int j = 0; j < t.n; ++j) v += t.c[j] * t.x[j][i];
             out[i] = v;
-        }
-    }
-}
-
-// next level in pair arithmetic: (nh, nl) = a u + b up + c (F + sum_t c_t x_t)
-__global__ void __launch_bounds__(256) k_obj_level32(CombTermsF t, const ObjLineF *rows, int nrows, const float *uh,
-                                                     const float *ul, const float *ph, const float *pl, float a,
-                                                     float b, float cF, float *nh, float *nl)
-{
-    for (int li = blockIdx.x; li < nrows; li += gridDim.x) {
-        const long long base = rows[li].base;
-        const int m = rows[li].m;
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            const long long i = base + k;
-            float F = 0.f;
-            for (int j = 0; j < t.n; ++j) F += t.c[j] * t.x[j][i];
-            float h, l;
-            molt::level_pair(uh[i], ul[i], b != 0.f ? ph[i] : 0.f, b != 0.f ? pl[i] : 0.f, F, a, b, cF, h, l);
-            nh[i] = h;
-            nl[i] = l;
         }
     }
 }
@@ -845,22 +870,13 @@ mol_status sweep(mol_embed_ctx *e, int a, const double *in, double *out, double 
     const ObjAxis &X = e->ax[a];
     const size_t smem = sizeof(double) * 4 * (size_t)X.threads;
     Timed t(e, a, s);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)X.ctas);
-    cfg.blockDim = dim3((unsigned)X.threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
     // a sweep that leaves SMs free lets the next one start while it ends (the
     // next one's threads fetch their tables and wait): 9 launches a step, each
     // as short as its latencies on small grids
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = X.ctas <= e->sms && !e->timing ? 1 : 0;
-    ECK(cudaLaunchKernelEx(&cfg, e->seg == 4 ? k_obj_sweep<4> : e->seg == 8 ? k_obj_sweep<8>
-                                 : e->seg == 12 ? k_obj_sweep<12> : k_obj_sweep<16>,
-                           X, (const ObjLine *)e->lines[a], in, out, out2, out3, mode, accum, cb ? *cb : none),
+    ECK(launch_kernel(e->seg == 4 ? k_obj_sweep<4> : e->seg == 8 ? k_obj_sweep<8> : e->seg == 12 ? k_obj_sweep<12>
+                                                                                                  : k_obj_sweep<16>,
+                      dim3(X.ctas), dim3(X.threads), smem, s, X.ctas <= e->sms && !e->timing, 1, X,
+                      (const ObjLine *)e->lines[a], in, out, out2, out3, mode, accum, cb ? *cb : none),
         "line-object sweep");
     ++e->launches;
     ECK(cudaGetLastError(), "line-object sweep");
@@ -1010,32 +1026,26 @@ mol_status run_update(mol_embed_ctx *e, const double *u, const double *up, doubl
 // ---- float32 sweeps (MOL_MIXED) ----
 // one difference-form sweep along axis a; lo: the lo plane when in is a pair level
 mol_status sweep32(mol_embed_ctx *e, int a, const float *in, const float *lo, float *out, float *out2, int mode,
-                   int accum, cudaStream_t s, float *out3 = nullptr)
+                   int accum, cudaStream_t s, float *out3 = nullptr, const LevelF *lv = nullptr)
 {
     if (e->nlines[a] == 0) return MOL_OK;
     const int cpb = kObjCpb[a];
     const int grid = std::min(e->grid32[a], (e->nlines[a] + cpb - 1) / cpb);
     Timed t(e, a, s);
-    auto launch = [&](auto kern) {
-        kern<<<grid, kObjThreads32 * cpb, e->smem32[a], s>>>(e->ax32[a], e->lines32[a], e->nlines[a], in, lo, out,
-                                                             out2, out3, mode, accum, e->slot);
-    };
-    if (cpb == 1) {
-        if (lo) launch(k_obj_sweep32<true, 1>);
-        else launch(k_obj_sweep32<false, 1>);
-    } else {
-        if (lo) launch(k_obj_sweep32<true, kObjCpb[1]>);
-        else launch(k_obj_sweep32<false, kObjCpb[1]>);
-    }
+    ECK(launch_kernel(sweep32_kernel(lo != nullptr, a), dim3(grid), dim3(kObjThreads32 * cpb), (size_t)e->smem32[a], s,
+                      grid <= e->sms && !e->timing, 1, e->ax32[a], (const ObjLineF *)e->lines32[a], e->nlines[a], in, lo,
+                      out, out2, out3, mode, accum, e->slot, lv ? *lv : LevelF{}),
+        "line-object sweep (float32)");
     ++e->launches;
     ECK(cudaGetLastError(), "line-object sweep (float32)");
     return MOL_OK;
 }
 
 // out = C v (eq. C_def_ADI) with L^{-1} = 1 - D: D_x v - D_y D_x v + D_y v - D_x D_y v.
-// dyv: D_y v when an earlier sweep has formed it, else null.
+// dyv: D_y v when an earlier sweep has formed it, else null.  lv: the level
+// update that takes C v in its last sweep (out then holds a partial sum).
 mol_status apply_C32(mol_embed_ctx *e, const float *v, const float *vlo, float *out, cudaStream_t s,
-                     const float *dyv = nullptr)
+                     const float *dyv = nullptr, const LevelF *lv = nullptr)
 {
     EST(sweep32(e, 0, v, vlo, e->t132, nullptr, OBJF_D, 0, s));               // t1 = D_x v
     EST(sweep32(e, 1, e->t132, nullptr, out, nullptr, OBJF_LINV, 0, s));      // out = L_y^{-1} t1
@@ -1043,7 +1053,7 @@ mol_status apply_C32(mol_embed_ctx *e, const float *v, const float *vlo, float *
         EST(sweep32(e, 1, v, vlo, e->t132, nullptr, OBJF_D, 0, s));           // t1 = D_y v
         dyv = e->t132;
     }
-    return sweep32(e, 0, dyv, nullptr, out, nullptr, OBJF_LINV, 1, s);       // out += L_x^{-1} D_y v
+    return sweep32(e, 0, dyv, nullptr, out, nullptr, OBJF_LINV, 1, s, nullptr, lv);   // out += L_x^{-1} D_y v
 }
 
 // out = D v (eq. D_def_ADI) = v - L_x^{-1} L_y^{-1} v = D_y v + D_x (L_y^{-1} v); dyv, when
@@ -1058,51 +1068,55 @@ mol_status combine32(mol_embed_ctx *e, const CombTermsF &t, float *out, cudaStre
 {
     if (e->nlines[0] == 0) return MOL_OK;
     Timed tm(e, 2, s);
-    k_obj_combine32<<<std::min(e->nlines[0], e->grid32[0]), 256, 0, s>>>(t, e->lines32[0], e->nlines[0], out);
+    k_obj_combine32<<<std::min(e->nlines[0], 8 * e->sms), 256, 0, s>>>(t, e->lines32[0], e->nlines[0], out);
     ++e->launches;
     ECK(cudaGetLastError(), "combine (float32)");
     return MOL_OK;
 }
 
 // F[u] of the pair level (uh, ul), Table 3 order as run_update.  With nh
-// set: (nh, nl) = ea u + eb up + ec F in pair arithmetic; else F (float32)
-// into F32.
+// set: (nh, nl) = ea u + eb up + ec F in pair arithmetic, in F's last sweep;
+// else F (float32) into F32.
 mol_status run_update32(mol_embed_ctx *e, const float *uh, const float *ul, const float *ph, const float *pl,
                         float *nh, float *nl, float *F32, float ea, float eb, float ec, cudaStream_t s)
 {
     const int P = e->P;
+    LevelF lv{};
+    lv.a = ea; lv.b = eb; lv.c = ec;
+    lv.uh = uh; lv.ul = ul; lv.ph = ph; lv.pl = pl;
+    lv.nh = nh; lv.nl = nl;
     for (int p = 1; p <= P; ++p) {
+        // F's partial sum.  The terms of stage 1 are tw_11 C u alone, and C u
+        // is still in tmp32 after stage 2 (whose only C swaps V_1 out), so
+        // with P > 1 they join the sum of stage 2 instead of a pass of their own
+        const bool fuse = p == P && nh;
+        CombTermsF &t = lv.t;
+        t.n = 0;
+        auto add = [&](double c, const float *x) { t.c[t.n] = (float)c; t.x[t.n++] = x; };
         if (p == 1) {
-            EST(apply_C32(e, uh, ul, e->V32[1], s));
+            add(e->tw[1 * 8 + 1], e->V32[1]);
+            lv.own = 0;
+            EST(apply_C32(e, uh, ul, e->V32[1], s, nullptr, fuse ? &lv : nullptr));
+            if (P > 1) continue;
         } else {
             // D_y V_{p-1} serves both D V_{p-1} and C V_{p-1}: formed once
             EST(apply_D32(e, e->V32[p - 1], e->V32[p], s, e->t332));
             for (int k = 1; k < p; ++k) {
-                EST(apply_C32(e, e->V32[k], nullptr, e->tmp32, s, k == p - 1 ? e->t332 : nullptr));
+                if (k == p - 1) {
+                    // (the last C V_k, of k = p - 1, goes to tmp32: then V_{p-1})
+                    if (p == 2) add(e->tw[1 * 8 + 1], e->V32[1]);
+                    else add(1.0, e->Fb32);
+                    for (int q = 1; q <= p; ++q) {
+                        if (q == k) lv.own = t.n;
+                        add(e->tw[p * 8 + (p - q + 1)], q == k ? e->tmp32 : e->V32[q]);
+                    }
+                }
+                EST(apply_C32(e, e->V32[k], nullptr, e->tmp32, s, k == p - 1 ? e->t332 : nullptr,
+                              fuse && k == p - 1 ? &lv : nullptr));
                 std::swap(e->V32[k], e->tmp32);
             }
         }
-        // F's partial sum.  The terms of stage 1 are tw_11 C u alone, and C u
-        // is still in tmp32 after stage 2 (whose only C swaps V_1 out), so
-        // with P > 1 they join the sum of stage 2 instead of a pass of their own
-        if (p == 1 && P > 1) continue;
-        CombTermsF t{};
-        if (p == 2) { t.c[t.n] = (float)e->tw[1 * 8 + 1]; t.x[t.n++] = e->tmp32; }
-        if (p > 2) { t.c[t.n] = 1.f; t.x[t.n++] = e->Fb32; }
-        for (int k = 1; k <= p; ++k) {
-            t.c[t.n] = (float)e->tw[p * 8 + (p - k + 1)];
-            t.x[t.n++] = e->V32[k];
-        }
-        if (p < P || !nh) {
-            EST(combine32(e, t, p < P ? e->Fb32 : F32, s));
-        } else {
-            if (e->nlines[0] == 0) continue;
-            Timed tm(e, 2, s);
-            k_obj_level32<<<std::min(e->nlines[0], e->grid32[0]), 256, 0, s>>>(t, e->lines32[0], e->nlines[0], uh, ul,
-                                                                                ph, pl, ea, eb, ec, nh, nl);
-            ++e->launches;
-            ECK(cudaGetLastError(), "level update (float32 pairs)");
-        }
+        if (!fuse) EST(combine32(e, t, p < P ? e->Fb32 : F32, s));
     }
     return MOL_OK;
 }
@@ -1292,7 +1306,7 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
     }
     if (st == MOL_OK) {
         // line arrays sized for the longest line (even, for 16-byte alignment)
-        e->slot = (int)((maxm + 2 + 1) & ~(int64_t)1);
+        e->slot = (obj_slot((int)maxm + 1) + 2) & ~1;
         // (float32: four arrays per line)
         int dev = 0, sms = 152;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1314,19 +1328,18 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
             }
             for (int a = 0; a < 2 && st == MOL_OK; ++a) st = obj_items(e, a, msz[a]);
         } else {
-            const void *kf[2][2] = {{(const void *)k_obj_sweep32<true, 1>, (const void *)k_obj_sweep32<false, 1>},
-                                    {(const void *)k_obj_sweep32<true, kObjCpb[1]>,
-                                     (const void *)k_obj_sweep32<false, kObjCpb[1]>}};
             for (int a = 0; a < 2 && st == MOL_OK; ++a) {
                 e->smem32[a] = (int)(sizeof(float) * 4 * (size_t)e->slot * kObjCpb[a]);
                 for (int v = 0; v < 2 && st == MOL_OK; ++v)
-                    if ((ce = cudaFuncSetAttribute(kf[a][v], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                    if ((ce = cudaFuncSetAttribute((const void *)sweep32_kernel(v == 0, a),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    e->smem32[a])) != cudaSuccess)
                         st = efail(e, MOL_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(ce));
                 int ps = 1;
-                if (st == MOL_OK && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kf[a][0], kObjThreads32 *
-                                                                                  kObjCpb[a], e->smem32[a]) !=
-                                        cudaSuccess) {
+                if (st == MOL_OK &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, (const void *)sweep32_kernel(true, a),
+                                                                  kObjThreads32 * kObjCpb[a], e->smem32[a]) !=
+                        cudaSuccess) {
                     cudaGetLastError();
                     ps = 1;
                 }

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <string>
+#include <utility>
 #include <vector>
 #include "molt.h"
 #include "molt_kernels.cuh"
@@ -19,6 +20,38 @@ double beta_max_of(int P);                         // Table 1; -1 outside 1..5
 bool expand_coefficients(int ndim, int P, double beta, std::vector<double> &out);
 double quad_R(double nu);                          // second-difference weight of the quadratic rule
 void axis_constants(double nu, int64_t n, int bc, int quad, AxisDev &A);
+
+// Launch with the attributes of a pass: a cluster of cluster_y CTAs along y
+// (> 1), and (pdl) programmatic dependent launch, under which the kernel's CTAs
+// may be scheduled while the previous kernel in the stream finishes (every
+// pass kernel waits for it in pdl_enter before touching the fields).
+template <class... KArgs, class... Args>
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                          int cluster_y, Args &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (cluster_y > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = 1;
+        attr[na].val.clusterDim.y = (unsigned)cluster_y;
+        attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 // Message for mol_last_error(NULL) (molt_api.cu).
 void set_global_error(const std::string &msg);

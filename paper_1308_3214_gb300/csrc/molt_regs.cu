@@ -10,37 +10,11 @@ namespace molt {
 
 namespace {
 
-// Launch with the launch attributes of a pass: a cluster of cluster_y CTAs
-// along y (> 1), and (L.pdl) programmatic dependent launch, under which the
-// kernel's CTAs may be scheduled while the previous kernel in the stream
-// finishes (every pass kernel waits for it in pdl_enter before touching
-// global memory).
 template <class... KArgs, class... Args>
 cudaError_t launch_pass(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                         const LineSet &L, int cluster_y, Args &&...args)
 {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (cluster_y > 1) {
-        attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = 1;
-        attr[na].val.clusterDim.y = (unsigned)cluster_y;
-        attr[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    if (L.pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    return launch_kernel(kernel, grid, block, smem, s, L.pdl != 0, cluster_y, std::forward<Args>(args)...);
 }
 
 constexpr int kContigWarps = 4;

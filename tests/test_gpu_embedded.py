@@ -311,3 +311,43 @@ def test_degenerate_domains(prec):
     assert not s.solve_host(z, 3).any()
     assert not s.apply_F(_dev(z)).cpu().numpy().any()
     s.close()
+
+
+# The float64 sweep's segment length follows the size: 4, 8, 12 and 16 nodes
+# per thread on 152 SMs at these sizes.
+@pytest.mark.parametrize("n", [257, 400, 520, 777])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_linv_at_every_segment_length(n, axis):
+    g = workloads.disk_grid(n)
+    s = _solver(g, 1.3, 2)
+    v = workloads.random_field((g.ny, g.nx), 31 + axis) * g.mask
+    got = s.linv(_dev(v), axis).cpu().numpy()
+    ref = oracle.linv_axis_embed(v, axis, g, oracle.beta_max(2) / (1.3 * g.hx))
+    assert _rel(got, ref) <= _tol(g)
+    assert not got[~g.mask].any()
+    s.close()
+
+
+@pytest.mark.parametrize("P", [1, 2, 3, 5])
+@pytest.mark.parametrize("shape", [("ellipse", 61), ("disk", 300)])
+def test_mixed_level_update_is_F_and_the_levels(P, shape):
+    """The update that rides on F's last sweep against apply_F's (stored) F:
+    the same float32 F, so the levels agree to the pair arithmetic: a level's
+    pair holds 48 bits, the update three rounded pair sums of 2^-46 each."""
+    from paper_1308_3214_gb300 import molt
+    g = workloads.ellipse_grid(shape[1]) if shape[0] == "ellipse" else workloads.disk_grid(shape[1])
+    s = molt.EmbedSolver(g, dt=1.2 * g.hx, P=P, prec="mixed")
+    u0 = workloads.random_field((g.ny, g.nx), 51) * g.mask
+    a = _dev(u0)
+    b = s.start(a)
+    ref = u0 + 0.5 * s.apply_F(a).cpu().numpy()
+    big = np.abs(u0).max() + np.abs(ref).max()
+    assert np.abs(b.cpu().numpy() - ref).max() <= 2.0 ** -44 * big
+    u1 = b.cpu().numpy()
+    F1 = s.apply_F(b).cpu().numpy()
+    s.step(a, b, 1)
+    ref = 2 * u1 - u0 + F1
+    big = 2 * np.abs(u1).max() + np.abs(u0).max() + np.abs(F1).max()
+    assert np.abs(b.cpu().numpy() - ref).max() <= 2.0 ** -44 * big
+    assert np.array_equal(a.cpu().numpy(), u1)
+    s.close()
