@@ -12,6 +12,24 @@ namespace {
 // segments whose inflow matters: d^(R win) <= 2^-60
 int f64_window(double nu, int R) { return std::max(1, (int)std::ceil(60.0 * std::log(2.0) / (nu * (double)R))); }
 
+// The window's sums over win of G segments: steps one by one cost an operation
+// each (64 cycles with few warps about), doubling one operation, a barrier and
+// a trip through shared memory; blocks = steps left after dbl doublings.
+void f64_window_sums(int win, int G, int *dbl, int *blocks)
+{
+    const int J = std::min(win, std::max(G - 1, 1));
+    double best = 0.0;
+    for (int k = 0; k <= 7; ++k) {
+        const int b = (J + (1 << k) - 1) >> k;
+        const double cost = b + 1.75 * k;
+        if (k == 0 || cost < best) {
+            best = cost;
+            *dbl = k;
+            *blocks = b;
+        }
+    }
+}
+
 double half_K(double nu) { return -std::expm1(-2.0 * nu) / (2.0 * nu); }
 
 F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
@@ -21,6 +39,10 @@ F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
     c.G = (A.n + R - 1) / R;
     c.len_last = A.n - (c.G - 1) * R;
     c.win = f64_window(nu, R) + (c.len_last < R ? 1 : 0);    // a short last segment spans less than d^R
+    c.R = R;
+    f64_window_sums(c.win, c.G, &c.dbl, &c.blocks);
+    for (int k = 0; k < 8; ++k) c.pd[k] = std::exp(-nu * (double)R * (double)(1 << k));
+    c.pB = c.pd[c.dbl];
     c.d = A.d;
     const double om2 = -std::expm1(-2.0 * nu);             // 1 - d^2
     c.kappa = f64_kappa(nu, quad);
@@ -51,6 +73,7 @@ template <int BC, int KM>
 cudaError_t run_f64_r(bool contig, const F64Plan &pl, const F64Axis &A, const F64Lines &L, const F64Prog &p, cudaStream_t s)
 {
     switch (pl.R) {
+    case 4: return run_f64<4, BC, KM>(contig, pl, A, L, p, s);
     case 8: return run_f64<8, BC, KM>(contig, pl, A, L, p, s);
     case 16: return run_f64<16, BC, KM>(contig, pl, A, L, p, s);
     case 32: return run_f64<32, BC, KM>(contig, pl, A, L, p, s);
@@ -69,7 +92,8 @@ cudaError_t attr_f64()
 template <int BC, int KM>
 cudaError_t attr_f64_r()
 {
-    cudaError_t e = attr_f64<8, BC, KM>();
+    cudaError_t e = attr_f64<4, BC, KM>();
+    if (e == cudaSuccess) e = attr_f64<8, BC, KM>();
     if (e == cudaSuccess) e = attr_f64<16, BC, KM>();
     return e == cudaSuccess ? attr_f64<32, BC, KM>() : e;
 }
@@ -101,21 +125,25 @@ bool f64_axis_ok(int n, bool contig) { return n <= kF64MaxR * kF64Threads / (con
 
 // Segment length R and lines per CTA C: the pair whose busiest quarter of an
 // SM (each issues its own warps) has the least to do.  A segment costs about 8
-// operations a point and sweep (12 with a Horner step's fields) and 5 per
-// segment of its inflow window; whole warps are issued whether their threads
-// are live or not; a quarter with one warp also waits about 0.4 of its time for
-// the recurrences, with k warps 0.4 / k.  Equal choices take the longer runs
-// (larger C).  Measured against every R and C: 96 x 100 x 75, P = 2: y 142 us
-// at R = 16, C = 16 (157 at R = 32, 166 at R = 8); 512^2, P = 3: y 26.6 us at R
-// = 16, C = 4 (30.9, 38.9); 1000 x 777: y 55.3 us at R = 32, C = 8 (59.3).
+// operations a point and sweep (12 with a Horner step's fields), 2 per block of
+// its inflow window, 3.5 per doubling, and 18 for its ends and barriers; whole
+// warps are issued whether their threads are live or not; a quarter with one
+// warp also waits about 0.4 of its time for the recurrences, with k warps 0.4 / k;
+// runs of two columns cost 1.15 (half a sector each).  Equal choices take the
+// longer runs (larger C).  Measured against other weights: 1000 x 777, P = 3: y 58
+// us at R = 32, C = 8 (68 at R = 8, C = 2); 288 x 2016, P = 1: y 19 us at R = 16, C =
+// 2 (27 at R = 32, C = 4); 70 x 300, P = 2: y 15 us at R = 4, C = 2 (21 at R = 16, C =
+// 4); 512^2, P = 3: x 38 us at R = 8 (42 at R = 16).
 bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sms, F64Plan *out)
 {
     if (!f64_axis_ok(n, contig)) return false;
     double best = 0.0;
     F64Plan pl{};
-    for (int R = 8; R <= kF64MaxR; R *= 2) {
+    for (int R = 4; R <= kF64MaxR; R *= 2) {
         const int G = (n + R - 1) / R;
-        const double ops = (horner ? 12.0 : 8.0) * R + 5.0 * std::min(f64_window(nu, R), G) + 12.0;
+        int dbl = 0, blocks = 0;
+        f64_window_sums(f64_window(nu, R), G, &dbl, &blocks);
+        const double ops = (horner ? 12.0 : 8.0) * R + 2.0 * blocks + 3.5 * dbl + 18.0;
         // strided accesses in runs of 4 columns or more, except where a column fills the CTA
         const int c_min = contig ? 1 : (4 * G <= kF64Threads ? 4 : 2);
         for (int C = c_min; C <= 32 && C * G <= kF64Threads; C *= 2) {
@@ -126,7 +154,7 @@ bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sm
             // warps a quarter works through; beyond one round of resident CTAs the SMs even out
             const double load = per_sm <= occ ? std::ceil(per_sm * warps / 4.0) : (double)ctas / sms * warps / 4.0 + 0.5;
             const double resident = std::min(load, std::max(1.0, occ * warps / 4.0));
-            const double cost = load * ops * (1.0 + 0.4 / resident);
+            const double cost = load * ops * (1.0 + 0.4 / resident) * (!contig && C == 2 ? 1.15 : 1.0);
             if (pl.R == 0 || cost < best || (cost == best && C > pl.C)) {
                 best = cost;
                 pl = F64Plan{R, G, C, threads, smem};

@@ -24,20 +24,27 @@
 //     a d^k + b d^(len-1-k) the two terms would cancel at slow decay.)  The
 //     earlier scheme reduced, rescanned and reduced again.
 //
-// Carries: each segment publishes E (its zero-inflow y at its last point) and
-// G (its zero-inflow g at its first point).  After one barrier every segment
-// sums the inflow from as many neighbours as matter (d^(R win) <= 2^-60; the
-// whole line where the decay is slow):
-//   yin = sum_j d^(R (j-1)) E_{m-j},
-//   gin = sum_{l>m} d^(R (l-m-1)) (G_l + w_0 Y_{l-1}),  Y_l = E_l + d^R Y_{l-1};
-//   a = yin,  b = gin.
+// Carries: each segment publishes E (its zero-inflow y at its last point); the
+// causal inflow of segment m is
+//   yin_m = sum_j d^(R (j-1)) E_{m-j},
+// with which its g at its first point, before anything flows in from the
+// right, is H_m = G_m + w_0 yin_m (G zero-inflow); published in turn, it gives
+//   gin_m = sum_j d^(R (j-1)) H_{m+j};   a = yin,  b = gin.
+// Either sum takes the segments that matter (d^(R win) <= 2^-60; the whole line
+// where the decay is slow): one operation a segment, or, for a wide window,
+// after log2 B rounds that leave in each slot the sum over a block of B
+// segments, one a block.  (Both sums from one exchange cost 5 operations a
+// segment, 64 cycles each where a quarter of an SM has a single warp: steps of
+// 72 x 65, P = 2, CFL 3.8 took 35.7 us, now 20.2; 256^2, P = 2, 34.0 -> 22.8; 512^2,
+// P = 3, 63 -> 55; 1000^2 periodic, P = 3, CFL 4, 183 -> 172.)
 // Dirichlet (e = 0, or given data, at the ends; s_0 := s_1, s_{n-1} := s_{n-2}):
 // the rows at the ends drop out of s, and A' d^j + B' d^(n-1-j) with
 //   A' + mu B' = r_0 = e_0/kappa - rho s_1 - g_0,
 //   mu A' + B' = r_1 = e_{n-1}/kappa - rho s_{n-2} - g_{n-1}
-// joins a and b in the segments it reaches (d^k = (1 - d^2)/d w_k + d^(2 len - k)).  Periodic lines wrap (all images
-// through 1 / (1 - mu) where the window covers the line).  The last segment
-// may hold fewer than R points.
+// joins a and b in the segments it reaches (d^k = (1 - d^2)/d w_k + d^(2 len - k)).
+// Periodic lines: what the line's last point hands to its first, all images
+// through 1 / (1 - mu), joins yin in the segments it reaches, and what its first
+// hands to its last joins gin.  The last segment may hold fewer than R points.
 //
 // One kernel serves every axis: on the contiguous one neighbouring threads hold
 // neighbouring segments of a row and each reads its own segment in 32-byte
@@ -48,10 +55,10 @@
 // run of C columns.  s waits in shared memory while its registers hold y and g.
 //
 // Measured, us per pass, against the earlier warp-per-row, clustered and
-// shared-memory kernels: 2048^2, P = 3, y 419 -> 219, x 1470 -> 355 (23 and 40
-// operations a point: 86 % and 84 % of the float64 pipe's cycles); 96 x 100 x
-// 75, P = 2, x 154 -> 52, y 260 -> 143, z 72 -> 32; 256^3 periodic, P = 2, x
-// 1150 -> 764, y 3000 -> 2124, z 746 -> 466.
+// shared-memory kernels: 2048^2, P = 3, y 419 -> 225, x 1470 -> 355 (23 and 40
+// operations a point: 84 % of the float64 pipe's cycles); 96 x 100 x 75, P = 2,
+// x 154 -> 56, y 260 -> 133, z 72 -> 31; 256^3 periodic, P = 2, x 1150 -> 774, y
+// 3000 -> 2150, z 746 -> 496.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -65,9 +72,12 @@ constexpr int kF64Threads = 256;       // threads per CTA at most
 // Constants of one axis for segments of R points (host, molt_f64.cu).
 struct F64Axis {
     int n, G, len_last;    // points, segments, points of the last one
-    int win;               // segments whose inflow matters on each side
+    int R;                 // points per segment
+    int win;               // segments whose inflow matters on each side,
+    int dbl, blocks;       // summed as blocks of 2^dbl
     double d, rho, kappa;
     double dR, dRl;        // d^R, d^len_last
+    double pB, pd[8];      // decay over a block; over 2^k segments
     double e1, id;         // (1 - d^2) / d, 1 / d
     double mu, inv;        // as AxisDev
     double pw[kF64MaxR + 1];   // d^k
@@ -104,11 +114,11 @@ struct F64Prog {
 
 // this thread's place on its line
 struct F64Seg {
-    double *E, *G, *ends;      // slots [threads] and [4][C]
+    double *E, *G, *first, *ends;   // slots [threads] and [4][C]
     double *s;                 // this segment's s: s[k ss]
     int ss;
     int t, st, t0;             // slot, distance to the next segment's slot, slot of segment 0
-    int seg, line, C;
+    int seg, line, C, a;       // a: its first point
     bool live, last, tail;     // on the line; its last segment; shorter than R
 };
 
@@ -121,66 +131,62 @@ __device__ __forceinline__ double f64_pick(const double (&z)[R], int k)
     return v;
 }
 
-// Inflow of this segment, a w_k + b d^(len-k), and the right sides r_0, r_1
-// of the boundary terms where this thread has them: on the strided axes every
-// thread within reach of an end sums them for itself (a warp holds one
-// segment, so the others skip it); on the contiguous axis the end segments
-// alone have them, from their own inflow.
-template <int R, int BC, bool CONTIG>
-__device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, double &a, double &b, double &r0, double &r1)
+// Inflow of this segment, a w_k + b d^(len-k), and the right sides r_0, r_1 of
+// the boundary terms, from the segments' e (its zero-inflow y at its last
+// point, already in E) and g0 (zero-inflow g at its first).  Sums over a wide
+// window first double the block each slot holds (A.dbl times), then run over
+// the blocks.  Every thread of the CTA calls it.
+template <int BC>
+__device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, double e, double g0, double &a, double &b,
+                                           double &r0, double &r1)
 {
-    const int G = A.G, m = c.seg;
-    const int J = A.win < G ? A.win : G;
-    const double *E = c.E, *Gs = c.G;
-    auto slot = [&](int l) { return c.t0 + l * c.st; };
-    auto pl = [&](int l) -> double { return l == G - 1 ? A.dRl : A.dR; };
-    double yin = 0.0, gin = 0.0;
-    r0 = r1 = 0.0;
+    const int G = A.G, m = c.seg, t = c.t;
+    const double *cur = c.E;
+    double *nxt = c.first;
+    double yin = 0.0, gin = 0.0, h = 0.0;
+    for (int k = 0; k < A.dbl; ++k) {
+        if (c.live) nxt[t] = m >= 1 << k ? fma(A.pd[k], cur[t - (c.st << k)], cur[t]) : cur[t];
+        __syncthreads();
+        cur = nxt;
+        nxt = nxt == c.E ? c.first : c.E;
+    }
+    if (c.live)
+        for (int j = min(A.blocks - 1, (m - 1) >> A.dbl); j >= 0; --j)
+            yin = fma(A.pB, yin, cur[t - (1 + (j << A.dbl)) * c.st]);
     if (BC == BC_PERIODIC) {
-        // J segments back, farthest first; then J segments on
-        int l = m - J;
-        if (l < 0) l += G;
-        for (int j = 0; j < J; ++j) {
-            yin = fma(pl(l), yin, E[slot(l)]);
-            l = l + 1 == G ? 0 : l + 1;
-        }
-        if (J == G) yin *= A.inv;
-        double Y = fma(pl(m), yin, E[c.t]), pr = 1.0;
-        l = m + 1 == G ? 0 : m + 1;
-        for (int j = 0; j < J; ++j) {
-            gin = fma(pr, fma(l == G - 1 ? A.wl[0] : A.w[0], Y, Gs[slot(l)]), gin);
-            Y = fma(pl(l), Y, E[slot(l)]);
-            pr *= pl(l);
-            l = l + 1 == G ? 0 : l + 1;
-        }
-        if (J == G) gin *= A.inv;
+        // what the line's last point hands to its first, all images
+        if (c.live && c.last) c.ends[c.line] = A.inv * fma(A.dRl, yin, e);
+        __syncthreads();
+        if (c.live && m < A.win) yin = fma(c.ends[c.line], A.dpow[c.a], yin);
+    }
+    if (c.live) {
+        h = fma(c.last ? A.wl[0] : A.w[0], yin, g0);
+        c.G[t] = h;
+    }
+    __syncthreads();
+    cur = c.G;
+    nxt = c.E;
+    for (int k = 0; k < A.dbl; ++k) {
+        if (c.live) nxt[t] = m + (1 << k) < G ? fma(A.pd[k], cur[t + (c.st << k)], cur[t]) : cur[t];
+        __syncthreads();
+        cur = nxt;
+        nxt = nxt == c.E ? c.G : c.E;
+    }
+    if (c.live)
+        for (int j = min(A.blocks - 1, (G - 2 - m) >> A.dbl); j >= 0; --j)
+            gin = fma(A.pB, gin, cur[t + (1 + (j << A.dbl)) * c.st]);
+    if (BC == BC_PERIODIC) {
+        if (c.live && m == 0) c.ends[c.C + c.line] = A.inv * fma(c.last ? A.dRl : A.dR, gin, h);
+        __syncthreads();
+        if (c.live && G - 1 - m < A.win) gin = fma(c.ends[c.C + c.line], A.dpow[c.last ? 0 : A.n - c.a - A.R], gin);
     } else {
-        for (int l = max(m - J, 0); l < m; ++l) yin = fma(A.dR, yin, E[slot(l)]);
-        double Y = fma(A.dR, yin, E[c.t]), pr = 1.0;
-        for (int l = m + 1; l <= min(m + J, G - 1); ++l) {
-            gin = fma(pr, fma(l == G - 1 ? A.wl[0] : A.w[0], Y, Gs[slot(l)]), gin);
-            Y = fma(A.dR, Y, E[slot(l)]);
-            pr *= A.dR;
-        }
-        if (CONTIG) {
-            if (m == 0) r0 = fma(-A.rho, c.ends[c.line], -fma(c.last ? A.dRl : A.dR, gin, Gs[c.t]));
-            if (c.last) r1 = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, yin, E[c.t]));
-        } else {
-            const bool all = A.win >= G;
-            if (all || m < A.win) {
-                double Yl = 0.0, pw = 1.0, g0 = 0.0;
-                for (int l = 0; l < min(J + 1, G); ++l) {
-                    g0 = fma(pw, fma(l == G - 1 ? A.wl[0] : A.w[0], Yl, Gs[slot(l)]), g0);
-                    Yl = fma(A.dR, Yl, E[slot(l)]);
-                    pw *= A.dR;
-                }
-                r0 = fma(-A.rho, c.ends[c.line], -g0);
-            }
-            if (all || G - 1 - m < A.win) {
-                double Yl = 0.0;
-                for (int l = max(G - 1 - J, 0); l < G - 1; ++l) Yl = fma(A.dR, Yl, E[slot(l)]);
-                r1 = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, Yl, E[slot(G - 1)]));
-            }
+        double *v = c.ends + 2 * c.C + c.line;
+        if (c.live && m == 0) v[0] = fma(-A.rho, c.ends[c.line], -fma(c.last ? A.dRl : A.dR, gin, h));
+        if (c.live && c.last) v[c.C] = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, yin, e));
+        __syncthreads();
+        if (c.live) {
+            r0 = v[0];
+            r1 = v[c.C];
         }
     }
     a = yin;
@@ -188,12 +194,13 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
 }
 
 // z: s on entry, rho s + T^{-1} s (with the boundary terms) on exit.  Every
-// thread of the CTA calls it (one barrier; two on a contiguous Dirichlet axis).
-template <int R, int BC, bool CONTIG>
+// thread of the CTA calls it.
+template <int R, int BC>
 __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, const F64Seg &c)
 {
     const double d = A.d;
     const int L = A.len_last;
+    double e = 0.0;
     if (c.live) {
         if (BC == BC_DIRICHLET) {
             if (c.seg == 0) {
@@ -212,7 +219,7 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
         for (int k = 0; k < R; ++k) c.s[k * c.ss] = z[k];
 #pragma unroll
         for (int k = 1; k < R; ++k) z[k] = fma(d, z[k - 1], z[k]);
-        double e = z[R - 1];
+        e = z[R - 1];
         if (c.tail) {                                  // y ends with the line
             e = f64_pick<R>(z, L - 1);
 #pragma unroll
@@ -221,21 +228,10 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
 #pragma unroll
         for (int k = R - 2; k >= 0; --k) z[k] = fma(d, z[k + 1], z[k]);
         c.E[c.t] = e;
-        c.G[c.t] = z[0];
     }
     __syncthreads();
     double a = 0.0, b = 0.0, r0 = 0.0, r1 = 0.0;
-    if (c.live) f64_inflow<R, BC, CONTIG>(A, c, a, b, r0, r1);
-    if (CONTIG && BC == BC_DIRICHLET) {
-        double *v = c.ends + 2 * c.C + c.line;
-        if (c.live && c.seg == 0) v[0] = r0;
-        if (c.live && c.last) v[c.C] = r1;
-        __syncthreads();
-        if (c.live) {
-            r0 = v[0];
-            r1 = v[c.C];
-        }
-    }
+    f64_inflow<BC>(A, c, e, z[0], a, b, r0, r1);
     if (c.live) {
         if (BC == BC_DIRICHLET) {
             // the boundary terms in the segments they reach: of both ends
@@ -246,13 +242,12 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
                 r1 = (r1 - A.mu * r0) * A.inv;
                 r0 = t0;
             }
-            const int a0 = c.seg * R;
             if (all || c.seg < A.win) {
-                const double t0 = r0 * A.dpow[a0];
+                const double t0 = r0 * A.dpow[c.a];
                 a = fma(t0, A.e1, a);
                 b = fma(t0, c.last ? A.dRl : A.dR, b);
             }
-            if (all || A.G - 1 - c.seg < A.win) b = fma(r1 * A.dpow[A.n - a0 - (c.last ? L : R)], A.id, b);
+            if (all || A.G - 1 - c.seg < A.win) b = fma(r1 * A.dpow[A.n - c.a - (c.last ? L : R)], A.id, b);
         }
 #pragma unroll
         for (int k = 0; k < R; ++k) z[k] = fma(A.rho, c.s[k * c.ss], z[k]);
@@ -359,6 +354,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
     const int T = blockDim.x, t = threadIdx.x, n = A.n, G = A.G;
     double *first = sm64 + 2 * T, *last = sm64 + 3 * T, *sbuf = sm64 + 4 * T + 4 * LS.C;
     F64Seg c;
+    c.first = first;
     c.E = sm64;
     c.G = sm64 + T;
     c.ends = sm64 + 4 * T;
@@ -381,7 +377,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
     }
     c.last = c.seg == G - 1;
     c.tail = c.last && A.len_last < R;
-    const int a = c.seg * R, len = c.last ? A.len_last : R;
+    const int a = c.a = c.seg * R, len = c.last ? A.len_last : R;
     const int64_t line = (int64_t)blockIdx.x * LS.C + c.line;
     const bool io = c.live && line < LS.nlines;
     const int64_t st = CONTIG ? 1 : LS.stride;
@@ -421,7 +417,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
     if (KM == 0) {
         for (int q = 0; q < p.P; ++q) {
             if (q > 0) exchange_sdiff();
-            f64_solve<R, BC, CONTIG>(z, A, c);
+            f64_solve<R, BC>(z, A, c);
             if (p.out[q] != nullptr && io) {
                 if (p.scaled >> q & 1u) {              // the last power of mol_apply_D
                     const double sc = p.scale[q];
@@ -467,7 +463,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
                     for (int k = 0; k < R; ++k) z[k] = fma(w, r[k * T], z[k]);
                 }
             }
-            f64_solve<R, BC, CONTIG>(z, A, c);
+            f64_solve<R, BC>(z, A, c);
             zero = false;
         }
         if (!io) continue;
