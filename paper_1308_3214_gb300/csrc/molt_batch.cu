@@ -11,6 +11,7 @@
 #include "molt.h"
 #include "molt_internal.h"
 #include "molt_batch.cuh"
+#include "molt_f64.cuh"
 
 using namespace molt;
 
@@ -31,12 +32,16 @@ struct mol_batch_ctx {
     int nitems_y = 0;
     std::vector<int64_t> uoff;          // packed user layout: nprob + 1 prefix sums
     std::vector<BatchProb> hp;          // host copy of the problem table
+    std::vector<double> nu;             // alpha h of its x and y axes, two per problem
     BatchProb *probs = nullptr;
     int *row_prob = nullptr;
     int2 *items = nullptr;
     long long *uoff_dev = nullptr;
     double *dp64 = nullptr;
     float *dp32 = nullptr;
+    F64Task *f64_tasks = nullptr;        // float64: the line passes' constants and work lists
+    int2 *f64_items = nullptr;
+    std::vector<F64BatchClass> f64_classes[2];
     BLevel lev[3];
     double *io[2] = {nullptr, nullptr};  // packed float64 fields of mol_batch_solve_host
     long long *irec = nullptr;           // receivers in the internal layout, then their distinct
@@ -62,12 +67,14 @@ struct mol_batch_ctx {
     int64_t one_warp_end() const { return xmid ? rows_small : rows_mid; }
     int y_launches() const
     {
+        if (tbytes == 8) return (int)f64_classes[1].size();
         int n = 0;
         for (int k = 0; k < 4; ++k) n += ycls_count[k] > 0 ? 1 : 0;
         return n;
     }
     int x_launches() const
     {
+        if (tbytes == 8) return (int)f64_classes[0].size();
         return (one_warp_end() > 0 ? 1 : 0) + ((xmid && rows_mid > rows_small) ? 1 : 0) + (nrows > rows_mid ? 1 : 0);
     }
     int smem_sm = 228 * 1024, smem_blk = 227 * 1024;
@@ -408,6 +415,41 @@ cudaError_t launch_pass_x(mol_batch_ctx *b, BatchPass bp, cudaStream_t s)
     return e;
 }
 
+// A float64 pass: one launch per class, the first on s, the others over side
+// streams forked from s and joined back into it.
+cudaError_t launch_pass_f64(mol_batch_ctx *b, int axis, bool adj, const BatchPass &x, cudaStream_t s)
+{
+    F64BatchPass bp{};
+    bp.tasks = b->f64_tasks;
+    bp.items = b->f64_items;
+    bp.u = (const double *)x.pr.u_hi;
+    bp.up = (const double *)x.pr.up_hi;
+    bp.un = (double *)x.pr.un_hi;
+    for (int k = 0; k < b->Pmax; ++k) {
+        bp.g[k] = (const double *)x.pr.g[k];
+        bp.out[k] = (double *)x.pr.out[k];
+    }
+    bp.ea = x.pr.ea; bp.eb = x.pr.eb; bp.ec = x.pr.ec;
+    const std::vector<F64BatchClass> &cls = b->f64_classes[axis];
+    const int nside = std::min<int>(3, (int)cls.size() - 1);
+    cudaError_t e = cudaSuccess;
+    if (nside > 0) {
+        for (int j = 0; j < nside && e == cudaSuccess; ++j)
+            if (!b->ys[j]) e = cudaStreamCreateWithFlags(&b->ys[j], cudaStreamNonBlocking);
+        for (int j = 0; j <= nside && e == cudaSuccess; ++j)
+            if (!b->yev[j]) e = cudaEventCreateWithFlags(&b->yev[j], cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(b->yev[0], s);
+        for (int j = 0; j < nside && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(b->ys[j], b->yev[0], 0);
+    }
+    for (size_t c = 0; c < cls.size() && e == cudaSuccess; ++c)
+        e = launch_f64_batch(axis, adj, cls[c], bp, c == 0 ? s : b->ys[(c - 1) % nside]);
+    for (int j = 0; j < nside && e == cudaSuccess; ++j) {
+        e = cudaEventRecord(b->yev[1 + j], b->ys[j]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->yev[1 + j], 0);
+    }
+    return e;
+}
+
 template <class T>
 cudaError_t set_kernel_smem(const mol_batch_ctx *b)
 {
@@ -441,13 +483,9 @@ mol_status run_pass(mol_batch_ctx *b, int axis, const BatchPass &bp, cudaStream_
         BCK(cudaEventRecord(e0, s), "event record");
     }
     cudaError_t e;
-    if (axis == 1) {
-        if (adj) e = b->tbytes == 4 ? launch_pass_y<float, true>(b, bp, s) : launch_pass_y<double, true>(b, bp, s);
-        else e = b->tbytes == 4 ? launch_pass_y<float, false>(b, bp, s) : launch_pass_y<double, false>(b, bp, s);
-    } else {
-        if (adj) e = b->tbytes == 4 ? launch_pass_x<float, true>(b, bp, s) : launch_pass_x<double, true>(b, bp, s);
-        else e = b->tbytes == 4 ? launch_pass_x<float, false>(b, bp, s) : launch_pass_x<double, false>(b, bp, s);
-    }
+    if (b->tbytes == 8) e = launch_pass_f64(b, axis, adj, bp, s);
+    else if (axis == 1) e = adj ? launch_pass_y<float, true>(b, bp, s) : launch_pass_y<float, false>(b, bp, s);
+    else e = adj ? launch_pass_x<float, true>(b, bp, s) : launch_pass_x<float, false>(b, bp, s);
     if (e != cudaSuccess) return bcuda(b, e, "batched pass launch");
     b->launches += (axis == 1) ? b->y_launches() : b->x_launches();
     if (b->timing) {
@@ -656,13 +694,13 @@ mol_status build_graph(mol_batch_ctx *b)
     if (b->gexec) return MOL_OK;
     if (!b->cap_stream) BCK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking), "stream create");
     int ych[3], xch[3], nch = 0;
-    const bool chains = b->chains && chain_plan(b, ych, xch, nch);
+    const bool chains = b->tbytes == 4 && b->chains && chain_plan(b, ych, xch, nch);
     cudaGraph_t g = nullptr;
     BCK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal), "graph capture begin");
     const int64_t before = b->launches;
     mol_status st = MOL_OK;
     if (chains) {
-        st = b->tbytes == 4 ? capture_chains<float>(b, ych, xch, nch) : capture_chains<double>(b, ych, xch, nch);
+        st = capture_chains<float>(b, ych, xch, nch);
     } else {
         for (int k = 0; k < 3 && st == MOL_OK; ++k)
             st = run_update(b, b->lev[(k + 1) % 3], b->lev[k % 3], b->lev[(k + 2) % 3], 2.0, -1.0, 1.0, b->cap_stream);
@@ -693,6 +731,7 @@ mol_status plan_batch(mol_batch_ctx *b, int nprob, const mol_grid *grids, const 
                       const double *beta, const int *P, int quad)
 {
     b->hp.assign(nprob, BatchProb{});
+    b->nu.assign(2 * (size_t)nprob, 0.0);
     b->uoff.assign(nprob + 1, 0);
     int64_t off = 0, rows = 0, items = 0;
     b->rows_small = 0;
@@ -720,6 +759,8 @@ mol_status plan_batch(mol_batch_ctx *b, int nprob, const mol_grid *grids, const 
         const double alpha = bt / (c[i] * dt[i]);                       // eq. L_def
         const double nux = alpha * (g.hi[0] - g.lo[0]) / (double)(nx - 1);
         const double nuy = alpha * (g.hi[1] - g.lo[1]) / (double)(ny - 1);
+        b->nu[2 * i] = nux;
+        b->nu[2 * i + 1] = nuy;
         axis_constants(nux, nx, BC_DIRICHLET, quad, pb.ax);
         axis_constants(nuy, ny, BC_DIRICHLET, quad, pb.ay);
         pb.rpt_x = pick_rpt_x(nx);
@@ -857,6 +898,26 @@ mol_status mol_batch_create(int nprob, const mol_grid *grids, const double *c, c
             goto bad;
         }
     }
+    if (b->tbytes == 8) {
+        std::vector<F64BatchGrid> g(nprob);
+        for (int i = 0; i < nprob; ++i) {
+            const BatchProb &pb = b->hp[i];
+            g[i] = F64BatchGrid{&pb.ax, &pb.ay, b->nu[2 * i], b->nu[2 * i + 1], pb.P, pb.pitch, BMAXP, pb.off, pb.cu,
+                                &pb.coef[0][0]};
+        }
+        F64BatchLists l;
+        f64_batch_plan(g.data(), nprob, b->quad, b->num_sms, l);
+        for (int a = 0; a < 2; ++a) b->f64_classes[a] = l.classes[a];
+        if ((st = balloc(b, (void **)&b->f64_tasks, sizeof(F64Task) * l.tasks.size())) != MOL_OK) goto bad;
+        if ((st = balloc(b, (void **)&b->f64_items, sizeof(int2) * l.items.size())) != MOL_OK) goto bad;
+        if ((e = cudaMemcpy(b->f64_tasks, l.tasks.data(), sizeof(F64Task) * l.tasks.size(), cudaMemcpyHostToDevice)) !=
+                cudaSuccess ||
+            (e = cudaMemcpy(b->f64_items, l.items.data(), sizeof(int2) * l.items.size(), cudaMemcpyHostToDevice)) !=
+                cudaSuccess) {
+            st = bcuda(b, e, "work list upload");
+            goto bad;
+        }
+    }
     {
         const size_t plane = (size_t)b->tbytes * b->total_int;
         for (int k = 0; k < 3; ++k) {
@@ -887,7 +948,7 @@ mol_status mol_batch_create(int nprob, const mol_grid *grids, const double *c, c
         b->cgrid = (int)std::min<int64_t>((b->nrows + 7) / 8, 8 * (int64_t)b->num_sms);
         // (rows of up to 1024 points: 8 chunks of 128 each)
         b->cgrid_y = (int)std::max<int64_t>(1, std::min<int64_t>(8, 8 * (int64_t)b->num_sms / b->cgrid));
-        e = b->tbytes == 4 ? set_kernel_smem<float>(b) : set_kernel_smem<double>(b);
+        e = b->tbytes == 4 ? set_kernel_smem<float>(b) : configure_f64_batch_kernels();
         if (e != cudaSuccess) { st = bcuda(b, e, "kernel attributes"); goto bad; }
     }
     *out = b;
@@ -1112,6 +1173,12 @@ mol_status mol_batch_autotune(mol_batch b, void *stream)
         if ((st = zero_level(b, b->lev[k], s)) != MOL_OK) return st;
     const int64_t launches0 = b->launches;
     double t[2];
+    if (b->tbytes == 8) {                              // the float64 passes pick their own shapes
+        if ((st = batch_pass_ms(b, s, t)) != MOL_OK) return st;
+        for (int a = 0; a < 2; ++a) b->tune_ms[a] = t[a];
+        b->launches = launches0;
+        return MOL_OK;
+    }
     // warps per CTA of each x launch (the other held; long rows also split
     // over two warps, W = 0 below), then the y segment rule
     auto upload = [&]() {

@@ -1,6 +1,7 @@
 // molt_f64.cu -- instantiation, launch shapes and constants of the float64
 // line passes (molt_f64.cuh).
 #include <algorithm>
+#include <map>
 #include <cmath>
 #include "molt_internal.h"
 #include "molt_f64.cuh"
@@ -98,6 +99,23 @@ cudaError_t attr_f64_r()
     return e == cudaSuccess ? attr_f64<32, BC, KM>() : e;
 }
 
+template <int KM, bool CONTIG, bool ADJ>
+const void *batch_kernel(int R)
+{
+    switch (R) {
+    case 4: return (const void *)k_f64_batch<4, KM, CONTIG, ADJ>;
+    case 8: return (const void *)k_f64_batch<8, KM, CONTIG, ADJ>;
+    case 16: return (const void *)k_f64_batch<16, KM, CONTIG, ADJ>;
+    default: return (const void *)k_f64_batch<32, KM, CONTIG, ADJ>;
+    }
+}
+
+const void *batch_kernel(int axis, bool adj, int R)
+{
+    if (axis == 0) return adj ? batch_kernel<1, true, true>(R) : batch_kernel<1, true, false>(R);
+    return adj ? batch_kernel<0, false, true>(R) : batch_kernel<0, false, false>(R);
+}
+
 }  // namespace
 
 double f64_kappa(double nu, int quad)
@@ -175,11 +193,95 @@ cudaError_t launch_f64(int bc, bool contig, const F64Plan &pl, double nu, int qu
         p.vec = (bits & 31) == 0;
     }
     const F64Axis A = f64_axis(nu, quad, bc, pl.R, ax);
-    F64Lines L{stride, inner, nlines, pl.C, 0};
+    F64Lines L{stride, inner, nlines, ax.n, pl.C, 0};
     while ((1 << L.cshift) < pl.C) ++L.cshift;
     if (bc == BC_PERIODIC)
         return horner ? run_f64_r<BC_PERIODIC, 1>(contig, pl, A, L, p, s) : run_f64_r<BC_PERIODIC, 0>(contig, pl, A, L, p, s);
     return horner ? run_f64_r<BC_DIRICHLET, 1>(contig, pl, A, L, p, s) : run_f64_r<BC_DIRICHLET, 0>(contig, pl, A, L, p, s);
+}
+
+// Tasks and work lists of a batch's passes: the shape of each problem's lines
+// as f64_plan picks it with the batch's points behind it, grouped by segment
+// length and CTA size (rounded up to 64 threads), the longest programs first.
+void f64_batch_plan(const F64BatchGrid *probs, int nprob, int quad, int sms, F64BatchLists &out)
+{
+    int64_t points = 0;
+    for (int i = 0; i < nprob; ++i) points += (int64_t)probs[i].ax->n * probs[i].ay->n;
+    out.tasks.assign(2 * (size_t)nprob, F64Task{});
+    out.items.clear();
+    for (int axis = 0; axis < 2; ++axis) {
+        const bool contig = axis == 0;
+        std::map<std::pair<int, int>, std::vector<int>> groups;
+        for (int i = 0; i < nprob; ++i) {
+            const F64BatchGrid &g = probs[i];
+            const AxisDev &A = contig ? *g.ax : *g.ay;
+            const int64_t lines = contig ? g.ay->n : g.ax->n;
+            const double nu = contig ? g.nux : g.nuy;
+            F64Plan pl{};
+            f64_plan(A.n, std::max(lines, points / A.n), contig, contig, nu, sms, &pl);
+            F64Task &t = out.tasks[(size_t)axis * nprob + i];
+            t.A = f64_axis(nu, quad, BC_DIRICHLET, pl.R, A);
+            t.L = F64Lines{contig ? 1 : (int64_t)g.pitch, lines, lines, g.pitch, pl.C, 0};
+            while ((1 << t.L.cshift) < pl.C) ++t.L.cshift;
+            t.off = g.off;
+            t.p.P = g.P;
+            t.p.vec = contig;                          // rows start on 32 bytes and are padded to 4 points
+            if (contig) {
+                t.p.ng = g.P;
+                t.p.nout = 1;
+                t.p.epi = 1;
+                // in the units of the powers: kappa per application of either axis' D
+                const double kx = f64_kappa(g.nux, quad), ky = f64_kappa(g.nuy, quad);
+                double ux = 1.0;
+                for (int q = 0; q <= g.P; ++q, ux *= kx) {
+                    double ug = ky;
+                    for (int k = 0; k < g.P; ++k, ug *= ky) {
+                        t.p.coef[0][q][k] = g.coef[q * g.ldc + k] * ux * ug;
+                        if (t.p.coef[0][q][k] != 0.0) t.p.add[0][q] |= 1u << k;
+                    }
+                    t.p.cu[0][q] = g.cu[q] * ux;
+                    if (t.p.cu[0][q] != 0.0) t.p.ucu[0] |= 1u << q;
+                }
+            }
+            groups[{pl.R, (pl.threads + 63) / 64 * 64}].push_back(i);
+        }
+        out.classes[axis].clear();
+        for (auto &g : groups) {
+            F64BatchClass c{g.first.first, g.first.second, 0, (int)out.items.size(), 0};
+            std::stable_sort(g.second.begin(), g.second.end(), [&](int a, int b) { return probs[a].P > probs[b].P; });
+            for (int i : g.second) {
+                const F64Task &t = out.tasks[(size_t)axis * nprob + i];
+                c.smem = std::max(c.smem, sizeof(double) * f64_task_words() + f64_smem(c.threads, t.L.C, c.R, contig));
+                for (int64_t l = 0; l < t.L.nlines; l += t.L.C)
+                    out.items.push_back(make_int2(axis * nprob + i, (int)(l / t.L.C)));
+            }
+            c.count = (int)out.items.size() - c.begin;
+            out.classes[axis].push_back(c);
+        }
+        // the class with the most threads first (it runs on the caller's stream)
+        std::sort(out.classes[axis].begin(), out.classes[axis].end(), [](const F64BatchClass &a, const F64BatchClass &b) {
+            return (int64_t)a.count * a.threads > (int64_t)b.count * b.threads;
+        });
+    }
+}
+
+cudaError_t launch_f64_batch(int axis, bool adj, const F64BatchClass &c, F64BatchPass bp, cudaStream_t s)
+{
+    bp.items += c.begin;
+    void *args[] = {&bp};
+    return cudaLaunchKernel(batch_kernel(axis, adj, c.R), dim3((unsigned)c.count), dim3((unsigned)c.threads), args, c.smem, s);
+}
+
+cudaError_t configure_f64_batch_kernels()
+{
+    for (int axis = 0; axis < 2; ++axis)
+        for (int adj = 0; adj < 2; ++adj)
+            for (int R = 4; R <= kF64MaxR; R *= 2) {
+                const cudaError_t e = cudaFuncSetAttribute(batch_kernel(axis, adj != 0, R),
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+                if (e != cudaSuccess) return e;
+            }
+    return cudaSuccess;
 }
 
 cudaError_t configure_f64_kernels()

@@ -61,6 +61,7 @@
 // 3000 -> 2150, z 746 -> 496.
 #pragma once
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 #include "molt_kernels.cuh"
 
@@ -68,6 +69,7 @@ namespace molt {
 
 constexpr int kF64MaxR = 32;
 constexpr int kF64Threads = 256;       // threads per CTA at most
+constexpr int kF64BatchP = 5;          // highest order of a batched problem
 
 // Constants of one axis for segments of R points (host, molt_f64.cu).
 struct F64Axis {
@@ -88,6 +90,7 @@ struct F64Axis {
 
 struct F64Lines {
     int64_t stride, inner, nlines;
+    int64_t pitch;         // contiguous axis: from one line to the next
     int C, cshift;         // lines per CTA; log2 C (strided axes)
 };
 
@@ -95,22 +98,25 @@ struct F64Lines {
 // D^p u / kappa^p) or the Horner pass of HornerParams with its weights times
 // kappa^t.  Zero weights, unit scales and the level's weights are flagged by
 // the host (a comparison would cost the float64 pipe an operation).
-struct F64Prog {
+// NO, NF: outputs and fields it has room for.
+template <int NO, int NF>
+struct F64ProgT {
     int P, ng, nout, epi;
-    unsigned add[MAXP][MAXP];  // [o][t]: bit k set where field k has a weight
-    unsigned ucu[MAXP];        // [o]: bit t set where u has a weight in step t
+    unsigned add[NO][MAXP];    // [o][t]: bit k set where field k has a weight
+    unsigned ucu[NO];          // [o]: bit t set where u has a weight in step t
     unsigned scaled;           // bit p-1: scale[p-1] != 1
     bool hea, heb, hec;        // ea, eb != 0, ec != 1
     bool vec;                  // contiguous axis: every segment starts on 32 bytes
-    const double *g[MAXG];
-    double *out[MAXG];
-    double scale[MAXG];
-    double coef[MAXP][MAXP][MAXG];
-    double cu[MAXP][MAXP];
+    const double *g[NF];
+    double *out[NF];
+    double scale[NF];
+    double coef[NO][MAXP][NF];
+    double cu[NO][MAXP];
     double ea, eb, ec;
     const double *u, *up;
     double *un;
 };
+struct F64Prog : F64ProgT<MAXP, MAXG> {};
 
 // this thread's place on its line
 struct F64Seg {
@@ -136,7 +142,7 @@ __device__ __forceinline__ double f64_pick(const double (&z)[R], int k)
 // point, already in E) and g0 (zero-inflow g at its first).  Sums over a wide
 // window first double the block each slot holds (A.dbl times), then run over
 // the blocks.  Every thread of the CTA calls it.
-template <int BC>
+template <int BC, bool ADJ>
 __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, double e, double g0, double &a, double &b,
                                            double &r0, double &r1)
 {
@@ -181,8 +187,14 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
         if (c.live && G - 1 - m < A.win) gin = fma(c.ends[c.C + c.line], A.dpow[c.last ? 0 : A.n - c.a - A.R], gin);
     } else {
         double *v = c.ends + 2 * c.C + c.line;
-        if (c.live && m == 0) v[0] = fma(-A.rho, c.ends[c.line], -fma(c.last ? A.dRl : A.dR, gin, h));
-        if (c.live && c.last) v[c.C] = fma(-A.rho, c.ends[c.C + c.line], -fma(A.dRl, yin, e));
+        if (c.live && m == 0) {
+            const double g = fma(c.last ? A.dRl : A.dR, gin, h);
+            v[0] = ADJ ? -g : fma(-A.rho, c.ends[c.line], -g);
+        }
+        if (c.live && c.last) {
+            const double g = fma(A.dRl, yin, e);
+            v[c.C] = ADJ ? -g : fma(-A.rho, c.ends[c.C + c.line], -g);
+        }
         __syncthreads();
         if (c.live) {
             r0 = v[0];
@@ -195,7 +207,13 @@ __device__ __forceinline__ void f64_inflow(const F64Axis &A, const F64Seg &c, do
 
 // z: s on entry, rho s + T^{-1} s (with the boundary terms) on exit.  Every
 // thread of the CTA calls it.
-template <int R, int BC>
+// ADJ (Dirichlet): on the interior points the operator is D = kappa (rho +
+// S M) Delta, S the solve with zero ends, M = 1 but 1 - rho d at each of the
+// two points next to the ends (what s_0 := s_1 and s_{n-1} := s_{n-2} put
+// into rows 1 and n-2).  S is symmetric, so D^T = kappa Delta^T (rho + M S):
+// here z becomes rho z + M S z for z with its end values dropped, and Delta^T,
+// the second difference with zeros past the interior, follows at the caller.
+template <int R, int BC, bool ADJ>
 __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, const F64Seg &c)
 {
     const double d = A.d;
@@ -204,11 +222,11 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
     if (c.live) {
         if (BC == BC_DIRICHLET) {
             if (c.seg == 0) {
-                c.ends[c.line] = z[1];
+                if (!ADJ) c.ends[c.line] = z[1];
                 z[0] = 0.0;
             }
             // s_{n-2}: the last segment's, or the end of the one before it
-            if (L >= 2 ? c.last : c.seg == A.G - 2) c.ends[c.C + c.line] = f64_pick<R>(z, L >= 2 ? L - 2 : R - 1);
+            if (!ADJ && (L >= 2 ? c.last : c.seg == A.G - 2)) c.ends[c.C + c.line] = f64_pick<R>(z, L >= 2 ? L - 2 : R - 1);
         }
         if (c.last) {
             const int keep = BC == BC_DIRICHLET ? L - 1 : L;
@@ -231,7 +249,7 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
     }
     __syncthreads();
     double a = 0.0, b = 0.0, r0 = 0.0, r1 = 0.0;
-    f64_inflow<BC>(A, c, e, z[0], a, b, r0, r1);
+    f64_inflow<BC, ADJ>(A, c, e, z[0], a, b, r0, r1);
     if (c.live) {
         if (BC == BC_DIRICHLET) {
             // the boundary terms in the segments they reach: of both ends
@@ -257,6 +275,19 @@ __device__ __forceinline__ void f64_solve(double (&z)[R], const F64Axis &A, cons
         } else {
 #pragma unroll
             for (int k = 0; k < R; ++k) z[k] = fma(b, A.pw[R - k], fma(a, A.w[k], z[k]));
+        }
+        if constexpr (ADJ) {
+            const int km = L >= 2 ? L - 2 : R - 1;     // point n - 2 and its segment
+            const bool hm = L >= 2 ? c.last : c.seg == A.G - 2;
+            double g1 = 0.0, gm = 0.0;
+            if (c.seg == 0) g1 = fma(-A.rho, c.s[c.ss], z[1]);
+            if (hm) gm = fma(-A.rho, c.s[km * c.ss], f64_pick<R>(z, km));
+            if (c.seg == 0) z[1] = fma(-A.rho * A.d, g1, z[1]);
+            if (hm) {
+                const double v = fma(-A.rho * A.d, gm, f64_pick<R>(z, km));
+#pragma unroll
+                for (int k = 0; k < R; ++k) z[k] = k == km ? v : z[k];
+            }
         }
         if (BC == BC_DIRICHLET) {
             if (c.seg == 0) z[0] = 0.0;
@@ -346,11 +377,12 @@ __host__ __device__ inline size_t f64_smem(int threads, int C, int R, bool horne
     return sizeof(double) * ((size_t)threads * 4 + 4 * C + (size_t)R * threads * (horner ? 2 : 1));
 }
 
-template <int R, int BC, int KM, bool CONTIG>
-__global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ F64Axis A, F64Lines LS,
-                                                       const __grid_constant__ F64Prog p)
+// One CTA's lines, from block * C on.  ADJ: the transposed operators (the
+// adjoint step; Dirichlet, one output).  PAD: lines end in padding (zeros) up
+// to a multiple of 4 points, which vectors may read and write back as zeros.
+template <int R, int BC, int KM, bool CONTIG, bool ADJ, bool PAD, class Prog>
+__device__ __forceinline__ void f64_pass(const F64Axis &A, const F64Lines &LS, const Prog &p, int block, double *sm64)
 {
-    extern __shared__ __align__(16) double sm64[];
     const int T = blockDim.x, t = threadIdx.x, n = A.n, G = A.G;
     double *first = sm64 + 2 * T, *last = sm64 + 3 * T, *sbuf = sm64 + 4 * T + 4 * LS.C;
     F64Seg c;
@@ -378,10 +410,10 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
     c.last = c.seg == G - 1;
     c.tail = c.last && A.len_last < R;
     const int a = c.a = c.seg * R, len = c.last ? A.len_last : R;
-    const int64_t line = (int64_t)blockIdx.x * LS.C + c.line;
+    const int64_t line = (int64_t)block * LS.C + c.line;
     const bool io = c.live && line < LS.nlines;
     const int64_t st = CONTIG ? 1 : LS.stride;
-    const int64_t lbase = !io ? 0 : CONTIG ? line * n : (line % LS.inner) + (line / LS.inner) * LS.inner * (int64_t)n;
+    const int64_t lbase = !io ? 0 : CONTIG ? line * LS.pitch : (line % LS.inner) + (line / LS.inner) * LS.inner * (int64_t)n;
     const int64_t at = lbase + (int64_t)a * st;        // this segment's first point
 
     double z[R];
@@ -393,9 +425,9 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
             if (BC == BC_PERIODIC) return j < 0 ? j + n : (j >= n ? j - n : j);
             return j < 0 ? 0 : (j > n - 1 ? n - 1 : j);
         };
-        const double zl = p.u[lbase + row(a - 1) * st], zr = p.u[lbase + row(a + len) * st];
+        const double zl = ADJ ? 0.0 : p.u[lbase + row(a - 1) * st], zr = ADJ ? 0.0 : p.u[lbase + row(a + len) * st];
         f64_each<R, CONTIG>(p.u + at, st, len, p.vec, [&](int k, double v) { z[k] = v; });
-        f64_sdiff<R>(z, zl, zr, A, c);
+        if (!ADJ) f64_sdiff<R>(z, zl, zr, A, c);
     }
     // neighbours' values through shared memory, then the second difference
     auto exchange_sdiff = [&]() {
@@ -414,10 +446,22 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
         }
     };
 
+    auto apply = [&]() {                               // ADJ: D^T / kappa of z
+        f64_solve<R, BC, ADJ>(z, A, c);
+        if (ADJ) exchange_sdiff();
+    };
+    auto pad = [&]() {                                 // points past the line's end, before they are stored
+        if (PAD && CONTIG && c.tail) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) z[k] = k < len ? z[k] : 0.0;
+        }
+    };
+
     if (KM == 0) {
         for (int q = 0; q < p.P; ++q) {
-            if (q > 0) exchange_sdiff();
-            f64_solve<R, BC>(z, A, c);
+            if (!ADJ && q > 0) exchange_sdiff();
+            apply();
+            if (ADJ) pad();
             if (p.out[q] != nullptr && io) {
                 if (p.scaled >> q & 1u) {              // the last power of mol_apply_D
                     const double sc = p.scale[q];
@@ -453,17 +497,17 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
             const double w = p.cu[o][q];
             if (zero) {
                 if (!(p.ucu[o] >> q & 1u)) continue;
-                __syncthreads();                   // the slots' last readers are done
+                if (!ADJ) __syncthreads();         // the slots' last readers are done
 #pragma unroll
                 for (int k = 0; k < R; ++k) z[k] = w * r[k * T];
             } else {
-                exchange_sdiff();
+                if (!ADJ) exchange_sdiff();
                 if (p.ucu[o] >> q & 1u) {
 #pragma unroll
                     for (int k = 0; k < R; ++k) z[k] = fma(w, r[k * T], z[k]);
                 }
             }
-            f64_solve<R, BC>(z, A, c);
+            apply();
             zero = false;
         }
         if (!io) continue;
@@ -476,8 +520,95 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
             if (p.hea) f64_each<R, CONTIG>(p.u + at, st, len, p.vec, [&](int k, double v) { z[k] = fma(p.ea, v, z[k]); });
             if (p.heb) f64_each<R, CONTIG>(p.up + at, st, len, p.vec, [&](int k, double v) { z[k] = fma(p.eb, v, z[k]); });
         }
+        pad();
         f64_store<R, CONTIG>((p.epi ? p.un : p.out[o]) + at, st, len, p.vec, z);
     }
+}
+
+template <int R, int BC, int KM, bool CONTIG>
+__global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ F64Axis A, F64Lines LS,
+                                                       const __grid_constant__ F64Prog p)
+{
+    extern __shared__ __align__(16) double sm64[];
+    f64_pass<R, BC, KM, CONTIG, false, false>(A, LS, p, (int)blockIdx.x, sm64);
+}
+
+// The same passes over the problems of a batch (Dirichlet): a CTA looks its
+// problem up in the work list and copies the problem's constants (1.8 KB) to
+// shared memory in front of the pass's own; one launch per segment length and
+// CTA size.  The constants cost shared-memory loads instead of constant operands,
+// which the float64 pipe hides.  Warps beyond the problem's lines leave.
+// Measured against the earlier batch passes (13 operations an application, a warp
+// per row, three exchanges per column): 100 problems of 64..256 points, 9 steps,
+// 5379 -> 4260 us; 4 problems, 1337 -> 879; gradient on 131 x 160, P = 2 (one problem,
+// 80 steps), 6861 -> 2912, on 500 x 301 3074 -> 1972.
+struct F64Task {
+    F64Axis A;
+    F64Lines L;
+    F64ProgT<1, kF64BatchP> p;  // its pointers: from the launch, off elements on
+    long long off;
+};
+
+struct F64BatchPass {
+    const F64Task *tasks;
+    const int2 *items;          // (task, group of C lines)
+    const double *u, *up, *g[kF64BatchP];
+    double *un, *out[kF64BatchP];
+    double ea, eb, ec;
+};
+
+// A problem of a batch as the plan needs it; coef rows are ldc apart.
+struct F64BatchGrid {
+    const AxisDev *ax, *ay;
+    double nux, nuy;
+    int P, pitch, ldc;
+    long long off;
+    const double *cu, *coef;
+};
+struct F64BatchClass {
+    int R, threads;
+    size_t smem;
+    int begin, count;           // of the work list
+};
+struct F64BatchLists {
+    std::vector<F64Task> tasks; // x passes, then y passes
+    std::vector<int2> items;
+    std::vector<F64BatchClass> classes[2];
+};
+void f64_batch_plan(const F64BatchGrid *probs, int nprob, int quad, int sms, F64BatchLists &out);
+cudaError_t launch_f64_batch(int axis, bool adj, const F64BatchClass &c, F64BatchPass bp, cudaStream_t s);
+cudaError_t configure_f64_batch_kernels();
+
+__host__ __device__ constexpr int f64_task_words() { return (int)((sizeof(F64Task) + 15) / 16 * 2); }
+
+template <int R, int KM, bool CONTIG, bool ADJ>
+__global__ void __launch_bounds__(kF64Threads, 2) k_f64_batch(const __grid_constant__ F64BatchPass bp)
+{
+    extern __shared__ __align__(16) double sm64[];
+    static_assert(sizeof(F64Task) % 8 == 0, "copied in words");
+    F64Task &k = *reinterpret_cast<F64Task *>(sm64);
+    const int2 item = bp.items[blockIdx.x];
+    {
+        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(bp.tasks + item.x);
+        unsigned long long *dst = reinterpret_cast<unsigned long long *>(sm64);
+        for (int i = threadIdx.x; i < (int)(sizeof(F64Task) / 8); i += blockDim.x) dst[i] = __ldg(src + i);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        k.p.u = bp.u + k.off;
+        k.p.up = bp.up + k.off;
+        k.p.un = bp.un + k.off;
+        for (int q = 0; q < k.p.P; ++q) {
+            k.p.g[q] = bp.g[q] + k.off;
+            k.p.out[q] = bp.out[q] + k.off;
+        }
+        k.p.ea = bp.ea; k.p.eb = bp.eb; k.p.ec = bp.ec;
+        k.p.hea = bp.ea != 0.0; k.p.heb = bp.eb != 0.0; k.p.hec = bp.ec != 1.0;
+    }
+    __syncthreads();
+    // (strided axes pad the threads of a line's C columns only: C G threads work)
+    if ((int)(threadIdx.x & ~31u) >= k.L.C * k.A.G) return;
+    f64_pass<R, BC_DIRICHLET, KM, CONTIG, ADJ, true>(k.A, k.L, k.p, item.y, sm64 + f64_task_words());
 }
 
 }  // namespace molt
