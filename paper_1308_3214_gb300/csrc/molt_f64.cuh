@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
 // which the float64 pipe hides.  Warps beyond the problem's lines leave.
 // Measured against the earlier batch passes (13 operations an application, a warp
 // per row, three exchanges per column): 100 problems of 64..256 points, 9 steps,
-// 5379 -> 4260 us; 4 problems, 1337 -> 879; gradient on 131 x 160, P = 2 (one problem,
+// 5379 -> 2958 us; 4 problems, 1337 -> 796; gradient on 131 x 160, P = 2 (one problem,
 // 80 steps), 6861 -> 2912, on 500 x 301 3074 -> 1972.
 struct F64Task {
     F64Axis A;

@@ -150,7 +150,10 @@ double f64_kappa(double nu, int quad);
 void f64_inflow_weights(double nu, int len, double *w);
 void f64_inverse_decay(double d, double om2, double &e1, double &id);
 bool f64_axis_ok(int n, bool contig);
-bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sms, F64Plan *out);
+// rmax, tmax: segment length and threads per CTA at most (more threads only
+// where the fewest lines need them)
+bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sms, F64Plan *out, int rmax = 32,
+              int tmax = 256);
 cudaError_t launch_f64(int bc, bool contig, const F64Plan &pl, double nu, int quad, const AxisDev &ax, int64_t stride,
                        int64_t inner, int64_t nlines, bool horner, F64Prog p, cudaStream_t s);
 cudaError_t configure_f64_kernels();
