@@ -110,14 +110,6 @@ __device__ __forceinline__ void warp_copy(S *dst, const S *src, int lane)
 
 __device__ __forceinline__ float vfirst(const float4 &v) { return v.x; }
 __device__ __forceinline__ float vlast(const float4 &v) { return v.w; }
-__device__ __forceinline__ double vfirst(const double2 &v) { return v.x; }
-__device__ __forceinline__ double vlast(const double2 &v) { return v.y; }
-
-// second difference of 2 consecutive points given their outer neighbours
-__device__ __forceinline__ double2 sdiff2(const double2 &h, double hl, double hr)
-{
-    return make_double2((h.y - h.x) - (h.x - hl), (hr - h.y) - (h.y - h.x));
-}
 
 // ---------------------------------------------------------------------------
 // x pass: one row
@@ -222,8 +214,7 @@ __device__ __forceinline__ void batch_row(const BatchProb &pb, const ProgParams 
                             for (int cc = 0; cc < VN; ++cc) e[cc] += lo4[cc];
                         }
                     } else {
-                        if constexpr (pair) r = sdiff4(h[i], l[i], hl, ll, hr, lr);
-                        else r = sdiff2(h[i], hl, hr);
+                        r = sdiff4(h[i], l[i], hl, ll, hr, lr);
                         if (v == 0) r.x = r.y;         // Dirichlet: the end node takes the interior centre
                     }
                     *reinterpret_cast<V *>(R + St::pos(VN * v)) = r;
@@ -424,8 +415,7 @@ __device__ __forceinline__ void batch_row_split(const BatchProb &pb, const ProgP
                             for (int cc = 0; cc < VN; ++cc) e[cc] += lo4[cc];
                         }
                     } else {
-                        if constexpr (pair) r = sdiff4(h[i], l[i], hl, ll, hr, lr);
-                        else r = sdiff2(h[i], hl, hr);
+                        r = sdiff4(h[i], l[i], hl, ll, hr, lr);
                         if (v == 0) r.x = r.y;         // Dirichlet: the end node takes the interior centre
                     }
                     *reinterpret_cast<V *>(R + St::pos(VN * v)) = r;
@@ -542,22 +532,6 @@ __device__ __forceinline__ void bcol_r_rag(const ProgParams &pr, int64_t lbase, 
         const float v = sdiff_pair(hm, h0, hp, lm, l0, lp);
         if (k == 0) rl = v; else if (k == RPT + 1) rr = v; else r[k - 1] = v;
         hm = h0; h0 = hp; lm = l0; l0 = lp;
-    }
-}
-
-template <int RPT>
-__device__ __forceinline__ void bcol_r_rag(const ProgParams &pr, int64_t lbase, int64_t st, int a, int n,
-                                           double (&r)[RPT], double &rl, double &rr)
-{
-    const double *U = (const double *)pr.u_hi + lbase;
-    auto row = [&](int j) { return (int64_t)(j < 0 ? 0 : (j > n - 1 ? n - 1 : j)) * st; };
-    double um = U[row(a - 2)], u0 = U[row(a - 1)];
-#pragma unroll
-    for (int k = 0; k <= RPT + 1; ++k) {
-        const double up = U[row(a + k)];
-        const double v = (up - u0) - (u0 - um);
-        if (k == 0) rl = v; else if (k == RPT + 1) rr = v; else r[k - 1] = v;
-        um = u0; u0 = up;
     }
 }
 

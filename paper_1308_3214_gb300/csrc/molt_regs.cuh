@@ -504,19 +504,6 @@ __device__ __forceinline__ void level_vec(const ProgParams &p, int64_t i, const 
     *reinterpret_cast<float4 *>((float *)p.un_hi + i) = nh;
     *reinterpret_cast<float4 *>((float *)p.un_lo + i) = nl;
 }
-__device__ __forceinline__ void level_vec(const ProgParams &p, int64_t i, const double2 &F)
-{
-    const double2 u = *reinterpret_cast<const double2 *>((const double *)p.u_hi + i);
-    double2 v;
-    v.x = p.ea * u.x + p.ec * F.x;
-    v.y = p.ea * u.y + p.ec * F.y;
-    if (p.feb != 0.f) {
-        const double2 q = *reinterpret_cast<const double2 *>((const double *)p.up_hi + i);
-        v.x += p.eb * q.x;
-        v.y += p.eb * q.y;
-    }
-    *reinterpret_cast<double2 *>((double *)p.un_hi + i) = v;
-}
 
 // level combination of CH vectors per thread (v = lane + NT (i0 + i) with NT
 // threads over the row), all loads issued before any store
@@ -558,34 +545,6 @@ template <int CH, int NT> struct LevelBatch<float, CH, NT> {
         }
     }
 };
-template <int CH, int NT> struct LevelBatch<double, CH, NT> {
-    __device__ static void run(const ProgParams &p, int64_t base, int lane, int i0, int nvec, const double2 (&F)[CH])
-    {
-        const double2 *__restrict__ U = reinterpret_cast<const double2 *>((const double *)p.u_hi + base);
-        const double2 *__restrict__ Q = reinterpret_cast<const double2 *>((const double *)p.up_hi + base);
-        double2 u[CH], q[CH];
-        const bool prev = p.eb != 0.0;
-#pragma unroll
-        for (int i = 0; i < CH; ++i) {
-            const int v = lane + NT * (i0 + i);
-            if (v < nvec) {
-                u[i] = __ldg(U + v);
-                q[i] = prev ? __ldg(Q + v) : make_double2(0.0, 0.0);
-            }
-        }
-        double2 *N = reinterpret_cast<double2 *>((double *)p.un_hi + base);
-#pragma unroll
-        for (int i = 0; i < CH; ++i) {
-            const int v = lane + NT * (i0 + i);
-            if (v < nvec) {
-                double2 r;
-                r.x = p.ea * u[i].x + p.ec * F[i].x + p.eb * q[i].x;
-                r.y = p.ea * u[i].y + p.ec * F[i].y + p.eb * q[i].y;
-                N[v] = r;
-            }
-        }
-    }
-};
 template <class T, int CH, int NT = 32, class V>
 __device__ __forceinline__ void level_batch(const ProgParams &p, int64_t base, int lane, int i0, int nvec, const V (&F)[CH])
 {
@@ -596,10 +555,6 @@ template <class V> __device__ __forceinline__ V vfma(typename std::remove_refere
 template <> __device__ __forceinline__ float4 vfma<float4>(float c, const float4 &a, const float4 &b)
 {
     return make_float4(b.x + c * a.x, b.y + c * a.y, b.z + c * a.z, b.w + c * a.w);
-}
-template <> __device__ __forceinline__ double2 vfma<double2>(double c, const double2 &a, const double2 &b)
-{
-    return make_double2(b.x + c * a.x, b.y + c * a.y);
 }
 
 // Coalesced side of the staging buffer: a lane covers vectors of VN
@@ -1947,24 +1902,6 @@ __device__ __forceinline__ void strided_r_pair(const ProgParams &pr, int64_t lba
         const float v = sdiff_pair(hm, h0, hp, lm, l0, lp);     // centre a + k - 1
         if (k == 0) rl = v; else if (k == RPT + 1) rr = v; else r[k - 1] = v;
         hm = h0; h0 = hp; lm = l0; l0 = lp;
-    }
-}
-
-template <int BC, int RPT>
-__device__ __forceinline__ void strided_r_pair(const ProgParams &pr, int64_t lbase, int64_t st, int a, int n,
-                                               double (&r)[RPT], double &rl, double &rr)
-{
-    const double *U = (const double *)pr.u_hi + lbase;
-    double um = U[wrap_or_clamp<BC>(a - 2, n) * st], u0 = U[wrap_or_clamp<BC>(a - 1, n) * st];
-    const double *pu = U + (int64_t)a * st;
-#pragma unroll
-    for (int k = 0; k <= RPT + 1; ++k) {
-        double up;
-        if (k < RPT) { up = *pu; pu += st; }
-        else up = U[wrap_or_clamp<BC>(a + k, n) * st];
-        const double v = (up - u0) - (u0 - um);
-        if (k == 0) rl = v; else if (k == RPT + 1) rr = v; else r[k - 1] = v;
-        um = u0; u0 = up;
     }
 }
 
