@@ -19,6 +19,9 @@
 //    the segments through shared and distributed shared memory, or one
 //    neighbour exchange per sweep where that is exact (batch_cols_nb).
 //
+// These are the float32 passes; a float64 batch runs the line passes of
+// molt_f64.cuh (k_f64_batch) on the same internal layout.
+//
 // Line lengths are arbitrary: the segment routines' RAG variants handle the
 // last point anywhere in a segment.  Fields live in an internal layout whose
 // rows are padded to a multiple of 4 points (16-byte aligned vectors); the
