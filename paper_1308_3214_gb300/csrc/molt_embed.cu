@@ -895,7 +895,7 @@ mol_status obj_items(mol_embed_ctx *e, int a, const std::vector<int> &m)
     for (int l = 0; l < n; ++l) gmax = std::max(gmax, segs(l));
     const int T = X.threads = gmax <= 128 ? 128 : gmax <= 256 ? 256 : 512;
     const double nu = e->alpha * (a == 0 ? e->hx : e->hy);
-    X.win = std::max(1, (int)std::ceil(60.0 * std::log(2.0) / (nu * (double)R)));
+    X.win = f64_window(nu, R, gmax);
     struct Group { int line, count, len; };              // len: segments of its longest line
     std::vector<Group> gr;
     for (int l = 0; l < n;) {

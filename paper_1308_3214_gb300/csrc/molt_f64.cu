@@ -10,9 +10,6 @@ namespace molt {
 
 namespace {
 
-// segments whose inflow matters: d^(R win) <= 2^-60
-int f64_window(double nu, int R) { return std::max(1, (int)std::ceil(60.0 * std::log(2.0) / (nu * (double)R))); }
-
 // The window's sums over win of G segments: steps one by one cost an operation
 // each (64 cycles with few warps about), doubling one operation, a barrier and
 // a trip through shared memory; blocks = steps left after dbl doublings.
@@ -39,7 +36,7 @@ F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
     c.n = A.n;
     c.G = (A.n + R - 1) / R;
     c.len_last = A.n - (c.G - 1) * R;
-    c.win = f64_window(nu, R) + (c.len_last < R ? 1 : 0);    // a short last segment spans less than d^R
+    c.win = f64_window(nu, R, c.G) + (c.len_last < R ? 1 : 0);    // a short last segment spans less than d^R
     c.R = R;
     f64_window_sums(c.win, c.G, &c.dbl, &c.blocks);
     for (int k = 0; k < 8; ++k) c.pd[k] = std::exp(-nu * (double)R * (double)(1 << k));
@@ -124,6 +121,12 @@ double f64_kappa(double nu, int quad)
     return -half_K(nu) - 0.5 * R2 * -std::expm1(-2.0 * nu);
 }
 
+int f64_window(double nu, int points, int count)
+{
+    const double w = std::ceil(60.0 * std::log(2.0) / (nu * (double)points));
+    return (int)std::max(1.0, std::min(w, (double)count));     // (w itself may exceed an int)
+}
+
 // (1 - d^2) / d and 1 / d carry the boundary terms past a segment's first and
 // last point; where d is so small that the next point sees nothing of them,
 // they drop out (the end points themselves are set)
@@ -160,7 +163,7 @@ bool f64_plan(int n, int64_t nlines, bool contig, bool horner, double nu, int sm
     for (int R = 4; R <= rmax; R *= 2) {
         const int G = (n + R - 1) / R;
         int dbl = 0, blocks = 0;
-        f64_window_sums(f64_window(nu, R), G, &dbl, &blocks);
+        f64_window_sums(f64_window(nu, R, G), G, &dbl, &blocks);
         const double ops = (horner ? 12.0 : 8.0) * R + 2.0 * blocks + 3.5 * dbl + 18.0;
         // strided accesses in runs of 4 columns or more, except where a column fills the CTA
         const int c_min = contig ? 1 : (4 * G <= kF64Threads ? 4 : 2);

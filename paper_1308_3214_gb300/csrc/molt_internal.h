@@ -146,6 +146,9 @@ struct F64Plan {
 };
 struct F64Prog;
 double f64_kappa(double nu, int quad);
+// of count pieces of a line, points each, how many from one on matter to it:
+// d^(points win) <= 2^-60, at most all of them
+int f64_window(double nu, int points, int count);
 // w_k = d^(k+1) (1 - d^(2 (len-k))) / (1 - d^2), k < len (molt_f64.cuh)
 void f64_inflow_weights(double nu, int len, double *w);
 void f64_inverse_decay(double d, double om2, double &e1, double &id);

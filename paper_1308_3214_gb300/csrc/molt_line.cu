@@ -12,10 +12,9 @@ struct F64LinePlan {
     int R, K, threads, nw;     // points per thread, CTAs (one cluster), threads per CTA, warps on the line
 };
 
-int f64_line_window(double nu, int R, int n)
+int f64_line_window(double nu, int R, int n, int nw)
 {
-    const int pts = 32 * R;
-    return std::max(1, (int)std::ceil(60.0 * std::log(2.0) / (nu * (double)pts))) + (n % pts ? 1 : 0);
+    return f64_window(nu, 32 * R, nw) + (n % (32 * R) ? 1 : 0);
 }
 
 // The split with the shortest sweep, in cycles: 7 operations a point and about
@@ -33,7 +32,7 @@ F64LinePlan f64_line_plan(int n, double nu)
         for (int K = 1; K <= 8; K *= 2) {
             const int wc = (nw + K - 1) / K;
             if (wc > 8 || (K > 1 && nw < K)) continue;
-            const double ops = 7.0 * R + 24.0 + 4.0 * std::min(f64_line_window(nu, R, n), nw);
+            const double ops = 7.0 * R + 24.0 + 4.0 * std::min(f64_line_window(nu, R, n, nw), nw);
             const double c = ops * ((wc + 3) / 4) * (wc >= 4 ? 76.0 : 64.0) + (K > 1 ? 1340.0 : 60.0);
             if (best.R == 0 || c < cost) {
                 cost = c;
@@ -115,7 +114,7 @@ cudaError_t launch_line_f64(int bc, double nu, int quad, const AxisDev &ax, cons
     A.gl = (n - 1) / R;
     A.len_last = n - A.gl * R;
     A.nw = pl.nw;
-    A.jw = f64_line_window(nu, R, n);
+    A.jw = f64_line_window(nu, R, n, pl.nw);
     A.d = ax.d;
     const double om2 = -std::expm1(-2.0 * nu), kap = f64_kappa(nu, quad);
     A.rho = quad >= 2 ? -0.5 * quad_R(nu) / kap : 0.0;

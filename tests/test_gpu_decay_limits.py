@@ -1,0 +1,99 @@
+"""The float64 passes at both ends of the decay per cell, nu = alpha h.
+
+Very slow decay (a domain far shorter than 1 / alpha): every segment sees every
+other one.  On a field that vanishes at both ends L^{-1} v is below (nu + (n nu)^2)
+|v| (the quadratic rule's own term and the domain's length), so D v is v
+itself.  Tolerance: that, plus 2 n eps64 / nu for the solve, which sums n values
+rounded once (second differences, at most 4 |v|) with the response 1 / (2 nu) of
+the open line and takes the two end terms out again.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_1308_3214_gb300 import workloads
+from test_gpu_parity import dev, field, make, rel_l2, spacing
+
+pytestmark = pytest.mark.gpu
+
+EPS64 = 2.0 ** -52
+
+
+def slow_tol(n, nu):
+    return 2 * n * EPS64 / nu + nu + (n * nu) ** 2
+
+
+# nu times 4 points a segment below 60 ln 2 / 2^31: the number of segments whose
+# inflow matters exceeds an int.  Lines whose last segment is full and short.
+SLOW = [1e-9, 4e-9, 3e-11]
+
+
+@pytest.mark.parametrize("n", [5, 64, 301, 1000])
+@pytest.mark.parametrize("nu", SLOW)
+@pytest.mark.parametrize("quad", [1, 2])
+def test_powers_of_slow_decay(n, nu, quad):
+    for shape, axis in (((n, 3), 1), ((3, n), 0)):
+        s = make(shape, oracle.beta_max(2) * spacing(n, "dirichlet") / nu, 2, "dirichlet", "fp64", quad)
+        assert abs(s.nu[axis] / nu - 1) < 1e-12
+        v = np.zeros(shape)
+        line = field((n,), 400 + n, "dirichlet")
+        line[0] = line[-1] = 0.0
+        v[:] = line[:, None] if axis == 1 else line[None, :]
+        got = s.apply_D(dev(v), axis, 1).cpu().numpy()
+        assert rel_l2(got, v) <= slow_tol(n, nu), (shape, rel_l2(got, v))
+        s.close()
+
+
+@pytest.mark.parametrize("n", [5, 64, 301, 1000, 3001])
+@pytest.mark.parametrize("nu", SLOW)
+def test_line_loop_of_slow_decay(n, nu):
+    """One step of the 1D loop against the level update with F[u] = f_1 D u = -beta^2 u
+    (P = 1)."""
+    beta = oracle.beta_max(1)
+    s = make((n,), beta * spacing(n, "dirichlet") / nu, 1, "dirichlet", "fp64")
+    u0, u1 = (field((n,), 410 + k, "dirichlet") for k in (0, 1))
+    u0[0] = u0[-1] = u1[0] = u1[-1] = 0.0
+    up, uc = dev(u0), dev(u1)
+    s.step(up, uc, 1)
+    ref = 2 * u1 - u0 - beta ** 2 * u1
+    assert np.array_equal(up.cpu().numpy(), u1)
+    assert rel_l2(uc.cpu().numpy(), ref) <= beta ** 2 * slow_tol(n, nu) * np.linalg.norm(u1) / np.linalg.norm(ref)
+    s.close()
+
+
+@pytest.mark.parametrize("nu", SLOW)
+def test_batch_of_slow_decay(nu):
+    """Two ragged problems, P = 1: F u = -beta^2 (D_x + D_y - 2 D_x D_y) u, nothing but
+    the errors of four applications where D is the identity."""
+    from paper_1308_3214_gb300 import molt
+    beta = oracle.beta_max(1)
+    ns = (61, 130)
+    b = molt.BatchSolver([(n, n) for n in ns], dt=[beta * spacing(n, "dirichlet") / nu for n in ns], P=1, prec="fp64")
+    us = [field((n, n), 420 + n, "dirichlet") for n in ns]
+    got = b.apply_F(dev(np.concatenate([u.ravel() for u in us]))).cpu().numpy()
+    o = 0
+    for n, u in zip(ns, us):
+        F = got[o:o + n * n]
+        o += n * n
+        assert np.linalg.norm(F) <= 4 * beta ** 2 * slow_tol(n, nu) * np.linalg.norm(u), n
+    b.close()
+
+
+@pytest.mark.parametrize("n", [24, 260])
+@pytest.mark.parametrize("nu", SLOW)
+@pytest.mark.parametrize("axis", [0, 1])
+def test_embedded_lines_of_slow_decay(n, nu, axis):
+    """L^{-1} v = v - D v vanishes on a disk far smaller than 1 / alpha (the rounding of an
+    end cell's second difference grows with the spacing over the shortest gap)."""
+    from paper_1308_3214_gb300 import molt
+    g = workloads.disk_grid(n)
+    live = g.mask.any(axis=1 - axis)
+    gaps = (g.ra[live], g.rb[live]) if axis == 0 else (g.ca[live], g.cb[live])
+    gmin = min(x.min() for x in gaps)
+    s = molt.EmbedSolver(g, dt=oracle.beta_max(1) * g.hx / nu, P=1)
+    v = workloads.random_field((n, n), 430 + n) * g.mask
+    w = s.linv(dev(v), axis).cpu().numpy()
+    assert np.linalg.norm(w) <= slow_tol(n, nu) * (g.hx / gmin) * np.linalg.norm(v)
+    s.close()
