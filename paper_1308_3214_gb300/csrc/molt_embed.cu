@@ -248,6 +248,16 @@ __global__ void __launch_bounds__(512) k_obj_sweep(const __grid_constant__ ObjAx
                 gin = fma(ca, ax.pw[len], gin);
             }
             if (nr) gin = fma(fma(-B * ln.mu, ln.dA, y1) * db, ax.id, gin);
+            // a decay too small to divide by (f64_inverse_decay) carries nothing
+            // past the end nodes m and 1, but these stand a gap away from the boundary
+            // points, whatever its length, and have their terms
+            if (ax.id == 0.0) {
+                if (seg == 0) z[0] = fma(B, ln.dB, z[0]);
+                if (last) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) z[j] = j == len - 1 ? z[j] + fma(-B * ln.mu, ln.dA, y1) : z[j];
+                }
+            }
         }
     }
     // e, then the result

@@ -129,7 +129,8 @@ int f64_window(double nu, int points, int count)
 
 // (1 - d^2) / d and 1 / d carry the boundary terms past a segment's first and
 // last point; where d is so small that the next point sees nothing of them,
-// they drop out (the end points themselves are set)
+// they drop out (the end points themselves are set; the end nodes of a line
+// object, which are interior, take theirs one by one, k_obj_sweep)
 void f64_inverse_decay(double d, double om2, double &e1, double &id)
 {
     id = d > 1e-140 ? 1.0 / d : 0.0;

@@ -97,3 +97,58 @@ def test_embedded_lines_of_slow_decay(n, nu, axis):
     w = s.linv(dev(v), axis).cpu().numpy()
     assert np.linalg.norm(w) <= slow_tol(n, nu) * (g.hx / gmin) * np.linalg.norm(v)
     s.close()
+
+
+# ---------------------------------------------------------------------------
+# Very fast decay: below d = 1e-140 (nu = 322.4) nothing divides by d any more.
+# The end nodes of an embedded line stand gaps of any length away from the
+# boundary points, so the terms of the two ends still reach them.
+# Tolerances: as in test_gpu_embedded, 100 eps64 over the shortest gap in cells;
+# mixed: 16 roundings of the decay sum, 2 eps32 each, of the field.
+# ---------------------------------------------------------------------------
+FAST = [80.0, 321.0, 323.0, 400.0, 1000.0]
+
+
+def notched_grid(gaps):
+    """A rectangle of 9 x 7 interior nodes with a column of two more above it (rows of
+    one node) and a row of three more beside it; the gaps are dealt out in turn,
+    in spacings."""
+    ny, nx, h = 12, 15, 0.1
+    mask = np.zeros((ny, nx), bool)
+    mask[1:8, 2:11] = True
+    mask[8:10, 5] = True
+    mask[3, 11:14] = True
+    k = [0]
+
+    def line(m):
+        n = len(m)
+        lo, hi = np.ones(n, np.int64), np.zeros(n, np.int64)
+        ga, gb = np.zeros(n), np.zeros(n)
+        for i in range(n):
+            j = np.flatnonzero(m[i])
+            if len(j) == 0:
+                continue
+            lo[i], hi[i] = j[0], j[-1]
+            ga[i], gb[i] = (h * gaps[(k[0] + q) % len(gaps)] for q in (0, 1))
+            k[0] += 1
+        return lo, hi, ga, gb
+    r0, r1, ra, rb = line(mask)
+    c0, c1, ca, cb = line(mask.T)
+    return workloads.EmbeddedGrid(nx, ny, 0.0, 0.0, h, h, r0, r1, ra, rb, c0, c1, ca, cb, mask)
+
+
+@pytest.mark.parametrize("nu", FAST)
+@pytest.mark.parametrize("gaps", [(1e-6, 0.7), (1e-3, 1e-6, 1.0), (1e-6,)])
+def test_embedded_lines_of_fast_decay(nu, gaps):
+    from paper_1308_3214_gb300 import molt
+    g = notched_grid(gaps)
+    P, beta, alpha = 2, oracle.beta_max(2), nu / g.hx
+    s = molt.EmbedSolver(g, dt=beta / alpha, P=P)
+    v = workloads.random_field((g.ny, g.nx), 440) * g.mask
+    tol = 100 * EPS64 / min(gaps)
+    for axis in (0, 1):
+        got = s.linv(dev(v), axis).cpu().numpy()
+        ref = oracle.linv_axis_embed(v, axis, g, alpha)
+        assert rel_l2(got, ref) <= tol, (axis, rel_l2(got, ref))
+    assert rel_l2(s.apply_F(dev(v)).cpu().numpy(), oracle.F_embed(v, g, alpha, P, beta)) <= tol
+    s.close()
