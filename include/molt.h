@@ -163,7 +163,8 @@ mol_status mol_solve_host(mol_handle h, const double *u0, double *u_out, int64_t
  * each row split over 2, 4 or 8 warps (rows of 32 W RPT points), one CTA per
  * row or persistent CTAs that prefetch their next row (MOL_TUNE_ROWS_PERSIST),
  * the strided segment length (64 or 32 points per thread for float32 sweeps)
- * and the segments per CTA at most (8 or 4, hence the cluster size) -- on the
+ * and the segments per CTA at most (8, 4 or the handle's default, hence the
+ * cluster size) -- on the
  * handle's own workspace (a few steps each, CUDA events, minimum of 3
  * timings) and keeps the fastest for every later call.  Synchronous on the
  * stream; the caller's fields are not touched.  The paper has no counterpart.
@@ -174,7 +175,9 @@ mol_status mol_autotune(mol_handle h, void *stream);
  * res_warps 1, 2 or 4; strided_rpt 0 (default) or 32; strided_warps 1..8;
  * rows_warps 0 (one warp per row) or 2, 4, 8 (each row split over that many
  * warps, where the row length allows it).  MOL_EINVAL if a choice is out of
- * range or does not fit an axis. */
+ * range or does not fit an axis.  A handle starts with strided_warps 8, or 4 or 2
+ * where its columns run over clusters whatever the choice and the grid is too
+ * narrow to give every SM a CTA; a choice made here is used as it is. */
 mol_status mol_set_tuning(mol_handle h, int res_warps, int strided_rpt, int strided_warps, int rows_warps);
 
 /* The launch choices in use: out[0] = warps per CTA of the resident x pass,

@@ -284,19 +284,6 @@ void smem_pass_geom(const mol_ctx *h, int axis, bool horner, PassGeom &G, AxisDe
     G.dps = pass_smem_bytes(horner, h->tbytes, G.W, A.ls, A.n, 1) <= h->smem_optin ? 1 : 0;
 }
 
-// Segments per CTA of the neighbour-exchange passes (their result does not
-// depend on it): fewer where the column groups would leave SMs without a CTA.
-void spread_segments(const mol_ctx *h, int64_t nlines, int n, int *rpt, int *S, int *K)
-{
-    for (int mw = *S / 2; mw >= 2 && (nlines + 31) / 32 * *K < h->num_sms; mw /= 2) {
-        int r = 0, s2 = 0, k2 = 0;
-        if (!regs_strided_plan(h->tbytes, h->bc, n, &r, &s2, &k2, h->tune_strided_rpt, mw)) return;
-        *rpt = r;
-        *S = s2;
-        *K = k2;
-    }
-}
-
 // A float64 pass: the Horner weights arrive in the units of the powers (times
 // kappa per application of this axis' D, f64_units); raw powers stay in them.
 cudaError_t run_f64(const mol_ctx *h, int axis, const PowersParams *pp, const HornerParams *hp, cudaStream_t s)
@@ -400,7 +387,6 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
             if (!regs_strided_plan(h->tbytes, h->bc, n, &rpt, &S, &K, h->tune_strided_rpt, h->tune_strided_warps))
                 return fail(h, MOL_EINVAL, "no register plan for the transposed y pass");
             LineSet L = lineset_of(h, axis);
-            if (h->tune_strided_nb && regs_strided_nb_plan(h->ax[axis].d, n, rpt)) spread_segments(h, L.nlines, n, &rpt, &S, &K);
             L.S = S;
             L.K = K;
             const AxisDev A = regs_axis(h, axis, rpt);
@@ -422,7 +408,6 @@ mol_status run_program(mol_ctx *h, int axis, const ProgParams &pr, const PowersP
     } else if (axis > 0 && regs_strided_plan(h->tbytes, h->bc, n, &rpt, &S, &K, h->tune_strided_rpt,
                                              h->tune_strided_warps)) {
         LineSet L = lineset_of(h, axis);
-        if (h->tune_strided_nb && regs_strided_nb_plan(h->ax[axis].d, n, rpt)) spread_segments(h, L.nlines, n, &rpt, &S, &K);
         L.S = S;
         L.K = K;
         const AxisDev A = regs_axis(h, axis, rpt);
@@ -865,6 +850,34 @@ void default_rows_split(mol_ctx *h)
     if (h->ndim >= 2 && regs_rows_plan(h->tbytes, (int)h->n[0], h->xtpl.ng, 2, &r)) h->tune_rows_warps = 2;
 }
 
+// Segments per CTA of the strided passes: as many as a CTA takes (8), or fewer
+// where the columns run over clusters anyway and the narrow grid would leave SMs
+// without a CTA.  Only for passes that exchange between neighbouring segments,
+// whose bits do not depend on it, and only where no other axis changes with it.
+// us per step, 8 segments at most against this rule: 1024^2, P = 2, 17.9 against 16.9;
+// 2048 x 96 13.2, 11.7; 1536^2, P = 3, 48.3, 46.4; 640^2, P = 3, 17.6, 16.4 (at worst 1536
+// rows of 1024, P = 2: 22.8, 23.2).  A column that fits one CTA is better left there
+// (no cluster barriers): 256^2, P = 2, 9.7 against 10.9 over two CTAs, 32 x 256 x 64
+// 58.3, 61.8.
+void default_strided_split(mol_ctx *h)
+{
+    for (int mw = 4; mw >= 2 && h->tbytes == 4; mw /= 2) {
+        bool wants = false, ok = true;
+        for (int a = 1; a < h->ndim; ++a) {
+            const int n = (int)h->n[a];
+            int r = 0, S = 0, K = 0, r2 = 0, S2 = 0, K2 = 0;
+            if (!regs_strided_plan(4, h->bc, n, &r, &S, &K, h->tune_strided_rpt, h->tune_strided_warps)) continue;
+            if (regs_strided_plan(4, h->bc, n, &r2, &S2, &K2, h->tune_strided_rpt, mw) && S2 == S) continue;
+            const int64_t groups = (h->N / n + 31) / 32;
+            const bool spread = S2 > 0 && K > 1 && groups * K < h->num_sms && regs_strided_nb_plan(h->ax[a].d, n, r);
+            wants |= spread;
+            ok &= spread;
+        }
+        if (!wants || !ok) return;
+        h->tune_strided_warps = mw;
+    }
+}
+
 }  // namespace
 
 void molt::set_global_error(const std::string &msg) { g_err = msg; }
@@ -994,6 +1007,7 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
             if ((st = dev_alloc(h, &h->inter[k], (size_t)h->tbytes * h->N)) != MOL_OK) goto bad;
     }
     default_rows_split(h);
+    default_strided_split(h);
     if (prec == MOL_MIXED && h->ndim == 2 && bc == MOL_BC_DIRICHLET && h->n[0] <= 1024 && h->n[1] <= 1024) {
         int r = 0, S = 0, K = 0;
         const bool xreg = regs_res_plan(h->tbytes, (int)h->n[0], h->xtpl.ng, &r) ||
@@ -1223,6 +1237,7 @@ mol_status mol_autotune(mol_handle h, void *stream)
         {h->tune_strided_rpt + 100 * h->tune_strided_nb + 1000 * h->tune_strided_stage, h->tune_strided_warps}};
     if (strided) {
         std::vector<std::pair<int, int>> base = {{0, 8}, {0, 4}};
+        if (h->tune_strided_warps != 8 && h->tune_strided_warps != 4) base.push_back({0, h->tune_strided_warps});
         if (h->tbytes == 4) { base.push_back({32, 8}); base.push_back({32, 4}); }
         str_c.clear();
         for (auto &b : base) {
