@@ -54,6 +54,7 @@ struct ObjAxis {
     const int4 *items;  // [ctas][threads]: line (-1: none), segment, slot of the line's segment 0,
                         // slots to the next segment
     int win;            // segments whose inflow matters
+    int direct;         // d too small to divide by: e1 = id = 0
     double d, e1, id;   // e^{-alpha h}, (1 - d^2)/d, 1/d
     double gc, ge;      // uniform rows
     const double *dpow; // d^k, k = 0..kObjMaxM
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(512) k_obj_sweep(const __grid_constant__ ObjAx
             // a decay too small to divide by (f64_inverse_decay) carries nothing
             // past the end nodes m and 1, but these stand a gap away from the boundary
             // points, whatever its length, and have their terms
-            if (ax.id == 0.0) {
+            if (ax.direct) {
                 if (seg == 0) z[0] = fma(B, ln.dB, z[0]);
                 if (last) {
 #pragma unroll
@@ -1234,6 +1235,7 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
             X.gc = sc * (2.0 * H - h / alpha);
             X.ge = -sc * X.d * H;
             f64_inverse_decay(X.d, c, X.e1, X.id);
+            X.direct = X.id == 0.0;
             for (int k = 0; k <= kObjR; ++k) X.pw[k] = std::exp(-alpha * h * (double)k);
             for (int k = 1; k <= kObjR; ++k) f64_inflow_weights(alpha * h, k, X.w[k]);
         }
