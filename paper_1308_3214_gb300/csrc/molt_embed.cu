@@ -316,7 +316,7 @@ struct ObjLineF {
     long long base;     // element index of the first interior node
     int m, pad_;
     float dA, dB;       // decays of the end cells
-    float rA, rB;       // dA / d, dB / d
+    float rA, rB;       // dA / d, dB / d (d as in the table d^k, obj_decay_floor32)
     float cA, cB;       // 1 - dA^2, 1 - dB^2
     float mu, inv;      // e^{-alpha (b - a)}, 1 / (1 - mu^2)
     float g11, g12;     // row 1: q_1 = g11 s_1 + g12 s_2
@@ -718,6 +718,11 @@ std::vector<double> obj_positions(int m, double h, double ga, double gb)
     return x;
 }
 
+// The table's d^1 is at least this (alpha h up to 83), so that dA / d times it stays
+// dA in float32, whose range both leave at alpha h of 88 and 104 (0 times infinity).
+// What crosses a whole cell is then 2^-120 of what enters instead of less.
+constexpr double obj_decay_floor32 = 7.52316384526264e-37;       // 2^-120
+
 // the float32 constants of a line object.  The rows 1 and N-1 of the
 // difference form are computed in float64 from the increments and written
 // as weights on the second divided differences (scaled by h^2): a row
@@ -733,8 +738,9 @@ ObjLineF make_line32(long long base, int m, double h, double ga, double gb, doub
     const double b = x[N];
     L.dA = (float)std::exp(-alpha * ga);
     L.dB = (float)std::exp(-alpha * gb);
-    L.rA = (float)std::exp(-alpha * (ga - h));
-    L.rB = (float)std::exp(-alpha * (gb - h));
+    const bool fast = std::exp(-alpha * h) < obj_decay_floor32;
+    L.rA = (float)(fast ? std::exp(-alpha * ga) / obj_decay_floor32 : std::exp(-alpha * (ga - h)));
+    L.rB = (float)(fast ? std::exp(-alpha * gb) / obj_decay_floor32 : std::exp(-alpha * (gb - h)));
     L.cA = (float)(-std::expm1(-2.0 * alpha * ga));
     L.cB = (float)(-std::expm1(-2.0 * alpha * gb));
     L.mu = (float)std::exp(-alpha * b);
@@ -1274,6 +1280,7 @@ mol_status mol_embed_create(const mol_embed_geom *g, double c, double dt, double
             Y.c = (float)(-std::expm1(-2.0 * alpha * h));
             uniform_rows32(h, alpha, Y.gc, Y.ge);
             std::vector<float> tab32(tab.begin(), tab.end());
+            tab32[1] = std::max(tab32[1], (float)obj_decay_floor32);
             std::vector<ObjLineF> ls32;
             for (int64_t l = 0; l < nl; ++l) {
                 if (lo[l] > hi[l]) continue;

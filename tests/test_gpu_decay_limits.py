@@ -152,3 +152,24 @@ def test_embedded_lines_of_fast_decay(nu, gaps):
         assert rel_l2(got, ref) <= tol, (axis, rel_l2(got, ref))
     assert rel_l2(s.apply_F(dev(v)).cpu().numpy(), oracle.F_embed(v, g, alpha, P, beta)) <= tol
     s.close()
+
+
+# float32 sweeps: e^{alpha h} exceeds a float at nu = 88.7, d is zero at 104
+@pytest.mark.parametrize("nu", [79.0, 81.0, 88.5, 89.0, 95.0, 110.0, 323.0, 1000.0])
+@pytest.mark.parametrize("gaps", [(0.5, 0.9), (1e-3, 0.7), (1e-3, 1e-2, 1.0), (2.5, 1e-3)])
+def test_mixed_embedded_lines_of_fast_decay(nu, gaps):
+    """Bounds of test_gpu_embedded: 16 eps32 (1 + 1 / (1 - d)), of the field for L^{-1} v, times
+    2P of F."""
+    from paper_1308_3214_gb300 import molt
+    g = notched_grid(gaps)
+    P, beta, alpha = 2, oracle.beta_max(2), nu / g.hx
+    s = molt.EmbedSolver(g, dt=beta / alpha, P=P, prec="mixed")
+    v = workloads.random_field((g.ny, g.nx), 441) * g.mask
+    tol = 16 * 2 * 2.0 ** -24 + 100 * EPS64 / min(gaps)
+    for axis in (0, 1):
+        got = s.linv(dev(v), axis).cpu().numpy()
+        ref = oracle.linv_axis_embed(v, axis, g, alpha)
+        assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(v), axis
+    F = oracle.F_embed(v, g, alpha, P, beta)
+    assert rel_l2(s.apply_F(dev(v)).cpu().numpy(), F) <= 2 * P * tol
+    s.close()
