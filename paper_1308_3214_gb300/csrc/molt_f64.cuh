@@ -317,10 +317,11 @@ __device__ __forceinline__ void f64_sdiff(double (&z)[R], double zl, double zr, 
     }
 }
 
-// f(k, v) for this segment's points k < len of a field, v = q[k st].  vec: in
-// 32-byte vectors (contiguous axis; len is a multiple of 4 then).
+// f(k, v) for this segment's points k < len of a field, v = q[k st].  (Plain
+// loads: u^{n-1}, which the next level may be written over, is one of the fields.)
+// vec: in 32-byte vectors (contiguous axis; len is a multiple of 4 then).
 template <int R, bool CONTIG, class F>
-__device__ __forceinline__ void f64_each(const double *__restrict__ q, int64_t st, int len, bool vec, F &&f)
+__device__ __forceinline__ void f64_each(const double *q, int64_t st, int len, bool vec, F &&f)
 {
     if (CONTIG && vec) {
 #pragma unroll

@@ -513,8 +513,9 @@ template <int CH, int NT> struct LevelBatch<float, CH, NT> {
     {
         const float4 *__restrict__ UH = reinterpret_cast<const float4 *>((const float *)p.u_hi + base);
         const float4 *__restrict__ UL = reinterpret_cast<const float4 *>((const float *)p.u_lo + base);
-        const float4 *__restrict__ PH = reinterpret_cast<const float4 *>((const float *)p.up_hi + base);
-        const float4 *__restrict__ PL = reinterpret_cast<const float4 *>((const float *)p.up_lo + base);
+        // (the next level may lie over up: plain loads, each before its own store)
+        const float4 *PH = reinterpret_cast<const float4 *>((const float *)p.up_hi + base);
+        const float4 *PL = reinterpret_cast<const float4 *>((const float *)p.up_lo + base);
         float4 uh[CH], ul[CH], ph[CH], pl[CH];
         const bool prev = p.feb != 0.f;
 #pragma unroll
@@ -523,8 +524,8 @@ template <int CH, int NT> struct LevelBatch<float, CH, NT> {
             if (v < nvec) {
                 uh[i] = __ldg(UH + v);
                 ul[i] = __ldg(UL + v);
-                ph[i] = prev ? __ldg(PH + v) : make_float4(0.f, 0.f, 0.f, 0.f);
-                pl[i] = prev ? __ldg(PL + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                ph[i] = prev ? PH[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+                pl[i] = prev ? PL[v] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
         const float ea = p.fea, eb = p.feb, ec = p.fec;
@@ -1539,6 +1540,7 @@ __global__ void __launch_bounds__(32 * W, W == 2 ? 8 : (W == 4 ? 7 : 4)) k_conti
     __syncthreads();
     const float4 *UH = reinterpret_cast<const float4 *>((const float *)pr.u_hi + base);
     const float4 *UL = reinterpret_cast<const float4 *>((const float *)pr.u_lo + base);
+    // (the next level may lie over up: plain loads, each before its own store)
     const float4 *PH = reinterpret_cast<const float4 *>((const float *)pr.up_hi + base);
     const float4 *PL = reinterpret_cast<const float4 *>((const float *)pr.up_lo + base);
     float4 *NH = reinterpret_cast<float4 *>((float *)pr.un_hi + base);
@@ -1554,8 +1556,8 @@ __global__ void __launch_bounds__(32 * W, W == 2 ? 8 : (W == 4 ? 7 : 4)) k_conti
             const int v = t + NT * (i0 + i);
             uh[i] = __ldg(UH + v);
             ul[i] = __ldg(UL + v);
-            ph[i] = prev ? __ldg(PH + v) : make_float4(0.f, 0.f, 0.f, 0.f);
-            pl[i] = prev ? __ldg(PL + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+            ph[i] = prev ? PH[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+            pl[i] = prev ? PL[v] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < CH; ++i) {
