@@ -961,6 +961,10 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
         st = cuda_fail(h, e, "kernel attributes");
         goto bad;
     }
+    if (h->ndim == 1 && prec == MOL_MIXED && (e = configure_line_kernels(h->smem_optin)) != cudaSuccess) {
+        st = cuda_fail(h, e, "kernel attributes");
+        goto bad;
+    }
     if (!expand_coefficients(h->ndim, P, beta, h->f)) { st = fail(h, MOL_EINVAL, "coefficient expansion failed"); goto bad; }
 
     for (int a = 0; a < h->ndim; ++a) {

@@ -1032,8 +1032,7 @@ mol_status run_update(mol_embed_ctx *e, const double *u, const double *up, doubl
             if (!end) std::swap(e->V[k], e->tmp);
         }
         if (last) continue;
-        // not the last stage: its own sum (V[1], its C u now in tmp, when p = 2)
-        if (p == 2) t.x[1] = e->tmp;
+        // not the last stage: its own sum
         add(t.cw, e->V[p - 1]);
         EST(combine(e, t, s));
     }

@@ -30,7 +30,7 @@ void f64_window_sums(int win, int G, int *dbl, int *blocks)
 
 double half_K(double nu) { return -std::expm1(-2.0 * nu) / (2.0 * nu); }
 
-F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
+F64Axis f64_axis(double nu, int quad, int R, const AxisDev &A)
 {
     F64Axis c{};
     c.n = A.n;
@@ -54,7 +54,6 @@ F64Axis f64_axis(double nu, int quad, int bc, int R, const AxisDev &A)
     f64_inflow_weights(nu, R, c.w);
     f64_inflow_weights(nu, c.len_last, c.wl);
     c.dpow = A.dpow64;
-    (void)bc;
     return c;
 }
 
@@ -196,7 +195,7 @@ cudaError_t launch_f64(int bc, bool contig, const F64Plan &pl, double nu, int qu
         for (int k = 0; k < MAXG; ++k) bits |= (uintptr_t)p.g[k] | (uintptr_t)p.out[k];
         p.vec = (bits & 31) == 0;
     }
-    const F64Axis A = f64_axis(nu, quad, bc, pl.R, ax);
+    const F64Axis A = f64_axis(nu, quad, pl.R, ax);
     F64Lines L{stride, inner, nlines, ax.n, pl.C, 0};
     while ((1 << L.cshift) < pl.C) ++L.cshift;
     if (bc == BC_PERIODIC)
@@ -231,7 +230,7 @@ void f64_batch_plan(const F64BatchGrid *probs, int nprob, int quad, int sms, F64
             f64_plan(A.n, std::max(lines, points / A.n), contig, contig, nu, sms, &pl, nprob > 1 ? 16 : kF64MaxR,
                      nprob > 1 ? 128 : kF64Threads);
             F64Task &t = out.tasks[(size_t)axis * nprob + i];
-            t.A = f64_axis(nu, quad, BC_DIRICHLET, pl.R, A);
+            t.A = f64_axis(nu, quad, pl.R, A);
             t.L = F64Lines{contig ? 1 : (int64_t)g.pitch, lines, lines, g.pitch, pl.C, 0};
             while ((1 << t.L.cshift) < pl.C) ++t.L.cshift;
             t.off = g.off;

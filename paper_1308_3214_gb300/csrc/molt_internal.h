@@ -166,6 +166,7 @@ struct F64LineRun;
 struct F32LineRun;
 cudaError_t launch_line_f64(int bc, double nu, int quad, const AxisDev &ax, const F64LineRun &p, cudaStream_t s);
 cudaError_t launch_line_f32(int bc, int rpt, const AxisDev &A, const F32LineRun &p, cudaStream_t s);
+cudaError_t configure_line_kernels(size_t smem_max);
 bool line_smem_ok(bool cta, const AxisDev &A, size_t smem_max);
 cudaError_t launch_line_f32_smem(int bc, bool cta, const AxisDev &A, const F32LineRun &p, size_t smem_max, cudaStream_t s);
 // 1 if a bounded wait of a register kernel gave up since the last call (and

@@ -95,9 +95,6 @@ cudaError_t run_line_smem(const AxisDev &A, const F32LineRun &p, size_t smem_max
 {
     const bool dps = line_smem_bytes(CTA, A.ls, A.n, true) <= smem_max;
     const size_t smem = line_smem_bytes(CTA, A.ls, A.n, dps);
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_line_f32_smem<BC, CTA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-    if (e != cudaSuccess) return e;
     k_line_f32_smem<BC, CTA><<<1, CTA ? kCtaLineThreads : 32, smem, s>>>(A, dps ? 1 : 0, p);
     return cudaGetLastError();
 }
@@ -137,6 +134,18 @@ cudaError_t launch_line_f64(int bc, double nu, int quad, const AxisDev &ax, cons
 cudaError_t launch_line_f32(int bc, int rpt, const AxisDev &A, const F32LineRun &p, cudaStream_t s)
 {
     return bc == BC_PERIODIC ? run_line_f32_r<BC_PERIODIC>(rpt, A, p, s) : run_line_f32_r<BC_DIRICHLET>(rpt, A, p, s);
+}
+
+cudaError_t configure_line_kernels(size_t smem_max)
+{
+    const void *kernels[] = {(const void *)k_line_f32_smem<BC_PERIODIC, false>, (const void *)k_line_f32_smem<BC_PERIODIC, true>,
+                             (const void *)k_line_f32_smem<BC_DIRICHLET, false>,
+                             (const void *)k_line_f32_smem<BC_DIRICHLET, true>};
+    for (const void *k : kernels) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 bool line_smem_ok(bool cta, const AxisDev &A, size_t smem_max)
