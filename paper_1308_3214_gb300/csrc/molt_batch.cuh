@@ -621,7 +621,8 @@ __device__ __forceinline__ void bsweep_T(const StridedCtx<T> &c, const AxisDev &
     T l2, l1, r0, r1;
     strided_halos<T, BC_DIRICHLET, RPT>(c, z, l2, l1, r0, r1, hbuf);
     const T c1 = A.cc1<T>(), c2 = A.cc2<T>();
-    if (c.seg == 0 || rag) post_T<T, RPT, true>(z, l2, l1, r0, r1, c1, c2, c.a, c.n);
+    // (the point after the segment may be n - 2, whose end row is folded in: kl = RPT + 1)
+    if (c.seg == 0 || (c.full && kl <= RPT + 1)) post_T<T, RPT, true>(z, l2, l1, r0, r1, c1, c2, c.a, c.n);
     else post_T<T, RPT, false>(z, l2, l1, r0, r1, c1, c2, c.a, c.n);
 }
 
