@@ -1012,13 +1012,18 @@ mol_status mol_create(const mol_grid *grid, double c, double dt, double beta, in
     }
     default_rows_split(h);
     default_strided_split(h);
-    if (prec == MOL_MIXED && h->ndim == 2 && bc == MOL_BC_DIRICHLET && h->n[0] <= 1024 && h->n[1] <= 1024) {
+    if (h->ndim == 2 && bc == MOL_BC_DIRICHLET && h->n[0] <= 1024 && h->n[1] <= 1024) {
         int r = 0, S = 0, K = 0;
         const bool xreg = regs_res_plan(h->tbytes, (int)h->n[0], h->xtpl.ng, &r) ||
                           regs_contig_plan(h->tbytes, h->bc, (int)h->n[0], &r);
         const bool yreg = regs_strided_plan(h->tbytes, h->bc, (int)h->n[1], &r, &S, &K);
         if (!xreg || !yreg) {
-            if ((st = mol_batch_create(1, grid, &c, &dt, &beta, &P, bc, prec, &o, &h->batch)) != MOL_OK) {
+            // (float64: of the adjoint entry points alone, but made here, so that these
+            // need no memory later and may be captured the first time; a beta that only
+            // the handle may have, MOL_EUNSTABLE, leaves them to refuse)
+            mol_batch *b = prec == MOL_MIXED ? &h->batch : &h->adj;
+            st = mol_batch_create(1, grid, &c, &dt, &beta, &P, bc, prec, &o, b);
+            if (st != MOL_OK && (prec == MOL_MIXED || st != MOL_EUNSTABLE)) {
                 h->err = mol_last_error(nullptr);
                 goto bad;
             }
