@@ -856,7 +856,7 @@ mol_status mol_batch_create(int nprob, const mol_grid *grids, const double *c, c
         for (int i = 0; i < nprob; ++i)
             for (int a = 0; a < 2; ++a) {
                 const AxisDev &A = a == 0 ? b->hp[i].ax : b->hp[i].ay;
-                const double nu = -std::log(A.d);
+                const double nu = A.d > 0.0 ? -std::log(A.d) : b->nu[2 * i + a];     // (0 times infinity is no d^0)
                 for (int64_t j = 0; j < tofs[2 * i + a + 1] - tofs[2 * i + a]; ++j) {
                     t64[tofs[2 * i + a] + j] = std::exp(-nu * (double)j);
                     t32[tofs[2 * i + a] + j] = (float)t64[tofs[2 * i + a] + j];

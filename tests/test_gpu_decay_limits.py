@@ -14,7 +14,7 @@ torch = pytest.importorskip("torch")
 
 import oracle
 from paper_1308_3214_gb300 import workloads
-from test_gpu_parity import dev, field, make, rel_l2, spacing
+from test_gpu_parity import cond_of, dev, field, make, rel_l2, spacing, tol_for
 
 pytestmark = pytest.mark.gpu
 
@@ -172,4 +172,26 @@ def test_mixed_embedded_lines_of_fast_decay(nu, gaps):
         assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(v), axis
     F = oracle.F_embed(v, g, alpha, P, beta)
     assert rel_l2(s.apply_F(dev(v)).cpu().numpy(), F) <= 2 * P * tol
+    s.close()
+
+
+@pytest.mark.parametrize("nu", [740.0, 746.0, 1200.0])
+@pytest.mark.parametrize("shape", [(77, 4), (5, 130), (33, 31)])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_batches_of_a_decay_below_the_float64_range(nu, shape, prec):
+    """d = e^{-nu} is zero from nu = 745.2 on (a few points across a long axis, or a tiny
+    step): F and F^T of batches and of ragged handles."""
+    from paper_1308_3214_gb300 import molt
+    P, beta = 2, oracle.beta_max(2)
+    dt = beta * spacing(min(shape), "dirichlet") / nu
+    s = make(shape, dt, P, "dirichlet", prec)
+    b = molt.BatchSolver([shape, shape], dt=dt, P=P, prec=prec)
+    v = field(shape, 450, "dirichlet")
+    for one, many, ref in ((s.apply_F, b.apply_F, oracle.F), (s.apply_FT, b.apply_FT, oracle.FT)):
+        want = ref(v, s.nu, P, beta, "dirichlet")
+        tol = tol_for(prec, s, 2 * P, cond_of(v, want))
+        assert rel_l2(one(dev(v)).cpu().numpy(), want) <= tol
+        got = many(dev(np.concatenate([v.ravel()] * 2))).cpu().numpy().reshape((2,) + shape)
+        assert rel_l2(got[0], want) <= tol and np.array_equal(got[0], got[1])
+    b.close()
     s.close()
