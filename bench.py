@@ -97,6 +97,16 @@ def workload_spec(name: str) -> dict:
     raise SystemExit(f"unknown workload {name}")
 
 
+def l2_note(spec: dict, prec: str) -> str:
+    """What a step touches (the two levels of the in-place time loop and the
+    staged fields) against the 129 MB of L2; no flush between steps."""
+    P, nd = spec["P"], len(spec["shape"])
+    staged = {1: 0, 2: P, 3: 2 * P + 1}[nd] * (4 if prec == "mixed" else 8)
+    mb = (16 + staged) * math.prod(spec["shape"]) / 1e6
+    return (f"no flush: per-step working set (2 levels + intermediate fields) of {mb:.3g} MB "
+            + ("exceeds the 129 MB L2" if mb > 129 else "fits in the 129 MB L2, where the time loop keeps it"))
+
+
 def bytes_per_point(spec: dict, prec: str) -> dict:
     """Algorithmic HBM bytes per point and step of each pass, the per-unit
     figures of the path's plan (one pass per axis, every field read or written
@@ -555,7 +565,7 @@ def main():
                        "bc": spec["bc"], "beta": solver.beta, "prec": args.prec,
                        "levels": "f32 hi+lo pairs" if args.prec == "mixed" else "f64",
                        "timed_region": TIMED_REGION,
-                       "l2": "no flush: per-step working set (3 levels + intermediate fields) exceeds the 129 MB L2",
+                       "l2": l2_note(spec, args.prec),
                        "parallelism": f"{world} independent replica(s)", "tuning": tuning},
             "gpu_launches": launches, "roofline": roofline, "clocks": clocks}
 
@@ -1046,17 +1056,17 @@ def main_extension(args, spec):
 
 def embedded_bytes_per_point(P: int, prec: str = "fp64") -> float:
     """Algorithmic bytes of the line-object sweeps per interior point and step.
-    float64: C = 4 sweeps (D_x, L_y^{-1}, D_y, L_x^{-1} accumulated: 16 + 16 +
-    16 + 24 B), D = 2 sweeps (L_y^{-1}, the subtraction from v: 16 + 24 B);
-    Table 3 builds 1 + P(P-1)/2 C's and P - 1 D's per step.
-    float32: C of the pair level (8 B in) 12 + 8 + 12 + 12 B; D (D_y v and
-    L_y^{-1} v in one sweep that also keeps D_y v for the C of the same field,
-    then D_x accumulated) 16 + 12 B; the C of that field, its D_y v already
-    formed, 8 + 8 + 12 B; any other C of a float32 field 8 + 8 + 8 + 12 B."""
+    Table 3 builds 1 + P(P-1)/2 C's and P - 1 D's per step: C = D_x, L_y^{-1},
+    D_y, L_x^{-1} accumulated; D (D_y v and L_y^{-1} v in one sweep that also keeps
+    D_y v for the C of the same field, then D_x accumulated); the C of that field
+    without its D_y.  (The level update's terms, read by the last sweep, are not
+    counted.)  float32: C of the pair level (8 B in) 12 + 8 + 12 + 12 B; D 16 + 12 B;
+    the C of that field 8 + 8 + 12 B; any other C of a float32 field 8 + 8 + 8 + 12 B.
+    float64: C 16 + 16 + 16 + 24 B; D 32 + 24 B; the C of that field 16 + 16 + 24 B."""
     nC = 1 + P * (P - 1) // 2
     if prec == "mixed":
         return 44.0 + (P - 1) * (28.0 + 28.0) + (nC - 1 - (P - 1)) * 36.0
-    return 88.0 * nC + 40.0 * (P - 1)
+    return 72.0 + (P - 1) * (56.0 + 56.0) + (nC - 1 - (P - 1)) * 72.0
 
 
 def main_embedded(args, spec):
@@ -1129,26 +1139,26 @@ def main_embedded(args, spec):
     hbm_achieved = bpp * npts * kt / (sweep_ms * 1e-3) / 1e9
     kinds_ms = {k: v[0] / kt for k, v in kinds.items()}
     if args.prec == "fp64":
-        # float64 operations of the sweep per interior node (a node between
-        # grid nodes): two 3-point increments (2 x 5 flops), each recurrence's
-        # chunk reduction (FMA, 2 flops) and re-scan (FMA, 2 flops) in both
-        # directions (8), the homogeneous terms and the sum (9): 27 flops.  The
-        # peak is the nominal float64 rate of a GB300 (1.25 TFLOP/s): the
-        # sweeps are bound by the narrow float64 pipe, not by HBM.
-        flops = 27.0 * npts * sweep_launches
-        achieved = flops / (sweep_ms * 1e-3) / 1e9
-        roofline = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
-                    "frac": achieved / FP64_PEAK_GFLOPS,
+        # float64 operations of the sweep per interior node: the second
+        # difference (2), q from three of them (3), the two recurrences (2), what
+        # flows in from both sides (2), v - D v or the sum (1): 10.  An operation
+        # occupies the pipe alike whether it multiplies, adds or does both, so the
+        # peak is half the nominal float64 rate of a GB300 (1.25 TFLOP/s of
+        # fused multiply-adds): the sweeps are bound by that narrow pipe.
+        ops = 10.0 * npts * sweep_launches
+        achieved = ops / (sweep_ms * 1e-3) / 1e9
+        roofline = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_GFLOPS / 2, "unit": "Gop/s",
+                    "frac": achieved / (FP64_PEAK_GFLOPS / 2),
                     "traffic": read_traffic(0, spec["name"], "fp64", "embed"),
-                    "peak_kind": "nominal float64 rate of a GB300 (no measured float64 peak on this pool)",
-                    "kernel": "k_obj_sweep (all line-object sweeps of a step; float64 recurrences)",
-                    "flops_per_node_sweep": 27, "hbm": {"achieved_GBps": hbm_achieved, "peak": hbm_peak,
-                                                         "frac": hbm_achieved / hbm_peak,
-                                                         "alg_bytes_per_point_step": bpp}}
+                    "peak_kind": "nominal float64 operations of a GB300 (measured on one: 0.53 T fma/s)",
+                    "kernel": "k_obj_sweep (all line-object sweeps of a step; float64 difference form)",
+                    "ops_per_node_sweep": 10, "hbm": {"achieved_GBps": hbm_achieved, "peak": hbm_peak,
+                                                       "frac": hbm_achieved / hbm_peak,
+                                                       "alg_bytes_per_point_step": bpp}}
     else:
         # float32 sweeps: at the HBM copy rate the algorithmic bytes take less
         # time than their float32 arithmetic at the nominal rate, so HBM is the
-        # roofline; one warp per line object leaves the sweeps latency bound
+        # roofline; shared-memory traffic and barriers keep the sweeps far from it
         roofline = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": hbm_achieved / hbm_peak,
                     "traffic": read_traffic(0, spec["name"], "mixed", "embed"),
