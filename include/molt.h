@@ -262,9 +262,10 @@ mol_status mol_adjoint(mol_handle h, int nrec, const int64_t *rec, int64_t nstep
  * (1 - d_xx/alpha^2)^{-1} with d_xx -> d_tt/c^2 at the ends (the inverse
  * Lax-Wendroff limit of Sec. 3.2), expanded to the scheme's order:
  * (-1)^p sum_{j=p..P} C(j-1, p-1) alpha^{-2j} data[k][side][j].  The end
- * nodes of every new level take the data.  Runs on the shared-memory line
- * kernels, one launch per step (no graph).  Errors: MOL_EINVAL for another
- * grid or NULL pointers. */
+ * nodes of every new level take the data.  Up to 48 steps per launch (24 in
+ * MOL_FP64), the line on chip between them; one launch per step where use_graphs
+ * is 0 or passes are timed.  Errors: MOL_EINVAL for another grid or NULL
+ * pointers. */
 mol_status mol_solve_dirichlet(mol_handle h, const double *u0, int64_t nsteps, const double *data, double *u_out,
                                void *stream);
 

@@ -103,10 +103,11 @@ __device__ __forceinline__ void affine_scan32(float &p, float &q, int lane)
 // end values (T'_1 is large where the first gap is small: lam multiplies it
 // before it is added to anything).  Bound by float64 latency on grids of a few hundred nodes per
 // line (64 cycles an operation and a warp per SM quarter), by the float64 pipe
-// above: about 11 operations a node instead of 18, spread over a line's worth
-// of threads instead of one warp.  us per step of the ellipse at P = 2, 10 sweeps
-// and a combination before, 9 sweeps now: 129^2 89 -> 76, 400^2 137 -> 96, 777^2
-// 217 -> 141, 2048^2 647 -> 562 (74 % of the float64 pipe).
+// above: 10 operations a node instead of 18 (14 to 16 issued, with the ends of
+// segments and lines), spread over a line's worth of threads instead of one warp.
+// us per step of the ellipse at P = 2, 10 sweeps and a combination before, 9 sweeps
+// now: 129^2 89 -> 78, 400^2 137 -> 97, 777^2 217 -> 142, 2048^2 647 -> 564 (73 % of the
+// float64 pipe).
 template <int R>
 __global__ void __launch_bounds__(512) k_obj_sweep(const __grid_constant__ ObjAxis ax, const ObjLine *__restrict__ lines,
                                                    const double *__restrict__ in, double *out, double *out2, double *out3,

@@ -1,4 +1,6 @@
-// molt_f64.cuh -- float64 line passes (sm_103a), any line length.
+// molt_f64.cuh -- float64 line passes (sm_103a): lines of up to 8192 points on the
+// contiguous axis and 4096 on the others, whole segments or not (longer ones
+// stay with the shared-memory kernels, molt_kernels.cuh).
 //
 // GB300 retires two float64 lane-operations per SM and clock (measured:
 // 0.53 T fma/s, against 0.85 T values/s of HBM traffic), so a float64 pass is
@@ -35,8 +37,10 @@
 // after log2 B rounds that leave in each slot the sum over a block of B
 // segments, one a block.  (Both sums from one exchange cost 5 operations a
 // segment, 64 cycles each where a quarter of an SM has a single warp: steps of
-// 72 x 65, P = 2, CFL 3.8 took 35.7 us, now 20.2; 256^2, P = 2, 34.0 -> 22.8; 512^2,
-// P = 3, 63 -> 55; 1000^2 periodic, P = 3, CFL 4, 183 -> 172.)
+// 72 x 65, P = 2, CFL 3.8 took 35.7 us, now 20.8; 256^2, P = 2, 34.0 -> 23.2; 512^2,
+// P = 3, 63 -> 55; 1000^2 periodic, P = 3, CFL 4, 183 -> 173.)  What the window
+// leaves out is below float64 rounding of the line's largest value; far ahead of a
+// point's response a value can be exactly zero.
 // Dirichlet (e = 0, or given data, at the ends; s_0 := s_1, s_{n-1} := s_{n-2}):
 // the rows at the ends drop out of s, and A' d^j + B' d^(n-1-j) with
 //   A' + mu B' = r_0 = e_0/kappa - rho s_1 - g_0,
@@ -55,10 +59,10 @@
 // run of C columns.  s waits in shared memory while its registers hold y and g.
 //
 // Measured, us per pass, against the earlier warp-per-row, clustered and
-// shared-memory kernels: 2048^2, P = 3, y 419 -> 225, x 1470 -> 355 (23 and 40
-// operations a point: 84 % of the float64 pipe's cycles); 96 x 100 x 75, P = 2,
-// x 154 -> 56, y 260 -> 133, z 72 -> 31; 256^3 periodic, P = 2, x 1150 -> 774, y
-// 3000 -> 2150, z 746 -> 496.
+// shared-memory kernels: 2048^2, P = 3, y 419 -> 225, x 1470 -> 354 (22 and 41
+// operations a point: 80 and 83 % of the float64 pipe's cycles); 96 x 100 x 75, P = 2,
+// x 154 -> 54, y 260 -> 133, z 72 -> 31; 256^3 periodic, P = 2, x 1150 -> 771, y
+// 3000 -> 2150 (87 %), z 746 -> 496.
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -535,7 +539,7 @@ __global__ void __launch_bounds__(kF64Threads, 2) k_f64(const __grid_constant__ 
 }
 
 // The same passes over the problems of a batch (Dirichlet): a CTA looks its
-// problem up in the work list and copies the problem's constants (1.8 KB) to
+// problem up in the work list and copies the problem's constants (1.5 KB) to
 // shared memory in front of the pass's own; one launch per segment length and
 // CTA size.  The constants cost shared-memory loads instead of constant operands,
 // which the float64 pipe hides.  Warps beyond the problem's lines leave.

@@ -9,7 +9,7 @@
 //     over the threads of one CTA or of a cluster, R points per thread, both
 //     levels in registers.  A float64 operation occupies a quarter of an SM
 //     for 64 cycles per warp (measured; the latency is the same 64), so short
-//     segments on many warps win until the carry scan (about 22 operations a
+//     segments on many warps win until the carry scan (about 24 operations a
 //     thread and sweep) outweighs them, and long lines take up to 8 SMs: a
 //     cluster barrier costs 0.2 us.
 //   * k_line_f32 (MOL_MIXED): the arithmetic of the one-step kernels, so that a
@@ -17,10 +17,11 @@
 //     sweep (k_contig_res) where the line splits into whole segments, else
 //     the shared-memory sweeps (k_horner), by a warp or by the whole CTA.
 //
-// Measured, us per step, one launch per step (graph) -> here: 256 points periodic,
-// P = 1, MOL_FP64, 7.3 -> 2.8; 352 points, P = 3, 25 -> 11; 10001 points with
-// boundary data, P = 3, MOL_MIXED, 35 -> 17.7 (three sweeps by 16 warps; bound by
-// their instructions); 768 points 16.7 -> 10.6 (one warp).
+// Measured, us per step, one launch per step (graph) -> here.  MOL_FP64: 256 points
+// periodic, P = 1, 7.4 -> 2.7; 352 points periodic, P = 3, 25 -> 11; 3000 points, P = 2,
+// 47 -> 9.6 (8 CTAs).  MOL_MIXED, P = 3: 768 points 6.0 -> 3.1 (whole segments on one
+// warp); 1000 points 19 -> 15 (one warp, shared memory); 10001 points, with boundary
+// data or without, 34 -> 17.4 (three sweeps by 16 warps; bound by their instructions).
 //
 // Boundary data (mol_solve_dirichlet) travel in the launch's parameters, up to
 // kLineDataSteps steps per launch.
